@@ -81,6 +81,48 @@ __device__ __forceinline__ float ex2_approx(float x) {
   return y;
 }
 
+// Two FP32 values in one 64-bit register pair and the packed operations on
+// them, each half rounded as the scalar operation rounds it. A packed FMA
+// keeps the FMA pipe busy for two cycles of a scheduler (measured: 2.2 against
+// 1.02 for a scalar one, so the rate per FMA is the same) but takes one issue
+// slot, and the pair bodies are short of issue slots, not of FMA lanes.
+typedef unsigned long long f32x2;
+
+__device__ __forceinline__ f32x2 pack2(float lo, float hi) {
+  f32x2 r;
+  asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(lo), "f"(hi));
+  return r;
+}
+__device__ __forceinline__ f32x2 dup2(float v) { return pack2(v, v); }
+__device__ __forceinline__ void unpack2(f32x2 v, float& lo, float& hi) {
+  asm("mov.b64 {%0, %1}, %2;" : "=f"(lo), "=f"(hi) : "l"(v));
+}
+__device__ __forceinline__ float sum2(f32x2 v) {
+  float lo, hi;
+  unpack2(v, lo, hi);
+  return lo + hi;
+}
+__device__ __forceinline__ f32x2 fma2(f32x2 a, f32x2 b, f32x2 c) {
+  f32x2 r;
+  asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c));
+  return r;
+}
+__device__ __forceinline__ f32x2 mul2(f32x2 a, f32x2 b) {
+  f32x2 r;
+  asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+  return r;
+}
+__device__ __forceinline__ f32x2 add2(f32x2 a, f32x2 b) {
+  f32x2 r;
+  asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+  return r;
+}
+__device__ __forceinline__ f32x2 sub2(f32x2 a, f32x2 b) {
+  f32x2 r;
+  asm("sub.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+  return r;
+}
+
 // One feature value: FP32 planes, or BF16 planes widened to FP32 (FB).
 template <bool FB>
 __device__ __forceinline__ float load_feat(const float* planes, size_t idx) {
@@ -173,6 +215,8 @@ struct BlockCtx {
   unsigned long long nnz_total, cand_total, nnz_grad, cand_grad;
   float R[9], T[3];       // FP32 centred pose: z~' = R z' + T
   float om[3], vc[3];     // unit step direction (centred frame)
+  float kw[3];            // (omega . v) omega / 6 l^2
+  float c_del, c_eps, k_eps;   // -|omega|^2 / 3, -|omega|^2 / 12, -(omega . v)^2 / 48 l^2
   float A, rc2, rplan_f, inv_l2f;
   // warp ranges: from group g0 of chunk j0 of cluster c0 up to (not
   // including) group g1 of chunk j1 of cluster c1
@@ -598,7 +642,19 @@ __device__ void gradient_direction(BlockCtx& b, const double* sums, int lane) {
     b.om[a] = x * inv;
     b.vc[a] = vc;
   }
-  if (lane == 0) b.fin = 0;
+  // the step pass's constants (step_terms): |omega|^2 and omega . v'
+  const float om = x * inv;
+  float ww = om * om, wv = om * vc;
+  ww += __shfl_sync(kFull, ww, 1) + __shfl_sync(kFull, ww, 2);   // lane 0's is used
+  wv += __shfl_sync(kFull, wv, 1) + __shfl_sync(kFull, wv, 2);
+  const float kap = __shfl_sync(kFull, wv, 0) * b.inv_l2f * (1.0f / 6.0f);
+  if (lane < 3) b.kw[a] = kap * om;
+  if (lane == 0) {
+    b.c_del = -ww * (1.0f / 3.0f);
+    b.c_eps = -ww * (1.0f / 12.0f);
+    b.k_eps = -wv * wv * b.inv_l2f * (1.0f / 48.0f);
+    b.fin = 0;
+  }
   __syncwarp();
 }
 
@@ -1154,10 +1210,13 @@ union WarpScratch {
 // Shared memory of the solve kernel.
 template <int DPS, int NU>
 struct SolveSmem {
-  float4 z[kWarps][kClusterMax];    // staged cluster, local: (-2 z_l, |z_l|^2), see stage_cluster
+  // staged cluster, local: (-2 z_l, |z_l|^2), see stage_cluster: float4 rows for a listed
+  // cluster, four planes of kClusterMax floats for the chunk path
+  float4 z[kWarps][kClusterMax];
   float4 zo[kWarps];                // origin of each warp's staged cluster (centred frame)
   float zf[kWarps][DPS][kClusterMax];
-  float4 u[kWarps][NU][kClusterMax];
+  float4 u[kWarps][NU][kClusterMax];   // step vectors of a listed cluster's points (step_terms)
+  float zw[kWarps][kClusterMax];       // step pass: -z_l . kw
   WarpScratch<DPS> ws[kWarps];      // cell-row segments of the staged cluster, or the pair list
   float red[kWarps][10];
   double red_d[kWarps][16];
@@ -1353,12 +1412,14 @@ __device__ void split_work(const SolveCfg* cfg, SolveSmem<DPS, NU>& sm, int tid,
 // octree cell of the plan's level), so |x_l| and |z_l| stay within a few
 // cutoff radii and the expansion loses no more than a few bits to
 // cancellation. Padding slots hold (0, 0, 0, +inf): beyond every cutoff,
-// zero weight. For the step pass the Taylor coefficient vectors of Eq.
-// fourth go to the warp's slots as well, their fourth components holding
-// the per-point constants that turn x_l . U_k into e . U_k (e = x' - z~').
+// zero weight. The chunk path reads four consecutive points of one component
+// at a time, so it gets the components as planes; a cluster with a pair list
+// (`listed`) is read point by point, so it gets rows, and for the step pass
+// the points' step vectors go to the warp's slots as well, their fourth
+// components holding the per-point constants that turn x_l . U_k into the term.
 template <bool STEP, int DP, int DPS, int NU>
 __device__ __forceinline__ void stage_cluster(SolveSmem<DPS, NU>& sm, int warp, int lane, bool zv,
-                                              float4 p, const float pf[DPS]) {
+                                              float4 p, const float pf[DPS], bool listed) {
   const BlockCtx& b = sm.b;
   float zt[3] = {0.f, 0.f, 0.f};
   if (zv) {
@@ -1370,65 +1431,105 @@ __device__ __forceinline__ void stage_cluster(SolveSmem<DPS, NU>& sm, int warp, 
   const float ox = __shfl_sync(kFull, zt[0], 0), oy = __shfl_sync(kFull, zt[1], 0),
               oz = __shfl_sync(kFull, zt[2], 0);
   const float lx = zv ? zt[0] - ox : 0.f, ly = zv ? zt[1] - oy : 0.f, lz = zv ? zt[2] - oz : 0.f;
-  sm.z[warp][lane] = zv ? make_float4(-2.f * lx, -2.f * ly, -2.f * lz,
+  const float4 row = zv ? make_float4(-2.f * lx, -2.f * ly, -2.f * lz,
                                       fmaf(lx, lx, fmaf(ly, ly, lz * lz)))
                         : make_float4(0.f, 0.f, 0.f, INFINITY);
+  if (listed) {
+    sm.z[warp][lane] = row;
+  } else {
+    float* pl = reinterpret_cast<float*>(sm.z[warp]);
+    pl[lane] = row.x;
+    pl[kClusterMax + lane] = row.y;
+    pl[2 * kClusterMax + lane] = row.z;
+    pl[3 * kClusterMax + lane] = row.w;
+  }
   if (lane == 0) sm.zo[warp] = make_float4(ox, oy, oz, 0.f);
 #pragma unroll
   for (int d = 0; d < DP; ++d) sm.zf[warp][d][lane] = zv ? pf[d] : 0.f;
   if (STEP) {
-    const float* om = b.om;
-    const float* vc = b.vc;
-    const float inv_l2 = b.inv_l2f;
-    float u1[3], u2[3], u3[3], u4[3];
-    u1[0] = om[1] * zt[2] - om[2] * zt[1] + vc[0];
-    u1[1] = om[2] * zt[0] - om[0] * zt[2] + vc[1];
-    u1[2] = om[0] * zt[1] - om[1] * zt[0] + vc[2];
-    u2[0] = om[1] * u1[2] - om[2] * u1[1];
-    u2[1] = om[2] * u1[0] - om[0] * u1[2];
-    u2[2] = om[0] * u1[1] - om[1] * u1[0];
-    u3[0] = om[1] * u2[2] - om[2] * u2[1];
-    u3[1] = om[2] * u2[0] - om[0] * u2[2];
-    u3[2] = om[0] * u2[1] - om[1] * u2[0];
-    u4[0] = om[1] * u3[2] - om[2] * u3[1];
-    u4[1] = om[2] * u3[0] - om[0] * u3[2];
-    u4[2] = om[0] * u3[1] - om[1] * u3[0];
-    const float u11 = u1[0] * u1[0] + u1[1] * u1[1] + u1[2] * u1[2];
-    const float u12 = u1[0] * u2[0] + u1[1] * u2[1] + u1[2] * u2[2];
-    const float u13 = u1[0] * u3[0] + u1[1] * u3[1] + u1[2] * u3[2];
-    const float u22 = u2[0] * u2[0] + u2[1] * u2[1] + u2[2] * u2[2];
-    // beta = e.U1; gamma = e.U2 - k2; delta = e.U3 - k3; eps = e.U4 - k4,
-    // with e.U = x_l.U - z_l.U: the fourth components hold -z_l.U - k
-    const float c1 = inv_l2, c2 = 0.5f * inv_l2, c3 = inv_l2 * (1.0f / 6.0f),
-                c4 = inv_l2 * (1.0f / 24.0f);
-    const float k2 = 0.5f * u11 * inv_l2, k3 = 0.5f * u12 * inv_l2,
-                k4 = (u13 * (1.0f / 6.0f) + u22 * 0.125f) * inv_l2;
-    const float4 U1 = make_float4(u1[0] * c1, u1[1] * c1, u1[2] * c1, 0.f);
-    const float4 U2 = make_float4(u2[0] * c2, u2[1] * c2, u2[2] * c2, 0.f);
-    const float4 U3 = make_float4(u3[0] * c3, u3[1] * c3, u3[2] * c3, 0.f);
-    const float4 U4 = make_float4(u4[0] * c4, u4[1] * c4, u4[2] * c4, 0.f);
-    const auto zl_dot = [&](const float4& U) { return fmaf(lx, U.x, fmaf(ly, U.y, lz * U.z)); };
-    sm.u[warp][0][lane] = make_float4(U1.x, U1.y, U1.z, -zl_dot(U1));
-    sm.u[warp][1 % NU][lane] = make_float4(U2.x, U2.y, U2.z, -zl_dot(U2) - k2);
-    sm.u[warp][2 % NU][lane] = make_float4(U3.x, U3.y, U3.z, -zl_dot(U3) - k3);
-    sm.u[warp][3 % NU][lane] = make_float4(U4.x, U4.y, U4.z, -zl_dot(U4) - k4);
+    sm.zw[warp][lane] = -fmaf(lx, b.kw[0], fmaf(ly, b.kw[1], lz * b.kw[2]));
+    if (listed) {
+      const float* om = b.om;
+      const float c1 = 0.5f * b.inv_l2f, c2 = 0.25f * b.inv_l2f;
+      const float u1[3] = {om[1] * zt[2] - om[2] * zt[1] + b.vc[0],
+                           om[2] * zt[0] - om[0] * zt[2] + b.vc[1],
+                           om[0] * zt[1] - om[1] * zt[0] + b.vc[2]};
+      const float u2[3] = {om[1] * u1[2] - om[2] * u1[1], om[2] * u1[0] - om[0] * u1[2],
+                           om[0] * u1[1] - om[1] * u1[0]};
+      const float u11 = fmaf(u1[0], u1[0], fmaf(u1[1], u1[1], u1[2] * u1[2]));
+      const float4 U1 = make_float4(u1[0] * c1, u1[1] * c1, u1[2] * c1, 0.f);
+      const float4 U2 = make_float4(u2[0] * c2, u2[1] * c2, u2[2] * c2, 0.f);
+      const auto zl_dot = [&](const float4& U) { return fmaf(lx, U.x, fmaf(ly, U.y, lz * U.z)); };
+      sm.u[warp][0][lane] = make_float4(U1.x, U1.y, U1.z, -zl_dot(U1));
+      sm.u[warp][1 % NU][lane] = make_float4(U2.x, U2.y, U2.z, -zl_dot(U2) - c2 * u11);
+    }
   }
 }
 
+// The step pass (Eq. fourth). Along P <- exp(t xi) P, xi = (omega, v) a unit
+// direction, a source point moves by u_1 = omega x z~' + v, u_2 = omega x u_1,
+// and Rodrigues' formula closes the series: u_3 = (omega . v) omega -
+// |omega|^2 u_1, u_4 = -|omega|^2 u_2, with u_1 . u_2 = 0, u_1 . u_3 = -|u_2|^2
+// and |u_2|^2 = |omega|^2 |u_1|^2 - (omega . v)^2. With e = x' - z~' the exponent's
+// coefficients are then
+//   beta  = e . u_1 / l^2
+//   gamma = (e . u_2 - |u_1|^2) / 2 l^2
+//   delta = (e . u_3 / 6 - u_1 . u_2 / 2) / l^2
+//         = (omega . v) (e . omega) / 6 l^2 - |omega|^2 beta / 6
+//   eps   = (e . u_4 / 24 - u_1 . u_3 / 6 - |u_2|^2 / 8) / l^2
+//         = -|omega|^2 gamma / 12 - (omega . v)^2 / 24 l^2
+// so a pair needs three inner products (beta, gamma, e . omega) where the printed
+// form takes four. The same holds seen from the target point: |x' - exp(t xi) z~'|
+// = |exp(-t xi) x' - z~'|, so with a_1 = omega x x' + v and a_2 = omega x a_1,
+// beta = e . a_1 / l^2 and gamma = (-e . a_2 - |a_1|^2) / 2 l^2: linear in e with
+// vectors that belong to the candidate alone. In the cluster's frame e = x_l + m / 2
+// (m = -2 z_l), each is c + m . V; V and c are formed once per chunk and stay in
+// the lane's registers, where vectors of the source point are shared loads per
+// pair. Halved terms (beta / 2, gamma / 2) keep factors of two out of the bodies;
+// the sums are scaled back, exactly, once per chunk.
+struct StepVectors {
+  f32x2 v1[3], v2[3], c1, c2, cw;
+};
+
+__device__ __forceinline__ StepVectors step_vectors(const BlockCtx& b, float x, float y, float z,
+                                                    float xl, float yl, float zl) {
+  const float w0 = b.om[0], w1 = b.om[1], w2 = b.om[2];
+  const float k1 = 0.5f * b.inv_l2f, k2 = -0.25f * b.inv_l2f;
+  const float a0 = w1 * z - w2 * y + b.vc[0], a1 = w2 * x - w0 * z + b.vc[1],
+              a2 = w0 * y - w1 * x + b.vc[2];
+  const float p0 = a0 * k1, p1 = a1 * k1, p2 = a2 * k1;
+  const float q0 = (w1 * a2 - w2 * a1) * k2, q1 = (w2 * a0 - w0 * a2) * k2,
+              q2 = (w0 * a1 - w1 * a0) * k2;
+  StepVectors s;
+  s.v1[0] = dup2(0.5f * p0);
+  s.v1[1] = dup2(0.5f * p1);
+  s.v1[2] = dup2(0.5f * p2);
+  s.v2[0] = dup2(0.5f * q0);
+  s.v2[1] = dup2(0.5f * q1);
+  s.v2[2] = dup2(0.5f * q2);
+  s.c1 = dup2(fmaf(xl, p0, fmaf(yl, p1, zl * p2)));
+  s.c2 = dup2(fmaf(k2, fmaf(a0, a0, fmaf(a1, a1, a2 * a2)), fmaf(xl, q0, fmaf(yl, q1, zl * q2))));
+  s.cw = dup2(fmaf(xl, b.kw[0], fmaf(yl, b.kw[1], zl * b.kw[2])));
+  return s;
+}
+
 // One 32-candidate chunk against the staged cluster: lane = candidate x'
-// (xp, features xf; padding points lie beyond every cutoff), inner loop over
-// the cluster's points [jlo, jhi) (multiples of 4, at most the cluster size
-// rounded up to 4; padding slots lie beyond the cutoff too). FP32 pair
+// (xp, features xf; padding points lie beyond every cutoff and carry w = 1),
+// over the cluster's points [jlo, jhi) (multiples of 4, at most the cluster
+// size rounded up to 4; padding slots lie beyond the cutoff too). FP32 pair
 // arithmetic, one ex2.approx per pair. Distances are taken relative to the
 // cluster's origin (stage_cluster): t = x_l . (-2 z_l) + |z_l|^2 equals
 // d^2 - |x_l|^2, so a pair is kept when t <= r_c^2 - |x_l|^2, and the
 // exponent A d^2 is A t + A |x_l|^2.
-// Points are taken four at a time: the four distance tests first, then, if
-// any lane of the warp keeps any of the four pairs (one vote, so the branch
-// is uniform), the four pair bodies without branches, a rejected pair
-// contributing exactly nothing (its weight is selected to zero and its step
-// terms are not added). The four bodies are independent, so their latencies
-// overlap.
+// Points are taken four at a time, as two packed pairs: the staged planes give
+// both halves of each operand with one 16-byte broadcast load per four points
+// and component. First the distance tests of every group of four, each lane
+// noting the groups in which it keeps a pair; one reduction over the warp then
+// gives the groups to evaluate, whose bodies run without votes or branches (a
+// rejected pair contributes exactly nothing: its weight is selected to zero, and
+// its beta, whose fourth power would be the first of its step terms to
+// overflow). Testing all groups first keeps the chain of loads, test, vote and
+// branch out of the bodies, which repeat the test's six packed FMAs instead.
 template <bool STEP, int DP, int MODE, int DPS, int NU>
 __device__ __forceinline__ unsigned chunk_pairs(SolveSmem<DPS, NU>& sm, int warp, float4 xp,
                                                 const float xf[DPS], int jlo, int jhi, float rc2,
@@ -1437,67 +1538,111 @@ __device__ __forceinline__ unsigned chunk_pairs(SolveSmem<DPS, NU>& sm, int warp
   const float xl = xp.x - o.x, yl = xp.y - o.y, zl = xp.z - o.z;
   const float x2 = fmaf(xl, xl, fmaf(yl, yl, zl * zl));
   const float thr = rc2 - x2;   // about -3e36 for a padding candidate: never kept
-  const float q0 = A * x2;
-  float W = 0.f, Mx = 0.f, My = 0.f, Mz = 0.f;
-  unsigned active = 0u;   // bit g: source group g kept a pair (the same in every lane)
+  const f32x2 X = dup2(xl), Y = dup2(yl), Z = dup2(zl);
+  const float* pl = reinterpret_cast<const float*>(sm.z[warp]);
+  struct Group {
+    ulonglong2 x, y, z;
+    f32x2 t[2];
+  };
+  const auto test = [&](int j0) {
+    Group g;
+    g.x = *reinterpret_cast<const ulonglong2*>(pl + j0);
+    g.y = *reinterpret_cast<const ulonglong2*>(pl + kClusterMax + j0);
+    g.z = *reinterpret_cast<const ulonglong2*>(pl + 2 * kClusterMax + j0);
+    const ulonglong2 w = *reinterpret_cast<const ulonglong2*>(pl + 3 * kClusterMax + j0);
+    g.t[0] = fma2(X, g.x.x, fma2(Y, g.y.x, fma2(Z, g.z.x, w.x)));
+    g.t[1] = fma2(X, g.x.y, fma2(Y, g.y.y, fma2(Z, g.z.y, w.y)));
+    return g;
+  };
+  unsigned mine = 0u;
+#pragma unroll 2
   for (int j0 = jlo; j0 < jhi; j0 += 4) {
-    float4 m[4];
-    float t[4];
-    bool keep[4];
+    const Group g = test(j0);
+    float t0, t1, t2, t3;
+    unpack2(g.t[0], t0, t1);
+    unpack2(g.t[1], t2, t3);
+    if (fminf(fminf(t0, t1), fminf(t2, t3)) <= thr) mine |= 1u << (j0 >> 2);
+  }
+  // bit g: source group g kept a pair (the same in every lane)
+  const unsigned active = __reduce_or_sync(kFull, mine);
+  if (active == 0u) return 0u;
+  const f32x2 q0 = dup2(A * x2), A2 = dup2(A);
+  f32x2 F[DPS];
 #pragma unroll
-    for (int jj = 0; jj < 4; ++jj) {
-      m[jj] = sm.z[warp][j0 + jj];
-      t[jj] = fmaf(xl, m[jj].x, fmaf(yl, m[jj].y, fmaf(zl, m[jj].z, m[jj].w)));
-      keep[jj] = t[jj] <= thr;
-    }
-    if (!__any_sync(kFull, keep[0] | keep[1] | keep[2] | keep[3])) continue;
-    active |= 1u << (j0 >> 2);
+  for (int d = 0; d < DP; ++d) F[d] = dup2(xf[d]);
+  StepVectors sv;
+  f32x2 c_del, c_eps, k_eps;
+  if (STEP) {
+    // a padding candidate takes the origin, so that its step terms stay finite
+    const bool pad = xp.w != 0.f;
+    sv = step_vectors(sm.b, pad ? 0.f : xp.x, pad ? 0.f : xp.y, pad ? 0.f : xp.z, pad ? 0.f : xl,
+                      pad ? 0.f : yl, pad ? 0.f : zl);
+    c_del = dup2(sm.b.c_del);
+    c_eps = dup2(sm.b.c_eps);
+    k_eps = dup2(sm.b.k_eps);
+  }
+  // gradient: W, M (3); step: the five sums, halved or quartered
+  f32x2 s[5] = {0ull, 0ull, 0ull, 0ull, 0ull};
+  for (unsigned rem = active; rem != 0u; rem &= rem - 1u) {
+    const int j0 = 4 * (__ffs(rem) - 1);
+    const Group g = test(j0);
+    f32x2 q[2] = {q0, q0};
+    f32x2 cdot[2] = {0ull, 0ull};
 #pragma unroll
-    for (int jj = 0; jj < 4; ++jj) {
-      const int j = j0 + jj;
-      float w;
+    for (int d = 0; d < DP; ++d) {
+      const ulonglong2 f = *reinterpret_cast<const ulonglong2*>(&sm.zf[warp][d][j0]);
       if (color_of(MODE) == kColorKernel) {
-        float qf = q0;
-#pragma unroll
-        for (int d = 0; d < DP; ++d) {
-          const float df = xf[d] - sm.zf[warp][d][j];
-          qf = fmaf(df, df, qf);
-        }
-        w = ex2_approx(-fmaf(A, t[jj], qf));
+        const f32x2 d0 = sub2(F[d], f.x), d1 = sub2(F[d], f.y);
+        q[0] = fma2(d0, d0, q[0]);
+        q[1] = fma2(d1, d1, q[1]);
       } else if (color_of(MODE) == kColorDot) {
-        float cdot = 0.f;
-#pragma unroll
-        for (int d = 0; d < DP; ++d) cdot = fmaf(xf[d], sm.zf[warp][d][j], cdot);
-        w = ex2_approx(-fmaf(A, t[jj], q0)) * cdot;
-      } else {
-        w = ex2_approx(-fmaf(A, t[jj], q0));
+        cdot[0] = fma2(F[d], f.x, cdot[0]);
+        cdot[1] = fma2(F[d], f.y, cdot[1]);
       }
-      w = keep[jj] ? w : 0.f;
-      nnz += keep[jj] ? 1u : 0u;
+    }
+    ulonglong2 zw;
+    if (STEP) zw = *reinterpret_cast<const ulonglong2*>(&sm.zw[warp][j0]);
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+      const f32x2 mx = h ? g.x.y : g.x.x, my = h ? g.y.y : g.y.x, mz = h ? g.z.y : g.z.x;
+      float t0, t1, e0, e1, w0, w1;
+      unpack2(g.t[h], t0, t1);
+      const bool k0 = t0 <= thr, k1 = t1 <= thr;
+      unpack2(fma2(A2, g.t[h], q[h]), e0, e1);
+      w0 = ex2_approx(-e0);
+      w1 = ex2_approx(-e1);
+      if (color_of(MODE) == kColorDot) {
+        float c0, c1;
+        unpack2(cdot[h], c0, c1);
+        w0 *= c0;
+        w1 *= c1;
+      }
+      const f32x2 w = pack2(k0 ? w0 : 0.f, k1 ? w1 : 0.f);
+      nnz += (k0 ? 1u : 0u) + (k1 ? 1u : 0u);
+      s[0] = add2(s[0], w);
       if (!STEP) {
         // m = (-2 z_l, .) is finite, so a zero weight adds exactly zero
-        W += w;
-        Mx = fmaf(w, m[jj].x, Mx);
-        My = fmaf(w, m[jj].y, My);
-        Mz = fmaf(w, m[jj].z, Mz);
+        s[1] = fma2(w, mx, s[1]);
+        s[2] = fma2(w, my, s[2]);
+        s[3] = fma2(w, mz, s[3]);
       } else {
-        const float4 U1 = sm.u[warp][0][j], U2 = sm.u[warp][1 % NU][j];
-        const float4 U3 = sm.u[warp][2 % NU][j], U4 = sm.u[warp][3 % NU][j];
-        const float beta = fmaf(xl, U1.x, fmaf(yl, U1.y, fmaf(zl, U1.z, U1.w)));
-        const float gam = fmaf(xl, U2.x, fmaf(yl, U2.y, fmaf(zl, U2.z, U2.w)));
-        const float del = fmaf(xl, U3.x, fmaf(yl, U3.y, fmaf(zl, U3.z, U3.w)));
-        const float eps = fmaf(xl, U4.x, fmaf(yl, U4.y, fmaf(zl, U4.z, U4.w)));
-        const float b2 = beta * beta;
-        const float g2 = fmaf(0.5f, b2, gam);
-        const float g3 = fmaf(beta, fmaf(b2, 1.0f / 6.0f, gam), del);
-        const float g4 = fmaf(b2 * b2, 1.0f / 24.0f,
-                              fmaf(0.5f * gam, b2 + gam, fmaf(beta, del, eps)));
-        // the polynomial of a far padding pair may overflow: select, not scale
-        acc[0] += w;
-        acc[1] = keep[jj] ? fmaf(w, beta, acc[1]) : acc[1];
-        acc[2] = keep[jj] ? fmaf(w, g2, acc[2]) : acc[2];
-        acc[3] = keep[jj] ? fmaf(w, g3, acc[3]) : acc[3];
-        acc[4] = keep[jj] ? fmaf(w, g4, acc[4]) : acc[4];
+        float b0, b1;
+        unpack2(fma2(mx, sv.v1[0], fma2(my, sv.v1[1], fma2(mz, sv.v1[2], sv.c1))), b0, b1);
+        const f32x2 beta = pack2(k0 ? b0 : 0.f, k1 ? b1 : 0.f);
+        const f32x2 gam = fma2(mx, sv.v2[0], fma2(my, sv.v2[1], fma2(mz, sv.v2[2], sv.c2)));
+        const f32x2 del = fma2(c_del, beta, add2(sv.cw, h ? zw.y : zw.x));
+        const f32x2 eps = fma2(c_eps, gam, k_eps);
+        // with b = beta / 2, c = gamma / 2: g2 = 2 (b^2 + c), g3 = 4 (b (b^2 / 3 + c) +
+        // delta / 4), g4 = 2 (b^2 (b^2 / 3 + c) + c (b^2 + c) + b delta + eps / 2)
+        const f32x2 b2 = mul2(beta, beta);
+        const f32x2 u = fma2(b2, dup2(1.0f / 3.0f), gam);
+        const f32x2 g2 = add2(b2, gam);
+        const f32x2 g3 = fma2(beta, u, mul2(dup2(0.25f), del));
+        const f32x2 g4 = fma2(b2, u, fma2(gam, g2, fma2(beta, del, eps)));
+        s[1] = fma2(w, beta, s[1]);
+        s[2] = fma2(w, g2, s[2]);
+        s[3] = fma2(w, g3, s[3]);
+        s[4] = fma2(w, g4, s[4]);
       }
     }
   }
@@ -1505,9 +1650,10 @@ __device__ __forceinline__ unsigned chunk_pairs(SolveSmem<DPS, NU>& sm, int warp
     // E_i = sum_j w e_ij = x_l W - sum_j w z_l = x_l W + M / 2; x' fixed per
     // lane: sum_j w (z~'_j x e_ij) = x' x E_i. A padding lane has W = M = 0
     // and a finite x_l.
-    const float Ex = fmaf(xl, W, 0.5f * Mx);
-    const float Ey = fmaf(yl, W, 0.5f * My);
-    const float Ez = fmaf(zl, W, 0.5f * Mz);
+    const float W = sum2(s[0]);
+    const float Ex = fmaf(xl, W, 0.5f * sum2(s[1]));
+    const float Ey = fmaf(yl, W, 0.5f * sum2(s[2]));
+    const float Ez = fmaf(zl, W, 0.5f * sum2(s[3]));
     acc[0] += W;
     acc[1] += xp.y * Ez - xp.z * Ey;
     acc[2] += xp.z * Ex - xp.x * Ez;
@@ -1515,6 +1661,12 @@ __device__ __forceinline__ unsigned chunk_pairs(SolveSmem<DPS, NU>& sm, int warp
     acc[4] += Ex;
     acc[5] += Ey;
     acc[6] += Ez;
+  } else {
+    acc[0] += sum2(s[0]);
+    acc[1] = fmaf(2.0f, sum2(s[1]), acc[1]);
+    acc[2] = fmaf(2.0f, sum2(s[2]), acc[2]);
+    acc[3] = fmaf(4.0f, sum2(s[3]), acc[3]);
+    acc[4] = fmaf(2.0f, sum2(s[4]), acc[4]);
   }
   return active;
 }
@@ -1568,7 +1720,7 @@ __device__ __forceinline__ int load_segments(const SolveCfg* cfg, SolveSmem<DPS,
 template <int DP, int DPS, int NU, bool FB>
 __device__ __forceinline__ float4 load_candidate(const GridView& g, SolveSmem<DPS, NU>& sm, int warp,
                                                  int q, int tc, int& seg, float xf[DPS]) {
-  float4 xp = make_float4(-kFar, -kFar, -kFar, 0.f);
+  float4 xp = make_float4(-kFar, -kFar, -kFar, 1.f);
 #pragma unroll
   for (int d = 0; d < DPS; ++d) xf[d] = 0.f;
   if (q < tc) {
@@ -1664,7 +1816,7 @@ __device__ __forceinline__ int stage_from_global(const SolveCfg* cfg, SolveSmem<
     for (int d = 0; d < DP; ++d)
       pf[d] = load_feat<bf16_of(MODE)>(cfg->src.feat, (size_t)d * cfg->src.m_pad + p0 + lane);
   }
-  stage_cluster<STEP, DP, DPS, NU>(sm, warp, lane, zv, p, pf);
+  stage_cluster<STEP, DP, DPS, NU>(sm, warp, lane, zv, p, pf, false);
   return cs;
 }
 
@@ -1754,7 +1906,7 @@ __device__ void pass_stream(const SolveCfg* cfg, SolveSmem<DPS, NU>& sm, int war
           const int cnt = min(32, cf.made - used);
           if (cnt <= 0) break;
           __syncwarp();
-          float4 xp = make_float4(-kFar, -kFar, -kFar, 0.f);
+          float4 xp = make_float4(-kFar, -kFar, -kFar, 1.f);
           float xf[DPS];
 #pragma unroll
           for (int d = 0; d < DPS; ++d) xf[d] = 0.f;
@@ -1823,7 +1975,7 @@ __device__ void pass_stream(const SolveCfg* cfg, SolveSmem<DPS, NU>& sm, int war
                                                            xfn);
       }
       __syncwarp();
-      float4 xp = make_float4(-kFar, -kFar, -kFar, 0.f);
+      float4 xp = make_float4(-kFar, -kFar, -kFar, 1.f);
       float xf[DPS];
 #pragma unroll
       for (int d = 0; d < DPS; ++d) xf[d] = 0.f;
@@ -2001,7 +2153,7 @@ __device__ void fill_cache(const SolveCfg* cfg, SolveSmem<DPS, NU>& sm, int warp
     const int nchk = je - jb + 1;
     for (int o = min(cur.made, want) + lane; o < 32 * nchk; o += 32) {   // padding
       float* sk = s0 + (size_t)(o >> 5) * slot_floats<DP>();
-      reinterpret_cast<float4*>(sk)[o & 31] = make_float4(-kFar, -kFar, -kFar, 0.f);
+      reinterpret_cast<float4*>(sk)[o & 31] = make_float4(-kFar, -kFar, -kFar, 1.f);
 #pragma unroll
       for (int d = 0; d < DP; ++d) sk[128 + d * 32 + (o & 31)] = 0.f;
     }
@@ -2070,21 +2222,25 @@ __device__ __forceinline__ bool list_pair(SolveSmem<DPS, NU>& sm, int warp, cons
     acc[5] = fmaf(w, ey, acc[5]);
     acc[6] = fmaf(w, ez, acc[6]);
   } else {
+    // beta / 2, gamma / 2 and the terms of chunk_pairs' step body
     const float4 U1 = sm.u[warp][0][j], U2 = sm.u[warp][1 % NU][j];
-    const float4 U3 = sm.u[warp][2 % NU][j], U4 = sm.u[warp][3 % NU][j];
-    const float beta = fmaf(xl, U1.x, fmaf(yl, U1.y, fmaf(zl, U1.z, U1.w)));
+    const float* kw = sm.b.kw;
+    float beta = fmaf(xl, U1.x, fmaf(yl, U1.y, fmaf(zl, U1.z, U1.w)));
+    beta = keep ? beta : 0.f;
     const float gam = fmaf(xl, U2.x, fmaf(yl, U2.y, fmaf(zl, U2.z, U2.w)));
-    const float del = fmaf(xl, U3.x, fmaf(yl, U3.y, fmaf(zl, U3.z, U3.w)));
-    const float eps = fmaf(xl, U4.x, fmaf(yl, U4.y, fmaf(zl, U4.z, U4.w)));
+    const float ew = fmaf(xl, kw[0], fmaf(yl, kw[1], fmaf(zl, kw[2], sm.zw[warp][j])));
+    const float del = fmaf(sm.b.c_del, beta, ew);
+    const float eps = fmaf(sm.b.c_eps, gam, sm.b.k_eps);
     const float b2 = beta * beta;
-    const float g2 = fmaf(0.5f, b2, gam);
-    const float g3 = fmaf(beta, fmaf(b2, 1.0f / 6.0f, gam), del);
-    const float g4 = fmaf(b2 * b2, 1.0f / 24.0f, fmaf(0.5f * gam, b2 + gam, fmaf(beta, del, eps)));
+    const float u = fmaf(b2, 1.0f / 3.0f, gam);
+    const float g2 = b2 + gam;
+    const float g3 = fmaf(beta, u, 0.25f * del);
+    const float g4 = fmaf(b2, u, fmaf(gam, g2, fmaf(beta, del, eps)));
     acc[0] += w;
-    acc[1] = keep ? fmaf(w, beta, acc[1]) : acc[1];
-    acc[2] = keep ? fmaf(w, g2, acc[2]) : acc[2];
-    acc[3] = keep ? fmaf(w, g3, acc[3]) : acc[3];
-    acc[4] = keep ? fmaf(w, g4, acc[4]) : acc[4];
+    acc[1] = fmaf(w, 2.0f * beta, acc[1]);
+    acc[2] = fmaf(w, 2.0f * g2, acc[2]);
+    acc[3] = fmaf(w, 4.0f * g3, acc[3]);
+    acc[4] = fmaf(w, 2.0f * g4, acc[4]);
   }
   return keep;
 }
@@ -2154,7 +2310,7 @@ __device__ void pass_cached(const SolveCfg* cfg, SolveSmem<DPS, NU>& sm, int war
       cur = sm.cache_cl[warp][s] & ((1 << kListShift) - 1);
       __syncwarp();   // every lane is done with the previous cluster
       cs = (int)(h & 0x3f);
-      stage_cluster<STEP, DP, DPS, NU>(sm, warp, lane, lane < cs, p, f);
+      stage_cluster<STEP, DP, DPS, NU>(sm, warp, lane, lane < cs, p, f, (h & kSlotList) != 0);
       cs4 = (cs + 3) & ~3;
       __syncwarp();
       if (h & kSlotList) {
@@ -2441,7 +2597,7 @@ __global__ void __launch_bounds__(kThreads, CVO_SOLVE_MIN_BLOCKS)
 solve_kernel(const SolveCfg* __restrict__ cfg, SolveState* __restrict__ st,
              double* __restrict__ partials, IterRecord* __restrict__ records, int cache_slots) {
   constexpr int DPS = DP > 0 ? DP : 1;
-  constexpr int NU = 4;
+  constexpr int NU = 2;
   __shared__ SolveSmem<DPS, NU> sm;
   extern __shared__ float4 dyn_smem[];
   solve_pair<DP, MODE, DPS, NU>(cfg, st, partials, records, Team{(int)blockIdx.x, (int)gridDim.x},
@@ -2543,7 +2699,7 @@ queue_kernel(const QueueEntry* __restrict__ entries, const QueueCtl* __restrict_
              unsigned long long* __restrict__ head, int* __restrict__ kstatus,
              unsigned long long idle_limit_ns, int cache_slots) {
   constexpr int DPS = DP > 0 ? DP : 1;
-  constexpr int NU = 4;
+  constexpr int NU = 2;
   __shared__ SolveSmem<DPS, NU> sm;
   extern __shared__ float4 dyn_smem[];
   for (;;) {
