@@ -72,6 +72,14 @@ constexpr int kCompactTeamMax = 32;
 #ifndef CVO_COST_ACTIVE
 #define CVO_COST_ACTIVE 12
 #endif
+// a warp's share of the work is cut into up to kMaxRanges pieces taken from
+// different parts of the cloud, one more for every kRangeWork pair-test units
+// of it (split_work)
+constexpr int kMaxRanges = 4;
+#ifndef CVO_RANGE_WORK
+#define CVO_RANGE_WORK 1500
+#endif
+constexpr int kRangeWork = CVO_RANGE_WORK;
 // work model: the pair bodies of a source group that kept a pair, in pair-test units
 constexpr int kCostActive = CVO_COST_ACTIVE;
 
@@ -218,9 +226,11 @@ struct BlockCtx {
   float kw[3];            // (omega . v) omega / 6 l^2
   float c_del, c_eps, k_eps;   // -|omega|^2 / 3, -|omega|^2 / 12, -(omega . v)^2 / 48 l^2
   float A, rc2, rplan_f, inv_l2f;
-  // warp ranges: from group g0 of chunk j0 of cluster c0 up to (not
-  // including) group g1 of chunk j1 of cluster c1
-  int w_c0[kWarps], w_j0[kWarps], w_g0[kWarps], w_c1[kWarps], w_j1[kWarps], w_g1[kWarps];
+  // warp ranges (n_range of them per warp): from group g0 of chunk j0 of cluster
+  // c0 up to (not including) group g1 of chunk j1 of cluster c1
+  int n_range;
+  int w_c0[kMaxRanges][kWarps], w_j0[kMaxRanges][kWarps], w_g0[kMaxRanges][kWarps];
+  int w_c1[kMaxRanges][kWarps], w_j1[kMaxRanges][kWarps], w_g1[kMaxRanges][kWarps];
   double dR[9], V[9];     // tail scratch: exp map rotation and its V matrix
 };
 
@@ -1221,8 +1231,11 @@ struct SolveSmem {
   float red[kWarps][10];
   double red_d[kWarps][16];
   long long scan[kThreads];
-  long long bnd_base[2 * kWarps];   // work offset of the group holding each warp boundary
-  int bnd_group[2 * kWarps];
+  long long wsum[kWarps];
+  long long bnd_base[2 * kWarps * kMaxRanges];   // per range end: its position in the work, then
+                                                 // (bnd_base) where the group holding it starts
+  long long bnd_at[2 * kWarps * kMaxRanges];
+  int bnd_group[2 * kWarps * kMaxRanges];
   double sums[10];
   int flag, last;
   long long q_slot;                 // queue: claimed slot (-1: none left)
@@ -1337,66 +1350,92 @@ __device__ void locate(const SolveCfg* cfg, const ClusterView& cv, int group, lo
   }
 }
 
-// Place the block's warps on an even split of the plan's work: warp w owns the
-// units (a chunk's source group) whose work starts in [floor(w TW/NW),
-// floor((w+1) TW/NW)).
+// Place the block's warps on an even split of the plan's work into NR x NW pieces
+// (NW warps in the team): a piece owns the units (a chunk's source group) whose
+// work starts in [floor(p TW / (NR NW)), floor((p + 1) TW / (NR NW))). Warp w of
+// block r takes the pieces p = (k kWarps + w) size + r, k < NR: the share of the
+// tests that keep a pair, which the plan does not know, varies smoothly over the
+// cloud, so a block whose warps take pieces from all over it ends its pass at
+// about the time the other blocks do, where one contiguous run of the work per
+// block left the slowest block 1.2 to 1.3 times the mean. Each further piece costs
+// its warp a cluster to stage and two ends to locate: one per kRangeWork units.
 template <int DPS, int NU>
 __device__ void split_work(const SolveCfg* cfg, SolveSmem<DPS, NU>& sm, int tid, Team team) {
   const ClusterView& cv = cfg->clusters[sm.b.level];
+  const int lane = tid & 31, warp = tid >> 5;
   const int ng = (cv.ncl + 31) / 32;
   const int per = (ng + kThreads - 1) / kThreads;
   const int g0 = min(ng, tid * per), g1 = min(ng, g0 + per);
   long long local = 0;
   for (int gi = g0; gi < g1; ++gi) local += __ldcg(&cfg->group_agg[gi]);
-  sm.scan[tid] = local;
-  if (tid < 2 * kWarps) sm.bnd_group[tid] = -1;
-  __syncthreads();
-  for (int off = 1; off < kThreads; off <<= 1) {
-    const long long v = tid >= off ? sm.scan[tid - off] : 0;
-    __syncthreads();
-    sm.scan[tid] += v;
-    __syncthreads();
-  }
-  const long long TW = sm.scan[kThreads - 1];
-  const long long NW = (long long)team.size * kWarps;
-  long long run = sm.scan[tid] - local;
-  for (int gi = g0; gi < g1; ++gi) {
-    const long long gtests = __ldcg(&cfg->group_agg[gi]);
+  // inclusive scan over the block's threads: within warps, then the warp totals
+  long long incl = local;
 #pragma unroll
-    for (int q = 0; q < 2 * kWarps; ++q) {
-      const long long w = (long long)team.rank * kWarps + (q >> 1) + (q & 1);
-      const long long s = TW > 0 ? (w * TW) / NW : 0;
-      if (gtests > 0 && s >= run && s < run + gtests) {
-        sm.bnd_group[q] = gi;
-        sm.bnd_base[q] = run;
+  for (int off = 1; off < 32; off <<= 1) {
+    const long long v = __shfl_up_sync(kFull, incl, off);
+    if (lane >= off) incl += v;
+  }
+  if (lane == 31) sm.wsum[warp] = incl;
+  __syncthreads();
+  long long TW = 0;
+#pragma unroll
+  for (int w = 0; w < kWarps; ++w) {
+    if (w < warp) incl += sm.wsum[w];
+    TW += sm.wsum[w];
+  }
+  sm.scan[tid] = incl;
+  const long long NW = (long long)team.size * kWarps;
+  const int nr = (int)min((long long)kMaxRanges, max(1ll, TW / (NW * kRangeWork)));
+  __syncthreads();
+  // end h of the k-th piece of warp w on thread (k kWarps + w) 2 + h: the thread
+  // whose run of groups holds it, by binary search, then the group
+  if (tid < 2 * kWarps * nr) {
+    const long long piece = (long long)(tid >> 1) * team.size + team.rank + (tid & 1);
+    const long long at = TW > 0 ? (piece * TW) / (NW * nr) : 0;
+    int group = -1;
+    long long base = 0;
+    if (at < TW) {
+      int lo = 0, hi = kThreads - 1;   // the first thread whose inclusive sum is beyond `at`
+      while (lo < hi) {
+        const int mid = (lo + hi) >> 1;
+        if (sm.scan[mid] > at) hi = mid;
+        else lo = mid + 1;
+      }
+      base = lo > 0 ? sm.scan[lo - 1] : 0;
+      const int ge = min(ng, (lo + 1) * per);
+      for (int gi = lo * per; gi < ge; ++gi) {
+        const long long w = __ldcg(&cfg->group_agg[gi]);
+        if (at < base + w) {
+          group = gi;
+          break;
+        }
+        base += w;
       }
     }
-    run += gtests;
+    sm.bnd_group[tid] = group;
+    sm.bnd_base[tid] = base;
+    sm.bnd_at[tid] = at;
   }
+  if (tid == 0) sm.b.n_range = nr;
   __syncthreads();
-  const int lane = tid & 31, warp = tid >> 5;
+  for (int k = 0; k < nr; ++k) {
 #pragma unroll
-  for (int h = 0; h < 2; ++h) {
-    const int q = 2 * warp + h;
-    const long long w = (long long)team.rank * kWarps + warp + h;
-    const long long s = TW > 0 ? (w * TW) / NW : 0;
-    int c, jj, gg;
-    if (TW == 0 || s >= TW || sm.bnd_group[q] < 0) {
-      c = cv.ncl;   // past the end: no chunk
-      jj = gg = 0;
-    } else {
-      locate(cfg, cv, sm.bnd_group[q], sm.bnd_base[q], s, lane, &c, &jj, &gg,
-             sm.b.use_kept != 0, sm.b.use_act != 0);
-    }
-    if (lane == 0) {
-      if (h == 0) {
-        sm.b.w_c0[warp] = c;
-        sm.b.w_j0[warp] = jj;
-        sm.b.w_g0[warp] = gg;
-      } else {
-        sm.b.w_c1[warp] = c;
-        sm.b.w_j1[warp] = jj;
-        sm.b.w_g1[warp] = gg;
+    for (int h = 0; h < 2; ++h) {
+      const int q = 2 * (k * kWarps + warp) + h;
+      int c = cv.ncl, jj = 0, gg = 0;   // past the end: no chunk
+      if (sm.bnd_group[q] >= 0)
+        locate(cfg, cv, sm.bnd_group[q], sm.bnd_base[q], sm.bnd_at[q], lane, &c, &jj, &gg,
+               sm.b.use_kept != 0, sm.b.use_act != 0);
+      if (lane == 0) {
+        if (h == 0) {
+          sm.b.w_c0[k][warp] = c;
+          sm.b.w_j0[k][warp] = jj;
+          sm.b.w_g0[k][warp] = gg;
+        } else {
+          sm.b.w_c1[k][warp] = c;
+          sm.b.w_j1[k][warp] = jj;
+          sm.b.w_g1[k][warp] = gg;
+        }
       }
     }
   }
@@ -1671,14 +1710,14 @@ __device__ __forceinline__ unsigned chunk_pairs(SolveSmem<DPS, NU>& sm, int warp
   return active;
 }
 
-// A warp's range of work (BlockCtx::w_*).
+// A warp's k-th range of work (BlockCtx::w_*).
 struct WarpRange {
   int c0, j0, g0, c1, j1, g1;
 };
 
-__device__ __forceinline__ WarpRange warp_range(const BlockCtx& b, int warp) {
-  return WarpRange{b.w_c0[warp], b.w_j0[warp], b.w_g0[warp],
-                   b.w_c1[warp], b.w_j1[warp], b.w_g1[warp]};
+__device__ __forceinline__ WarpRange warp_range(const BlockCtx& b, int warp, int k) {
+  return WarpRange{b.w_c0[k][warp], b.w_j0[k][warp], b.w_g0[k][warp],
+                   b.w_c1[k][warp], b.w_j1[k][warp], b.w_g1[k][warp]};
 }
 
 // Chunks [jb, je] of cluster c (nch chunks) that hold work of the range.
@@ -1820,20 +1859,20 @@ __device__ __forceinline__ int stage_from_global(const SolveCfg* cfg, SolveSmem<
   return cs;
 }
 
-// One warp's share of a pair pass, streamed from global memory (L2): lane
+// One range of a warp's share of a pair pass, streamed from global memory (L2): lane
 // sums in acc, counts in nnz / cand. The filtered candidates of each chunk
 // are gathered through a ring of 64 entries in the warp's (otherwise unused)
 // cache region, with the next block of 32 candidates loading while the
 // current chunk runs.
 template <bool STEP, int DP, int MODE, int DPS, int NU>
 __device__ void pass_stream(const SolveCfg* cfg, SolveSmem<DPS, NU>& sm, int warp, int lane,
-                            float* ring, float acc[7], unsigned& nnz, unsigned& cand) {
+                            int range, float* ring, float acc[7], unsigned& nnz, unsigned& cand) {
   const BlockCtx& b = sm.b;
   const GridView& g = cfg->grids[b.level];
   const ClusterView& cv = cfg->clusters[b.level];
   const float rc2 = b.rc2, A = b.A;
   const float rp2 = b.rplan_f * b.rplan_f;
-  const WarpRange r = warp_range(b, warp);
+  const WarpRange r = warp_range(b, warp, range);
   const bool collect = !STEP && b.collect_kept;
   float4* rxyz = reinterpret_cast<float4*>(ring);
   float* rfeat = ring + 4 * 64;
@@ -2092,10 +2131,10 @@ __device__ void fill_cache(const SolveCfg* cfg, SolveSmem<DPS, NU>& sm, int warp
   const BlockCtx& b = sm.b;
   const GridView& g = cfg->grids[b.level];
   const ClusterView& cv = cfg->clusters[b.level];
-  const WarpRange r = warp_range(b, warp);
+  const WarpRange r = warp_range(b, warp, 0);
   const float rp2 = b.rplan_f * b.rplan_f;
-  // count the slots the share needs
-  int need = 0;
+  // count the slots the share needs (one in several pieces is too large for them)
+  int need = b.n_range > 1 ? kCacheSlots + 1 : 0;
   for (int c = r.c0; c <= r.c1 && c < cv.ncl; ++c) {
     int jb, je;
     if (range_chunks(r, c, (__ldcg(&cfg->cl_fcand[c]) + 31) >> 5, jb, je)) need += 2 + je - jb;
@@ -2350,9 +2389,10 @@ __device__ __forceinline__ void pass_warp(const SolveCfg* cfg, SolveSmem<DPS, NU
   if (sm.cache_n[warp] >= 0)
     pass_cached<STEP, DP, MODE, DPS, NU>(cfg, sm, warp, lane, cache, slots, acc, nnz, cand);
   else
-    pass_stream<STEP, DP, MODE, DPS, NU>(cfg, sm, warp, lane,
-                                         cache + (size_t)warp * slots * slot_floats<DP>(), acc,
-                                         nnz, cand);
+    for (int k = 0; k < sm.b.n_range; ++k)
+      pass_stream<STEP, DP, MODE, DPS, NU>(cfg, sm, warp, lane, k,
+                                           cache + (size_t)warp * slots * slot_floats<DP>(), acc,
+                                           nnz, cand);
 }
 
 // One pass over the block's warps, then the block partial (fixed order).
