@@ -6,18 +6,24 @@
 //   pixels     validity (depth in range), intensity gradient of the V channel
 //              (central differences, one-sided at the border) and its
 //              magnitude, FP32 with one rounding per operation
-//   threshold  the valid magnitudes are compacted, radix-sorted on their bit
-//              patterns (non-negative floats sort as integers) and the
-//              linear-interpolation percentile taken from the order
-//              statistics in FP64
-//   keep       valid and magnitude > threshold; a device-wide scan ranks the
-//              kept pixels in raster order; above max_points the ranks
-//              floor(k m / max_points) are kept
+//   threshold  the linear-interpolation percentile of the valid magnitudes, in
+//              FP64, from its two order statistics, which a radix select on the
+//              bit patterns finds (non-negative floats order as integers): three
+//              histograms of 11, 11 and 10 bits, each of the magnitudes that
+//              share the digits found so far
+//   keep       valid and magnitude > threshold; kept pixels are counted per
+//              block, ranked in raster order from the counts before their
+//              block; above max_points the ranks floor(k m / max_points) are
+//              kept
 //   points     z = depth, x = ((u - cx) / fx) z, y = ((v - cy) / fy) z and the
 //              features H, S, V, clip(gx / s), clip(gy / s), FP32
 //
 // Pixel selection is index work: the kept set and its order are exact, the
-// same on any run.
+// same on any run. Five launches and one wait: at 640 x 480 every kernel is a few
+// microseconds of latency, so what counts is how few there are (sorting the
+// magnitudes to read two of them took 12 of the 23 launches, and their count had
+// to visit the host): 279 -> 87 us per frame, of which the call's host side, with
+// its allocation, wait and read-back, is about a third.
 #include <cuda_runtime.h>
 
 #include <algorithm>
@@ -37,117 +43,238 @@ __device__ __forceinline__ float intensity(const float* hsv, int W, int x, int y
   return hsv[3 * ((size_t)y * W + x) + 2];
 }
 
-__global__ void fe_pixels_kernel(const float* __restrict__ depth, const float* __restrict__ hsv,
-                                 int W, int H, float dmin, float dmax, float* __restrict__ gxo,
-                                 float* __restrict__ gyo, float* __restrict__ mag,
-                                 int* __restrict__ valid) {
-  const int p = blockIdx.x * blockDim.x + threadIdx.x;
-  if (p >= W * H) return;
-  const int y = p / W, x = p - y * W;
-  float gx, gy;
+// Intensity gradient of pixel (x, y).
+__device__ __forceinline__ void fe_gradient(const float* hsv, int W, int H, int x, int y, float& gx,
+                                            float& gy) {
   if (x == 0) gx = __fsub_rn(intensity(hsv, W, 1, y), intensity(hsv, W, 0, y));
   else if (x == W - 1) gx = __fsub_rn(intensity(hsv, W, W - 1, y), intensity(hsv, W, W - 2, y));
   else gx = __fmul_rn(0.5f, __fsub_rn(intensity(hsv, W, x + 1, y), intensity(hsv, W, x - 1, y)));
   if (y == 0) gy = __fsub_rn(intensity(hsv, W, x, 1), intensity(hsv, W, x, 0));
   else if (y == H - 1) gy = __fsub_rn(intensity(hsv, W, x, H - 1), intensity(hsv, W, x, H - 2));
   else gy = __fmul_rn(0.5f, __fsub_rn(intensity(hsv, W, x, y + 1), intensity(hsv, W, x, y - 1)));
-  gxo[p] = gx;
-  gyo[p] = gy;
-  mag[p] = __fsqrt_rn(__fadd_rn(__fmul_rn(gx, gx), __fmul_rn(gy, gy)));
-  const float d = depth[p];
-  valid[p] = (isfinite(d) && d >= dmin && d <= dmax) ? 1 : 0;
 }
 
-// Exclusive scan of one block of kScanBlock flags; block totals to sums[].
-__global__ void fe_scan_block_kernel(const int* __restrict__ in, int n, int* __restrict__ out,
-                                     int* __restrict__ sums) {
-  __shared__ int s[kScanBlock];
-  const int t = threadIdx.x;
-  const int i = blockIdx.x * kScanBlock + t;
-  const int v = i < n ? in[i] : 0;
-  s[t] = v;
+// Device scratch of a selection, zeroed before each run.
+struct FeCounts {
+  unsigned hist[3][2048];     // digit counts: top 11 bits, next 11, last 10
+  unsigned above;             // ~(smallest key beyond the first two digits found)
+  int kept[kScanBlock];       // kept pixels per block of kScanBlock pixels
+};
+
+// The key of a pixel without a valid depth: no magnitude has it (a NaN result
+// is 0x7fffffff).
+constexpr unsigned kNoKey = 0xffffffffu;
+
+// Adds the block's shared digit counts to the device's.
+__device__ __forceinline__ void fe_flush(const unsigned* s_hist, unsigned* hist) {
   __syncthreads();
-  for (int off = 1; off < kScanBlock; off <<= 1) {
-    const int a = t >= off ? s[t - off] : 0;
-    __syncthreads();
-    s[t] += a;
-    __syncthreads();
-  }
-  if (i < n) out[i] = s[t] - v;
-  if (t == kScanBlock - 1) sums[blockIdx.x] = s[t];
+  for (int i = threadIdx.x; i < 2048; i += kScanBlock)
+    if (s_hist[i]) atomicAdd(&hist[i], s_hist[i]);
 }
 
-// Exclusive scan of the block totals (one block, nb <= kScanBlock); total[0]
-// receives the grand total.
-__global__ void fe_scan_sums_kernel(int* __restrict__ sums, int nb, int* __restrict__ total) {
-  __shared__ int s[kScanBlock];
-  const int t = threadIdx.x;
-  const int v = t < nb ? sums[t] : 0;
-  s[t] = v;
+__global__ void __launch_bounds__(kScanBlock)
+fe_pixels_kernel(const float* __restrict__ depth, const float* __restrict__ hsv, int W, int H,
+                 float dmin, float dmax, unsigned* __restrict__ keys, FeCounts* __restrict__ c) {
+  __shared__ unsigned s_hist[2048];
+  for (int i = threadIdx.x; i < 2048; i += kScanBlock) s_hist[i] = 0u;
   __syncthreads();
-  for (int off = 1; off < kScanBlock; off <<= 1) {
-    const int a = t >= off ? s[t - off] : 0;
-    __syncthreads();
-    s[t] += a;
-    __syncthreads();
+  const int p = blockIdx.x * kScanBlock + threadIdx.x;
+  if (p < W * H) {
+    const int y = p / W, x = p - y * W;
+    float gx, gy;
+    fe_gradient(hsv, W, H, x, y, gx, gy);
+    const float mag = __fsqrt_rn(__fadd_rn(__fmul_rn(gx, gx), __fmul_rn(gy, gy)));
+    const float d = depth[p];
+    const bool valid = isfinite(d) && d >= dmin && d <= dmax;
+    const unsigned key = valid ? __float_as_uint(mag) : kNoKey;
+    keys[p] = key;
+    if (valid) atomicAdd(&s_hist[key >> 21], 1u);
   }
-  if (t < nb) sums[t] = s[t] - v;
-  if (t == kScanBlock - 1) *total = s[t];
+  fe_flush(s_hist, c->hist[0]);
 }
 
-__global__ void fe_scan_add_kernel(int* __restrict__ out, int n, const int* __restrict__ sums) {
-  const int i = blockIdx.x * kScanBlock + threadIdx.x;
-  if (i < n) out[i] += sums[blockIdx.x];
-}
+// Where rank r falls in 2048 digit counts: the digit, the rank left within it
+// and the total. Every thread of the block calls it (kScanBlock threads, two
+// digits each); a rank at or beyond the total gives digit 2047.
+struct FeDigit {
+  unsigned digit, left, total;
+};
 
-// Magnitudes of the valid pixels, compacted, as sort keys.
-__global__ void fe_compact_kernel(const float* __restrict__ mag, const int* __restrict__ valid,
-                                  const int* __restrict__ pos, int n, uint32_t* __restrict__ keys,
-                                  uint32_t* __restrict__ vals) {
-  const int p = blockIdx.x * blockDim.x + threadIdx.x;
-  if (p >= n || !valid[p]) return;
-  keys[pos[p]] = __float_as_uint(mag[p]);
-  vals[pos[p]] = (uint32_t)p;
-}
-
-// The linear-interpolation percentile (numpy's 'linear' method) of the sorted
-// valid magnitudes, FP64, one thread.
-__global__ void fe_threshold_kernel(const uint32_t* __restrict__ sorted, const int* __restrict__ nv,
-                                    double q, double* __restrict__ thr) {
-  const int n = *nv;
-  if (n <= 0) {
-    *thr = 0.0;
-    return;
+__device__ FeDigit fe_find(const unsigned* hist, unsigned rank) {
+  __shared__ unsigned s_warp[kScanBlock / 32];
+  __shared__ FeDigit s_found;
+  const int t = threadIdx.x, lane = t & 31, warp = t >> 5;
+  const unsigned a = __ldcg(&hist[2 * t]), b = __ldcg(&hist[2 * t + 1]);
+  unsigned incl = a + b;
+  for (int off = 1; off < 32; off <<= 1) {
+    const unsigned v = __shfl_up_sync(0xffffffffu, incl, off);
+    if (lane >= off) incl += v;
   }
-  const double h = (double)(n - 1) * (q / 100.0);
-  const int lo = (int)floor(h);
-  const int hi = min(lo + 1, n - 1);
-  const double t = h - (double)lo;
-  const double a = (double)__uint_as_float(sorted[lo]), b = (double)__uint_as_float(sorted[hi]);
-  const double d = b - a;
-  *thr = t < 0.5 ? a + d * t : b - d * (1.0 - t);
+  __syncthreads();   // the shared words of an earlier call have been read
+  if (lane == 31) s_warp[warp] = incl;
+  if (t == 0) s_found = FeDigit{2047u, 0u, 0u};
+  __syncthreads();
+  unsigned total = 0u;
+  for (int w = 0; w < kScanBlock / 32; ++w) {
+    if (w < warp) incl += s_warp[w];
+    total += s_warp[w];
+  }
+  const unsigned before = incl - a - b;
+  if (rank >= before && rank < incl) {
+    const bool second = rank >= before + a;
+    s_found.digit = 2u * t + (second ? 1u : 0u);
+    s_found.left = rank - before - (second ? a : 0u);
+  }
+  __syncthreads();
+  FeDigit f = s_found;
+  f.total = total;
+  return f;
 }
 
-__global__ void fe_keep_kernel(const float* __restrict__ mag, const int* __restrict__ valid, int n,
-                               const double* __restrict__ thr, int* __restrict__ keep) {
-  const int p = blockIdx.x * blockDim.x + threadIdx.x;
-  if (p >= n) return;
-  keep[p] = (valid[p] && (double)mag[p] > *thr) ? 1 : 0;
+// The lower order statistic's rank among n values at percentile q, and the FP64
+// position (numpy's 'linear' method).
+__device__ __forceinline__ unsigned fe_rank(unsigned n, double q, double* h) {
+  *h = n > 0u ? (double)(int)(n - 1u) * (q / 100.0) : 0.0;
+  return (unsigned)(int)floor(*h);
+}
+
+// The digits found so far: the top one (level 1), and the next (level 2).
+struct FePrefix {
+  unsigned n, rank, d0, d1, left;
+  double h;
+};
+
+__device__ FePrefix fe_prefix(const FeCounts* c, double q, int level) {
+  __shared__ unsigned s_rank;
+  __shared__ double s_h;
+  FePrefix f;
+  FeDigit d = fe_find(c->hist[0], 0u);
+  f.n = d.total;
+  if (threadIdx.x == 0) {   // FP64 on one thread of one warp
+    double h;
+    s_rank = fe_rank(f.n, q, &h);
+    s_h = h;
+  }
+  __syncthreads();
+  f.rank = s_rank;
+  f.h = s_h;
+  d = fe_find(c->hist[0], f.rank);
+  f.d0 = d.digit;
+  f.left = d.left;
+  f.d1 = 0u;
+  if (level > 1) {
+    d = fe_find(c->hist[1], f.left);
+    f.d1 = d.digit;
+    f.left = d.left;
+  }
+  return f;
+}
+
+// Digit counts of the keys that share the digits found so far; at the last
+// level also the smallest key beyond them (where the upper order statistic lies
+// when the lower one is the last of its prefix).
+__global__ void __launch_bounds__(kScanBlock)
+fe_digits_kernel(const unsigned* __restrict__ keys, int n, double q, int level,
+                 FeCounts* __restrict__ c) {
+  __shared__ unsigned s_hist[2048];
+  __shared__ unsigned s_above;
+  for (int i = threadIdx.x; i < 2048; i += kScanBlock) s_hist[i] = 0u;
+  if (threadIdx.x == 0) s_above = 0u;
+  const FePrefix f = fe_prefix(c, q, level);
+  __syncthreads();
+  const int p = blockIdx.x * kScanBlock + threadIdx.x;
+  if (p < n) {
+    const unsigned key = keys[p];
+    if (key != kNoKey) {
+      if (level == 1) {
+        if (key >> 21 == f.d0) atomicAdd(&s_hist[(key >> 10) & 2047u], 1u);
+      } else {
+        const unsigned pre = f.d0 << 11 | f.d1;
+        if (key >> 10 == pre) atomicAdd(&s_hist[key & 1023u], 1u);
+        else if (key >> 10 > pre && ~key > s_above) atomicMax(&s_above, ~key);
+      }
+    }
+  }
+  fe_flush(s_hist, c->hist[level]);
+  if (level == 2 && threadIdx.x == 0 && s_above) atomicMax(&c->above, s_above);
+}
+
+// The percentile, from its two order statistics, in FP64.
+__device__ double fe_threshold(const FeCounts* c, double q) {
+  __shared__ double s_thr;
+  const FePrefix f = fe_prefix(c, q, 2);
+  const FeDigit lo = fe_find(c->hist[2], f.left), hi = fe_find(c->hist[2], f.left + 1u);
+  if (threadIdx.x == 0) {
+    const unsigned pre = (f.d0 << 11 | f.d1) << 10;
+    const unsigned ka = pre | lo.digit;
+    // the next rank: in the same prefix, beyond it, or (the last rank) the same
+    const unsigned kb = f.rank + 1u >= f.n ? ka : f.left + 1u < hi.total ? pre | hi.digit
+                                                                         : ~__ldcg(&c->above);
+    const double t = f.h - (double)(int)f.rank;
+    const double a = (double)__uint_as_float(ka), b = (double)__uint_as_float(kb);
+    const double d = b - a;
+    s_thr = f.n > 0u ? (t < 0.5 ? a + d * t : b - d * (1.0 - t)) : 0.0;
+  }
+  __syncthreads();
+  return s_thr;
+}
+
+__device__ __forceinline__ bool fe_kept(unsigned key, double thr) {
+  return key != kNoKey && (double)__uint_as_float(key) > thr;
+}
+
+// Kept pixels per block; block 0 leaves the threshold for the next kernel.
+__global__ void __launch_bounds__(kScanBlock)
+fe_count_kernel(const unsigned* __restrict__ keys, int n, double q, FeCounts* __restrict__ c,
+                double* __restrict__ thr_out) {
+  const double thr = fe_threshold(c, q);
+  const int p = blockIdx.x * kScanBlock + threadIdx.x;
+  const int m = __syncthreads_count(p < n && fe_kept(keys[p], thr));
+  if (threadIdx.x == 0) {
+    c->kept[blockIdx.x] = m;
+    if (blockIdx.x == 0) *thr_out = thr;
+  }
 }
 
 // Kept pixel of rank r goes to output slot r, or, when m > cap, to the slot k
-// with floor(k m / cap) == r (if any).
-__global__ void fe_emit_kernel(const float* __restrict__ depth, const float* __restrict__ hsv,
-                               const float* __restrict__ gx, const float* __restrict__ gy,
-                               const int* __restrict__ keep, const int* __restrict__ rank,
-                               const int* __restrict__ m_total, int W, int H, long long cap,
-                               float fx, float fy, float cx, float cy, float gs,
-                               float* __restrict__ out_xyz, float* __restrict__ out_feat,
-                               int* __restrict__ out_pix) {
-  const int p = blockIdx.x * blockDim.x + threadIdx.x;
-  if (p >= W * H || !keep[p]) return;
-  const long long m = *m_total;
-  const long long r = rank[p];
+// with floor(k m / cap) == r (if any). Nothing is written when more points than
+// `room` would be (room 0: there is room for every pixel). totals: valid pixels,
+// kept pixels.
+__global__ void __launch_bounds__(kScanBlock)
+fe_emit_kernel(const float* __restrict__ depth, const float* __restrict__ hsv,
+               const unsigned* __restrict__ keys, const FeCounts* __restrict__ c,
+               const double* __restrict__ thr, int W, int H, long long cap, long long room,
+               float fx, float fy, float cx, float cy, float gs, float* __restrict__ out_xyz,
+               float* __restrict__ out_feat, int* __restrict__ out_pix, int* __restrict__ totals) {
+  __shared__ int s_before[kScanBlock / 32], s_total[kScanBlock / 32], s_warp[kScanBlock / 32];
+  const int t = threadIdx.x, lane = t & 31, warp = t >> 5;
+  // kept pixels in the blocks before this one, and in all of them
+  const int v = t < (int)gridDim.x ? __ldcg(&c->kept[t]) : 0;
+  const int vb = __reduce_add_sync(0xffffffffu, t < (int)blockIdx.x ? v : 0);
+  const int va = __reduce_add_sync(0xffffffffu, v);
+  const int p = blockIdx.x * kScanBlock + t;
+  const bool keep = p < W * H && fe_kept(keys[p], *thr);
+  const unsigned mask = __ballot_sync(0xffffffffu, keep);
+  if (lane == 0) {
+    s_before[warp] = vb;
+    s_total[warp] = va;
+    s_warp[warp] = __popc(mask);
+  }
+  __syncthreads();
+  long long m = 0, r = __popc(mask & ((1u << lane) - 1u));
+  for (int w = 0; w < kScanBlock / 32; ++w) {
+    m += s_total[w];
+    r += s_before[w] + (w < warp ? s_warp[w] : 0);
+  }
+  if (blockIdx.x == 0) {
+    const FeDigit all = fe_find(c->hist[0], 0u);   // its total is every valid pixel
+    if (t == 0) {
+      totals[0] = (int)all.total;
+      totals[1] = (int)m;
+    }
+  }
+  const long long n_emit = cap > 0 && m > cap ? cap : m;
+  if (!keep || (room > 0 && n_emit > room)) return;
   long long k = r;
   if (cap > 0 && m > cap) {
     k = (r * cap + m - 1) / m;   // smallest k with k m / cap >= r
@@ -159,25 +286,18 @@ __global__ void fe_emit_kernel(const float* __restrict__ depth, const float* __r
   out_xyz[3 * k + 1] = __fmul_rn(__fdiv_rn(__fsub_rn((float)y, cy), fy), z);
   out_xyz[3 * k + 2] = z;
   if (out_feat) {
+    float gx, gy;
+    fe_gradient(hsv, W, H, x, y, gx, gy);
     out_feat[5 * k + 0] = hsv[3 * (size_t)p + 0];
     out_feat[5 * k + 1] = hsv[3 * (size_t)p + 1];
     out_feat[5 * k + 2] = hsv[3 * (size_t)p + 2];
-    out_feat[5 * k + 3] = fminf(fmaxf(__fdiv_rn(gx[p], gs), -1.0f), 1.0f);
-    out_feat[5 * k + 4] = fminf(fmaxf(__fdiv_rn(gy[p], gs), -1.0f), 1.0f);
+    out_feat[5 * k + 3] = fminf(fmaxf(__fdiv_rn(gx, gs), -1.0f), 1.0f);
+    out_feat[5 * k + 4] = fminf(fmaxf(__fdiv_rn(gy, gs), -1.0f), 1.0f);
   }
   if (out_pix) out_pix[k] = p;
 }
 
 inline int nblocks(long long n, int t) { return (int)((n + t - 1) / t); }
-
-// Exclusive scan of n flags into out; the total lands in d_total (device).
-cudaError_t scan_flags(const int* in, int n, int* out, int* sums, int* d_total, cudaStream_t s) {
-  const int nb = nblocks(n, kScanBlock);
-  fe_scan_block_kernel<<<nb, kScanBlock, 0, s>>>(in, n, out, sums);
-  fe_scan_sums_kernel<<<1, kScanBlock, 0, s>>>(sums, nb, d_total);
-  fe_scan_add_kernel<<<nb, kScanBlock, 0, s>>>(out, n, sums);
-  return cudaGetLastError();
-}
 
 // The selection into caller-visible device buffers (context lock held).
 // out_xyz / out_feat / out_pix have room for cap points (cap > 0) or for
@@ -196,13 +316,13 @@ int frontend_run(cvo_ctx* ctx, const float* depth, const float* hsv, int W, int 
   const int n = (int)npix;
   const int nb = nblocks(n, kScanBlock);
   // one scratch allocation carved into 256-byte aligned pieces, sized with the
-  // same rounding the carving uses: thr, totals, block sums, the images (when
-  // they come from the host), then the per-pixel arrays
+  // same rounding the carving uses: counts, threshold, totals, the images (when
+  // they come from the host) and the keys
   auto round_up = [](size_t b) { return (b + 255) / 256 * 256; };
   const size_t pix4 = round_up(sizeof(float) * (size_t)n);
-  const size_t bytes = round_up(sizeof(double) * 2) + round_up(sizeof(int) * 4) +
-                       round_up(sizeof(int) * (size_t)(nb + 1)) +
-                       (on_dev ? 0 : pix4 + round_up(sizeof(float) * 3 * (size_t)n)) + 9 * pix4;
+  const size_t bytes = round_up(sizeof(FeCounts)) + round_up(sizeof(double)) +
+                       round_up(sizeof(int) * 2) +
+                       (on_dev ? 0 : pix4 + round_up(sizeof(float) * 3 * (size_t)n)) + pix4;
   char* scratch = nullptr;
   if (cudaMallocFromPoolAsync((void**)&scratch, bytes, ctx->pool, s) != cudaSuccess)
     return fail(ctx, CVO_ERR_CUDA, "front-end scratch allocation failed");
@@ -212,9 +332,9 @@ int frontend_run(cvo_ctx* ctx, const float* depth, const float* hsv, int W, int 
     cur += round_up(b);
     return r;
   };
-  double* thr = (double*)take(sizeof(double) * 2);
-  int* totals = (int*)take(sizeof(int) * 4);   // [0] valid count, [1] kept count
-  int* sums = (int*)take(sizeof(int) * (size_t)(nb + 1));
+  FeCounts* counts = (FeCounts*)take(sizeof(FeCounts));
+  double* thr = (double*)take(sizeof(double));
+  int* totals = (int*)take(sizeof(int) * 2);   // valid pixels, kept pixels
   const float* d_depth = depth;
   const float* d_hsv = hsv;
   cudaError_t e = cudaSuccess;
@@ -233,60 +353,33 @@ int frontend_run(cvo_ctx* ctx, const float* depth, const float* hsv, int W, int 
     if (e == cudaSuccess) e = cudaStreamWaitEvent(s, ev, 0);
     cudaEventDestroy(ev);
   }
-  float* gx = (float*)take(sizeof(float) * (size_t)n);
-  float* gy = (float*)take(sizeof(float) * (size_t)n);
-  float* mag = (float*)take(sizeof(float) * (size_t)n);
-  int* valid = (int*)take(sizeof(int) * (size_t)n);
-  int* pos = (int*)take(sizeof(int) * (size_t)n);
-  int* keep = (int*)take(sizeof(int) * (size_t)n);
-  int* rank = (int*)take(sizeof(int) * (size_t)n);
-  uint32_t* keys = (uint32_t*)take(sizeof(uint32_t) * (size_t)n);
-  uint32_t* vals = (uint32_t*)take(sizeof(uint32_t) * (size_t)n);
+  unsigned* keys = (unsigned*)take(sizeof(unsigned) * (size_t)n);
   if ((size_t)(cur - scratch) > bytes) {   // the sizing above must cover the carving
     cudaFreeAsync(scratch, s);
     return fail(ctx, CVO_ERR_INTERNAL, "front-end scratch sizing");
   }
-  const int T = 256;
+  if (e == cudaSuccess) e = cudaMemsetAsync(counts, 0, sizeof(FeCounts), s);
   if (e == cudaSuccess) {
-    fe_pixels_kernel<<<nblocks(n, T), T, 0, s>>>(d_depth, d_hsv, W, H, (float)fp.depth_min,
-                                                 (float)fp.depth_max, gx, gy, mag, valid);
+    fe_pixels_kernel<<<nb, kScanBlock, 0, s>>>(d_depth, d_hsv, W, H, (float)fp.depth_min,
+                                               (float)fp.depth_max, keys, counts);
+    fe_digits_kernel<<<nb, kScanBlock, 0, s>>>(keys, n, fp.percentile, 1, counts);
+    fe_digits_kernel<<<nb, kScanBlock, 0, s>>>(keys, n, fp.percentile, 2, counts);
+    fe_count_kernel<<<nb, kScanBlock, 0, s>>>(keys, n, fp.percentile, counts, thr);
+    fe_emit_kernel<<<nb, kScanBlock, 0, s>>>(
+        d_depth, d_hsv, keys, counts, thr, W, H, fp.max_points, cap, (float)fp.fx, (float)fp.fy,
+        (float)fp.cx, (float)fp.cy, (float)fp.grad_scale, out_xyz, out_feat, out_pix, totals);
     e = cudaGetLastError();
   }
-  if (e == cudaSuccess) e = scan_flags(valid, n, pos, sums, totals + 0, s);
-  if (e == cudaSuccess) {
-    fe_compact_kernel<<<nblocks(n, T), T, 0, s>>>(mag, valid, pos, n, keys, vals);
-    e = cudaGetLastError();
-  }
-  // the sort needs the count on the host
-  if (e == cudaSuccess)
-    e = cudaMemcpyAsync(ctx->h_int, totals, sizeof(int), cudaMemcpyDeviceToHost, s);
-  if (e == cudaSuccess) e = cudaStreamSynchronize(s);
-  const int n_valid = e == cudaSuccess ? ctx->h_int[0] : 0;
-  if (e == cudaSuccess && n_valid > 1) e = radix_sort_pairs(keys, vals, n_valid, 32, ctx->pool, s);
-  if (e == cudaSuccess) {
-    fe_threshold_kernel<<<1, 1, 0, s>>>(keys, totals + 0, fp.percentile, thr);
-    fe_keep_kernel<<<nblocks(n, T), T, 0, s>>>(mag, valid, n, thr, keep);
-    e = cudaGetLastError();
-  }
-  if (e == cudaSuccess) e = scan_flags(keep, n, rank, sums, totals + 1, s);
   if (e == cudaSuccess)
     e = cudaMemcpyAsync(ctx->h_int, totals, sizeof(int) * 2, cudaMemcpyDeviceToHost, s);
+  cudaFreeAsync(scratch, s);
   if (e == cudaSuccess) e = cudaStreamSynchronize(s);
+  const int n_valid = e == cudaSuccess ? ctx->h_int[0] : 0;
   const long long m = e == cudaSuccess ? ctx->h_int[1] : 0;
   long long n_emit = m;
   if (fp.max_points > 0 && m > fp.max_points) n_emit = fp.max_points;
-  if (e == cudaSuccess && cap > 0 && n_emit > cap) {
-    cudaFreeAsync(scratch, s);
+  if (e == cudaSuccess && cap > 0 && n_emit > cap)
     return fail(ctx, CVO_ERR_INVALID_ARG, "output buffers too small for the selected points");
-  }
-  if (e == cudaSuccess && n_emit > 0) {
-    fe_emit_kernel<<<nblocks(n, T), T, 0, s>>>(
-        d_depth, d_hsv, gx, gy, keep, rank, totals + 1, W, H, fp.max_points, (float)fp.fx,
-        (float)fp.fy, (float)fp.cx, (float)fp.cy, (float)fp.grad_scale, out_xyz, out_feat, out_pix);
-    e = cudaGetLastError();
-  }
-  cudaFreeAsync(scratch, s);
-  if (e == cudaSuccess) e = cudaStreamSynchronize(s);
   if (e != cudaSuccess) return fail(ctx, CVO_ERR_CUDA, std::string("front end: ") + cudaGetErrorString(e));
   if (n_valid == 0) return fail(ctx, CVO_ERR_INVALID_ARG, "no pixel has a depth in range");
   *n_out = n_emit;
