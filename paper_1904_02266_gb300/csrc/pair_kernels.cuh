@@ -36,7 +36,7 @@
 // radius 10% wider than the cutoff and rebuilt when the grid level changes,
 // when the pose has drifted by more than that margin (an FP64 bound over the
 // whole source cloud), or when it has become much wider than needed. A warp
-// whose share of a reused plan fits its cache slots also lists, once per
+// whose share of a reused plan fits its cache also lists, once per
 // plan, the (candidate, source point) pairs of each cached cluster within the
 // plan radius, and its passes evaluate the lists instead of whole chunks.
 #pragma once
@@ -2041,21 +2041,31 @@ __device__ void pass_stream(const SolveCfg* cfg, SolveSmem<DPS, NU>& sm, int war
   }
 }
 
-// Shared-memory cache of a warp's share of the plan. A slot holds 32 points
-// (float4 xyz, then DP feature planes of 32 floats): either the raw centred
-// source points of a cluster (header kSlotCluster | cluster size) or the
-// candidates of a chunk of filtered candidates (header: number of valid
-// candidates | first source group << 6 | end source group << 10; the rest are
-// padding points beyond every cutoff). Filled once per plan when the warp's
-// whole share fits, so that the passes of every iteration that reuses the
-// plan (at the lengthscale floor, most of the solve) read no global memory.
-constexpr int kCacheSlots = 32;                 // header capacity per warp
+// Shared-memory cache of a warp's share of the plan (cap floats): chunk slots
+// from the front, each the 32 candidates of a chunk (float4 xyz, then DP
+// feature planes of 32 floats; padding points beyond every cutoff), and the raw
+// centred source points of the clusters from the back, each cluster just as
+// large as it is (float4 rows, then DP planes, of its size rounded up to 4: a
+// cluster of the floor holds 5.5 points of the room pair on average, and a
+// 32-point slot for each took about a third of the cache). The items follow in
+// order in cache_hdr: a cluster (kSlotCluster | its size), then its chunks
+// (number of valid candidates | first source group << 6 | end source group
+// << 10). Filled once per plan when the warp's whole share fits, so that the
+// passes of every iteration that reuses the plan (at the lengthscale floor, most
+// of the solve) read no global memory.
+constexpr int kCacheSlots = 32;                 // items per warp
 constexpr unsigned short kSlotCluster = 0x8000;
-constexpr unsigned short kSlotList = 0x4000;      // cluster slot whose pairs are listed
+constexpr unsigned short kSlotList = 0x4000;      // cluster whose pairs are listed
 
 template <int DP>
 __device__ __forceinline__ constexpr int slot_floats() {
   return 32 * (4 + DP);
+}
+
+// Floats a cluster of cs points takes in the cache.
+template <int DP>
+__device__ __forceinline__ int cluster_floats(int cs) {
+  return ((cs + 3) & ~3) * (4 + DP);
 }
 
 // Pair lists of a plan that will be reused (Verlet-style): for each cached
@@ -2066,12 +2076,12 @@ __device__ __forceinline__ constexpr int slot_floats() {
 // begin_iteration), so these pairs are a superset of the pairs within the
 // cutoff, and the passes evaluate only them (each with the exact cutoff test)
 // instead of every candidate against every source group. An entry is
-// candidate lane | slot << 5 | source point << 10; the lists live in the
+// candidate lane | chunk slot << 5 | source point << 10; the lists live in the
 // warp's shared scratch (list_max entries). A cluster whose list would not
 // fit keeps the chunk-by-chunk evaluation.
 template <int DP, int DPS, int NU>
 __device__ void build_lists(SolveSmem<DPS, NU>& sm, int warp, int lane, const float* base,
-                            int n) {
+                            int cap, int n) {
   unsigned short* pl = sm.ws[warp].list;
   constexpr int kCap = list_max<DPS>();
   const BlockCtx& b = sm.b;
@@ -2082,24 +2092,24 @@ __device__ void build_lists(SolveSmem<DPS, NU>& sm, int warp, int lane, const fl
   for (int i = 0; i < 3; ++i) T[i] = __double2float_rn(b.Tp[i]);
   const float rp2 = b.rplan_f * b.rplan_f;
   const unsigned lt = (1u << lane) - 1u;
-  int run = 0;
+  int run = 0, coff = cap, k = 0;
   for (int s = 0; s < n; ++s) {
     const unsigned h = sm.cache_hdr[warp][s];
-    if (!(h & kSlotCluster)) continue;
     const int cs = (int)(h & 0x3f);
-    const float4 p = reinterpret_cast<const float4*>(base + (size_t)s * slot_floats<DP>())[lane];
+    coff -= cluster_floats<DP>(cs);
+    const float4 p = reinterpret_cast<const float4*>(base + coff)[min(lane, cs - 1)];
     const float zx = fmaf(R[0], p.x, fmaf(R[1], p.y, fmaf(R[2], p.z, T[0])));
     const float zy = fmaf(R[3], p.x, fmaf(R[4], p.y, fmaf(R[5], p.z, T[1])));
     const float zz = fmaf(R[6], p.x, fmaf(R[7], p.y, fmaf(R[8], p.z, T[2])));
     const int start = run;
     bool fits = true;
     int t = s + 1;
-    for (; t < n && !(sm.cache_hdr[warp][t] & kSlotCluster); ++t) {
+    for (; t < n && !(sm.cache_hdr[warp][t] & kSlotCluster); ++t, ++k) {
       const unsigned hc = sm.cache_hdr[warp][t];
       const int cnt = (int)(hc & 0x3f);
       const int jlo = 4 * (int)((hc >> 6) & 0xf), jhi = min(cs, 4 * (int)((hc >> 10) & 0xf));
       const float4 xp =
-          reinterpret_cast<const float4*>(base + (size_t)t * slot_floats<DP>())[lane];
+          reinterpret_cast<const float4*>(base + (size_t)k * slot_floats<DP>())[lane];
       const bool valid = lane < cnt;
       for (int j = jlo; j < jhi && fits; ++j) {
         const float dx = xp.x - __shfl_sync(kFull, zx, j);
@@ -2110,7 +2120,7 @@ __device__ void build_lists(SolveSmem<DPS, NU>& sm, int warp, int lane, const fl
         if (run + __popc(m) > kCap) {
           fits = false;   // warp-uniform
         } else {
-          if (in) pl[run + __popc(m & lt)] = (unsigned short)(lane | (t << 5) | (j << 10));
+          if (in) pl[run + __popc(m & lt)] = (unsigned short)(lane | (k << 5) | (j << 10));
           run += __popc(m);
         }
       }
@@ -2127,41 +2137,44 @@ __device__ void build_lists(SolveSmem<DPS, NU>& sm, int warp, int lane, const fl
 
 template <int DP, int MODE, int DPS, int NU>
 __device__ void fill_cache(const SolveCfg* cfg, SolveSmem<DPS, NU>& sm, int warp, int lane,
-                           float* cache, int slots) {
+                           float* cache, int cap) {
   const BlockCtx& b = sm.b;
   const GridView& g = cfg->grids[b.level];
   const ClusterView& cv = cfg->clusters[b.level];
   const WarpRange r = warp_range(b, warp, 0);
   const float rp2 = b.rplan_f * b.rplan_f;
-  // count the slots the share needs (one in several pieces is too large for them)
-  int need = b.n_range > 1 ? kCacheSlots + 1 : 0;
+  // what the share needs (one in several pieces is too large for the cache)
+  int need = 0, items = b.n_range > 1 ? kCacheSlots + 1 : 0;
   for (int c = r.c0; c <= r.c1 && c < cv.ncl; ++c) {
     int jb, je;
-    if (range_chunks(r, c, (__ldcg(&cfg->cl_fcand[c]) + 31) >> 5, jb, je)) need += 2 + je - jb;
+    if (!range_chunks(r, c, (__ldcg(&cfg->cl_fcand[c]) + 31) >> 5, jb, je)) continue;
+    need += cluster_floats<DP>(cv.cstart[c + 1] - cv.cstart[c]) + (1 + je - jb) * slot_floats<DP>();
+    items += 2 + je - jb;
+    if (need > cap || items > kCacheSlots) break;
   }
-  if (need > min(slots, kCacheSlots)) {
+  if (need > cap || items > kCacheSlots) {
     if (lane == 0) sm.cache_n[warp] = -1;
     __syncwarp();
     return;
   }
-  float* base = cache + (size_t)warp * slots * slot_floats<DP>();
-  int n = 0;
+  float* base = cache + (size_t)warp * cap;
+  int n = 0, k = 0, coff = cap;   // items, chunk slots, where the clusters begin
   for (int c = r.c0; c <= r.c1 && c < cv.ncl; ++c) {
     const int tc = __ldcg(&cfg->cl_cand[c]);
     const int fc = __ldcg(&cfg->cl_fcand[c]);
     int jb, je;
     if (!range_chunks(r, c, (fc + 31) >> 5, jb, je)) continue;
     const int p0 = cv.cstart[c];
-    const int cs = cv.cstart[c + 1] - p0;
-    float* sl = base + (size_t)n * slot_floats<DP>();
-    float4 p = make_float4(0.f, 0.f, 0.f, 0.f);
-    if (lane < cs) p = cfg->src.xyz[p0 + lane];
-    reinterpret_cast<float4*>(sl)[lane] = p;
+    const int cs = cv.cstart[c + 1] - p0, cs4 = (cs + 3) & ~3;
+    coff -= cluster_floats<DP>(cs);
+    float* sl = base + coff;
+    if (lane < cs) {
+      reinterpret_cast<float4*>(sl)[lane] = cfg->src.xyz[p0 + lane];
 #pragma unroll
-    for (int d = 0; d < DP; ++d)
-      sl[128 + d * 32 + lane] =
-          lane < cs ? load_feat<bf16_of(MODE)>(cfg->src.feat, (size_t)d * cfg->src.m_pad + p0 + lane)
-                    : 0.f;
+      for (int d = 0; d < DP; ++d)
+        sl[(4 + d) * cs4 + lane] =
+            load_feat<bf16_of(MODE)>(cfg->src.feat, (size_t)d * cfg->src.m_pad + p0 + lane);
+    }
     if (lane == 0) {
       sm.cache_hdr[warp][n] = (unsigned short)(kSlotCluster | cs);
       sm.cache_cl[warp][n] = c;
@@ -2176,7 +2189,7 @@ __device__ void fill_cache(const SolveCfg* cfg, SolveSmem<DPS, NU>& sm, int warp
     }
     FCursor cur = fcursor_at<DPS, NU>(sm, warp, nseg, jb * 32);
     const int want = min(fc, 32 * (je + 1)) - 32 * jb;
-    float* s0 = base + (size_t)n * slot_floats<DP>();
+    float* s0 = base + (size_t)k * slot_floats<DP>();
     while (cur.made < want && cur.u < tc) {
       float xf[DPS];
       const float4 xp =
@@ -2205,11 +2218,12 @@ __device__ void fill_cache(const SolveCfg* cfg, SolveSmem<DPS, NU>& sm, int warp
       sm.cache_cl[warp][n + lane] = j;   // a chunk slot keeps its chunk index
     }
     n += nchk;
+    k += nchk;
     __syncwarp();   // the segment arrays are reused by the next cluster
   }
   if (lane == 0) sm.cache_n[warp] = (short)n;
   __syncwarp();
-  if (b.plan_filter) build_lists<DP, DPS, NU>(sm, warp, lane, base, n);
+  if (b.plan_filter) build_lists<DP, DPS, NU>(sm, warp, lane, base, cap, n);
 }
 
 // One entry of a cluster's pair list (build_lists) against the staged
@@ -2287,7 +2301,7 @@ __device__ __forceinline__ bool list_pair(SolveSmem<DPS, NU>& sm, int warp, cons
 // A listed cluster (staged): its nl pairs, 64 per round (two per lane, whose
 // chains overlap), the next round's entries loading while this one runs. In
 // the plan's first gradient pass (collect) the source groups of each chunk that
-// kept a pair are gathered per slot: lane t holds slot t's mask in act.
+// kept a pair are gathered per chunk slot: lane t holds slot t's mask in act.
 template <bool STEP, int DP, int MODE, int DPS, int NU>
 __device__ void list_pairs(SolveSmem<DPS, NU>& sm, int warp, int lane, const float* base,
                            const unsigned short* pl, int nl, float rc2, float A, float acc[7],
@@ -2325,35 +2339,37 @@ __device__ void list_pairs(SolveSmem<DPS, NU>& sm, int warp, int lane, const flo
 // The same share as pass_stream, from the warp's cache.
 template <bool STEP, int DP, int MODE, int DPS, int NU>
 __device__ void pass_cached(const SolveCfg* cfg, SolveSmem<DPS, NU>& sm, int warp, int lane,
-                            const float* cache, int slots, float acc[7], unsigned& nnz,
+                            const float* cache, int cap, float acc[7], unsigned& nnz,
                             unsigned& cand) {
   const float rc2 = sm.b.rc2, A = sm.b.A;
   const bool collect = !STEP && sm.b.collect_kept;
-  const float* base = cache + (size_t)warp * slots * slot_floats<DP>();
+  const float* base = cache + (size_t)warp * cap;
   const unsigned short* pl = sm.ws[warp].list;
   const int n = sm.cache_n[warp];
-  int cs = 0, cs4 = 0, cur = -1, loff = 0;
+  int cs = 0, cs4 = 0, cur = -1, loff = 0, k = 0, coff = cap;
   unsigned nnz0 = nnz;
   for (int s = 0; s < n; ++s) {
     const unsigned h = sm.cache_hdr[warp][s];
-    const float* sl = base + (size_t)s * slot_floats<DP>();
-    const float4 p = reinterpret_cast<const float4*>(sl)[lane];
-    float f[DPS];
-#pragma unroll
-    for (int d = 0; d < DPS; ++d) f[d] = d < DP ? sl[128 + d * 32 + lane] : 0.f;
     if (h & kSlotCluster) {
       if (collect) {
         add_kept(cfg, cur, nnz - nnz0, lane);
         nnz0 = nnz;
       }
       cur = sm.cache_cl[warp][s] & ((1 << kListShift) - 1);
-      __syncwarp();   // every lane is done with the previous cluster
       cs = (int)(h & 0x3f);
-      stage_cluster<STEP, DP, DPS, NU>(sm, warp, lane, lane < cs, p, f, (h & kSlotList) != 0);
       cs4 = (cs + 3) & ~3;
+      coff -= cluster_floats<DP>(cs);
+      const float* sl = base + coff;
+      const int i = min(lane, cs - 1);
+      const float4 p = reinterpret_cast<const float4*>(sl)[i];
+      float f[DPS];
+#pragma unroll
+      for (int d = 0; d < DPS; ++d) f[d] = d < DP ? sl[(4 + d) * cs4 + i] : 0.f;
+      __syncwarp();   // every lane is done with the previous cluster
+      stage_cluster<STEP, DP, DPS, NU>(sm, warp, lane, lane < cs, p, f, (h & kSlotList) != 0);
       __syncwarp();
       if (h & kSlotList) {
-        // the cluster's chunks through its pair list, then past its chunk slots
+        // the cluster's chunks through its pair list, then past its chunks
         int t = s + 1;
         while (t < n && !(sm.cache_hdr[warp][t] & kSlotCluster)) ++t;
         const int nl = (int)((unsigned)sm.cache_cl[warp][s] >> kListShift);
@@ -2361,16 +2377,24 @@ __device__ void pass_cached(const SolveCfg* cfg, SolveSmem<DPS, NU>& sm, int war
         list_pairs<STEP, DP, MODE, DPS, NU>(sm, warp, lane, base, pl + loff, nl, rc2, A, acc, nnz,
                                             cand, collect, act);
         loff += nl;
-        if (collect && lane > s && lane < t && act && cur >= 0) {
-          const int j = sm.cache_cl[warp][lane];
+        const int nk = t - s - 1;   // its chunk slots: k .. k + nk - 1, items s + 1 .. t - 1
+        if (collect && lane >= k && lane < k + nk && act && cur >= 0) {
+          const int j = sm.cache_cl[warp][s + 1 + lane - k];
           if (j < kActChunks) {
             atomicOr(&cfg->ch_act[(size_t)cur * kActChunks + j], act);
             atomicAdd(&cfg->cl_act[cur], __popc(act));
           }
         }
+        k += nk;
         s = t - 1;
       }
     } else {
+      const float* sl = base + (size_t)k * slot_floats<DP>();
+      const float4 p = reinterpret_cast<const float4*>(sl)[lane];
+      float f[DPS];
+#pragma unroll
+      for (int d = 0; d < DPS; ++d) f[d] = d < DP ? sl[128 + d * 32 + lane] : 0.f;
+      ++k;
       const int cnt = (int)(h & 0x3f);
       const int jlo = 4 * (int)((h >> 6) & 0xf), jhi = min(cs4, 4 * (int)((h >> 10) & 0xf));
       if (lane < cnt) cand += (unsigned)max(0, min(cs, jhi) - jlo);
@@ -2384,28 +2408,27 @@ __device__ void pass_cached(const SolveCfg* cfg, SolveSmem<DPS, NU>& sm, int war
 
 template <bool STEP, int DP, int MODE, int DPS, int NU>
 __device__ __forceinline__ void pass_warp(const SolveCfg* cfg, SolveSmem<DPS, NU>& sm, int warp,
-                                          int lane, float* cache, int slots, float acc[7],
+                                          int lane, float* cache, int cap, float acc[7],
                                           unsigned& nnz, unsigned& cand) {
   if (sm.cache_n[warp] >= 0)
-    pass_cached<STEP, DP, MODE, DPS, NU>(cfg, sm, warp, lane, cache, slots, acc, nnz, cand);
+    pass_cached<STEP, DP, MODE, DPS, NU>(cfg, sm, warp, lane, cache, cap, acc, nnz, cand);
   else
     for (int k = 0; k < sm.b.n_range; ++k)
       pass_stream<STEP, DP, MODE, DPS, NU>(cfg, sm, warp, lane, k,
-                                           cache + (size_t)warp * slots * slot_floats<DP>(), acc,
-                                           nnz, cand);
+                                           cache + (size_t)warp * cap, acc, nnz, cand);
 }
 
 // One pass over the block's warps, then the block partial (fixed order).
 template <bool STEP, int DP, int MODE, int DPS, int NU>
 __device__ void run_pass(const SolveCfg* cfg, SolveSmem<DPS, NU>& sm, double* partials,
-                         float* cache, int slots) {
+                         float* cache, int cap) {
   constexpr int NACC = STEP ? 5 : 7;
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   float acc[7];
 #pragma unroll
   for (int i = 0; i < 7; ++i) acc[i] = 0.f;
   unsigned nnz = 0, cand = 0;
-  pass_warp<STEP, DP, MODE, DPS, NU>(cfg, sm, warp, lane, cache, slots, acc, nnz, cand);
+  pass_warp<STEP, DP, MODE, DPS, NU>(cfg, sm, warp, lane, cache, cap, acc, nnz, cand);
   __syncwarp();
   if (STEP) {
     // the first warp done with its share forms the FP64 gradient (it reads
@@ -2475,7 +2498,7 @@ template <int DP, int MODE, int DPS, int NU>
 __device__ void solve_pair(const SolveCfg* __restrict__ cfg, SolveState* __restrict__ st,
                            double* __restrict__ partials, IterRecord* __restrict__ records,
                            Team team, SolveSmem<DPS, NU>& sm, bool join, float* cache,
-                           int slots) {
+                           int cap) {
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   unsigned gen = 0;
   double* part_g = partials;
@@ -2570,7 +2593,7 @@ __device__ void solve_pair(const SolveCfg* __restrict__ cfg, SolveState* __restr
       }
       if (!grid_sync(st, gen, &sm.flag, team.size, sm.b.tc.wait_polls)) break;
       split_work<DPS, NU>(cfg, sm, tid, team);
-      fill_cache<DP, MODE, DPS, NU>(cfg, sm, warp, lane, cache, slots);
+      fill_cache<DP, MODE, DPS, NU>(cfg, sm, warp, lane, cache, cap);
       if (tid == 0) {
         sm.b.need_plan = 0;
         sm.b.collect_kept = replan && (cfg->cost_kept > 0.f || sm.b.plan_filter);
@@ -2581,7 +2604,7 @@ __device__ void solve_pair(const SolveCfg* __restrict__ cfg, SolveState* __restr
     }
     if (stamp) t1 = globaltimer();
     // ---- gradient pass ----
-    run_pass<false, DP, MODE, DPS, NU>(cfg, sm, part_g, cache, slots);
+    run_pass<false, DP, MODE, DPS, NU>(cfg, sm, part_g, cache, cap);
     if (stamp) tg1 = globaltimer();
     if (!grid_sync_reduce(st, gen, sm, part_g, 9, team.size)) break;
     if (stamp) tg2 = globaltimer();
@@ -2592,7 +2615,7 @@ __device__ void solve_pair(const SolveCfg* __restrict__ cfg, SolveState* __restr
     __syncthreads();
     if (stamp) t2 = globaltimer();
     // ---- step pass ----
-    run_pass<true, DP, MODE, DPS, NU>(cfg, sm, part_s, cache, slots);
+    run_pass<true, DP, MODE, DPS, NU>(cfg, sm, part_s, cache, cap);
     if (stamp) ts1 = globaltimer();
     if (!grid_sync_reduce(st, gen, sm, part_s, 7, team.size)) break;
     if (stamp) ts2 = globaltimer();
@@ -2635,13 +2658,13 @@ __device__ void solve_pair(const SolveCfg* __restrict__ cfg, SolveState* __restr
 template <int DP, int MODE>
 __global__ void __launch_bounds__(kThreads, CVO_SOLVE_MIN_BLOCKS)
 solve_kernel(const SolveCfg* __restrict__ cfg, SolveState* __restrict__ st,
-             double* __restrict__ partials, IterRecord* __restrict__ records, int cache_slots) {
+             double* __restrict__ partials, IterRecord* __restrict__ records, int cache_cap) {
   constexpr int DPS = DP > 0 ? DP : 1;
   constexpr int NU = 2;
   __shared__ SolveSmem<DPS, NU> sm;
   extern __shared__ float4 dyn_smem[];
   solve_pair<DP, MODE, DPS, NU>(cfg, st, partials, records, Team{(int)blockIdx.x, (int)gridDim.x},
-                                sm, false, reinterpret_cast<float*>(dyn_smem), cache_slots);
+                                sm, false, reinterpret_cast<float*>(dyn_smem), cache_cap);
 }
 
 __device__ __forceinline__ unsigned long long ld_acquire_sys_u64(const unsigned long long* p) {
@@ -2737,7 +2760,7 @@ template <int DP, int MODE>
 __global__ void __launch_bounds__(kThreads, CVO_SOLVE_MIN_BLOCKS)
 queue_kernel(const QueueEntry* __restrict__ entries, const QueueCtl* __restrict__ ctl,
              unsigned long long* __restrict__ head, int* __restrict__ kstatus,
-             unsigned long long idle_limit_ns, int cache_slots) {
+             unsigned long long idle_limit_ns, int cache_cap) {
   constexpr int DPS = DP > 0 ? DP : 1;
   constexpr int NU = 2;
   __shared__ SolveSmem<DPS, NU> sm;
@@ -2755,7 +2778,7 @@ queue_kernel(const QueueEntry* __restrict__ entries, const QueueCtl* __restrict_
     const QueueEntry en = load_entry(entries + sm.q_entry);
     const Team team{(int)(sm.q_slot - en.slot0), en.team};
     solve_pair<DP, MODE, DPS, NU>(en.cfg, en.st, en.partials, nullptr, team, sm, true,
-                                  reinterpret_cast<float*>(dyn_smem), cache_slots);
+                                  reinterpret_cast<float*>(dyn_smem), cache_cap);
     if (threadIdx.x == 0) {
       __threadfence();
       const unsigned left = atomicAdd(&en.st->leave_count, 1u);
@@ -2770,9 +2793,9 @@ queue_kernel(const QueueEntry* __restrict__ entries, const QueueCtl* __restrict_
 
 // Dynamic shared memory of the plan cache: what CVO_SOLVE_MIN_BLOCKS blocks
 // per SM leave of the SM's shared memory after their static shared memory,
-// in whole warp shares of slots (set once per kernel instantiation).
+// in equal shares of whole 64 bytes per warp (set once per kernel instantiation).
 struct CacheCfg {
-  int bytes = 0, slots = 0;
+  int bytes = 0, cap = 0;   // cap: floats per warp
   cudaError_t err = cudaSuccess;
 };
 
@@ -2789,15 +2812,15 @@ const CacheCfg& cache_cfg() {
       c.err = cudaDeviceGetAttribute(&reserved, cudaDevAttrReservedSharedMemoryPerBlock, dev);
     if (c.err == cudaSuccess) c.err = cudaFuncGetAttributes(&fa, solve_kernel<DP, MODE>);
     if (c.err != cudaSuccess) return c;
-    const int slot_bytes = 4 * 32 * (4 + DP);
+    const int slot = 32 * (4 + DP);   // slot_floats
     const int avail = smem_sm / CVO_SOLVE_MIN_BLOCKS - reserved - (int)fa.sharedSizeBytes;
-    c.slots = std::max(0, std::min(kCacheSlots, avail / (kWarps * slot_bytes)));
-    // the streamed passes gather candidates through two slots of each warp
-    if (c.slots < 2) {
+    c.cap = std::max(0, std::min(kCacheSlots * slot, avail / kWarps / 64 * 16));
+    // the streamed passes gather candidates through 64 entries of each warp
+    if (c.cap < 2 * slot) {
       c.err = cudaErrorInvalidConfiguration;
       return c;
     }
-    c.bytes = c.slots * kWarps * slot_bytes;
+    c.bytes = c.cap * kWarps * (int)sizeof(float);
     if (c.bytes > 0) {
       c.err = cudaFuncSetAttribute(solve_kernel<DP, MODE>,
                                    cudaFuncAttributeMaxDynamicSharedMemorySize, c.bytes);
@@ -2815,8 +2838,8 @@ cudaError_t launch_solve_t(int nblocks, const SolveCfg* cfg, SolveState* st, dou
                            IterRecord* records, cudaStream_t s) {
   const CacheCfg& cc = cache_cfg<DP, MODE>();
   if (cc.err != cudaSuccess) return cc.err;
-  int slots = cc.slots;
-  void* args[] = {(void*)&cfg, (void*)&st, (void*)&partials, (void*)&records, (void*)&slots};
+  int cap = cc.cap;
+  void* args[] = {(void*)&cfg, (void*)&st, (void*)&partials, (void*)&records, (void*)&cap};
   return cudaLaunchCooperativeKernel((const void*)solve_kernel<DP, MODE>, dim3(nblocks),
                                      dim3(kThreads), args, (size_t)cc.bytes, s);
 }
@@ -2827,9 +2850,9 @@ cudaError_t launch_queue_t(int nblocks, const QueueEntry* entries, const QueueCt
                            cudaStream_t s) {
   const CacheCfg& cc = cache_cfg<DP, MODE>();
   if (cc.err != cudaSuccess) return cc.err;
-  int slots = cc.slots;
+  int cap = cc.cap;
   void* args[] = {(void*)&entries, (void*)&ctl,     (void*)&head,
-                  (void*)&kstatus, (void*)&idle_ns, (void*)&slots};
+                  (void*)&kstatus, (void*)&idle_ns, (void*)&cap};
   return cudaLaunchCooperativeKernel((const void*)queue_kernel<DP, MODE>, dim3(nblocks),
                                      dim3(kThreads), args, (size_t)cc.bytes, s);
 }
