@@ -72,14 +72,16 @@ constexpr int kCompactTeamMax = 32;
 #ifndef CVO_COST_ACTIVE
 #define CVO_COST_ACTIVE 12
 #endif
-// a warp's share of the work is cut into up to kMaxRanges pieces taken from
-// different parts of the cloud, one more for every kRangeWork pair-test units
-// of it (split_work)
-constexpr int kMaxRanges = 4;
-#ifndef CVO_RANGE_WORK
-#define CVO_RANGE_WORK 1500
-#endif
-constexpr int kRangeWork = CVO_RANGE_WORK;
+// a warp's share of the work is cut into pieces taken from different parts of the
+// cloud (split_work): one per kRangeWork pair-test units of it, at most
+// kMaxRanges, from kRangeFrom units on. Whole-GPU teams, 100k room pair: up to 4
+// pieces of 1500 units 46.9 ms, 8 of 1500 46.2, 8 of 700 45.4; at 20k points
+// (about 1000 units a warp) a second piece costs a cluster and two ends more than
+// it evens out. Teams of at most kCompactTeamMax blocks hold long shares already:
+// one piece (64-pair batch: 1 to 4 pieces 110.1, 110.9, 111.8, 113.4 ms)
+constexpr int kMaxRanges = 8;
+constexpr int kRangeWork = 700;
+constexpr int kRangeFrom = 2000;
 // work model: the pair bodies of a source group that kept a pair, in pair-test units
 constexpr int kCostActive = CVO_COST_ACTIVE;
 
@@ -231,6 +233,8 @@ struct BlockCtx {
   int n_range;
   int w_c0[kMaxRanges][kWarps], w_j0[kMaxRanges][kWarps], w_g0[kMaxRanges][kWarps];
   int w_c1[kMaxRanges][kWarps], w_j1[kMaxRanges][kWarps], w_g1[kMaxRanges][kWarps];
+  // where the streamed rest of a partly cached share begins (c < 0: there is none)
+  int rest_c[kWarps], rest_j[kWarps], rest_g[kWarps];
   double dR[9], V[9];     // tail scratch: exp map rotation and its V matrix
 };
 
@@ -1217,6 +1221,16 @@ union WarpScratch {
   unsigned short list[list_max<DPS>()];
 };
 
+// Per block: the work split.
+struct SplitScratch {
+  long long scan[kThreads];
+  long long wsum[kWarps];
+  // per end of a warp's range: its position in the work, and the group of
+  // clusters that holds it with the position where that group starts
+  long long at[2 * kWarps * kMaxRanges], base[2 * kWarps * kMaxRanges];
+  int group[2 * kWarps * kMaxRanges];
+};
+
 // Shared memory of the solve kernel.
 template <int DPS, int NU>
 struct SolveSmem {
@@ -1227,17 +1241,13 @@ struct SolveSmem {
   float zf[kWarps][DPS][kClusterMax];
   float4 u[kWarps][NU][kClusterMax];   // step vectors of a listed cluster's points (step_terms)
   float zw[kWarps][kClusterMax];       // step pass: -z_l . kw
-  WarpScratch<DPS> ws[kWarps];      // cell-row segments of the staged cluster, or the pair list
+  union {
+    WarpScratch<DPS> ws[kWarps];    // cell-row segments of the staged cluster, or the pair list
+    SplitScratch split;             // between the plan and the cache fill, when neither is live
+  };
   float red[kWarps][10];
-  double red_d[kWarps][16];
-  long long scan[kThreads];
-  long long wsum[kWarps];
-  long long bnd_base[2 * kWarps * kMaxRanges];   // per range end: its position in the work, then
-                                                 // (bnd_base) where the group holding it starts
-  long long bnd_at[2 * kWarps * kMaxRanges];
-  int bnd_group[2 * kWarps * kMaxRanges];
   double sums[10];
-  int flag, last;
+  int flag;
   long long q_slot;                 // queue: claimed slot (-1: none left)
   int q_entry;                      //        entry that slot belongs to
   short cache_n[kWarps];            // slots cached per warp (-1: streamed)
@@ -1358,7 +1368,7 @@ __device__ void locate(const SolveCfg* cfg, const ClusterView& cv, int group, lo
 // cloud, so a block whose warps take pieces from all over it ends its pass at
 // about the time the other blocks do, where one contiguous run of the work per
 // block left the slowest block 1.2 to 1.3 times the mean. Each further piece costs
-// its warp a cluster to stage and two ends to locate: one per kRangeWork units.
+// its warp a cluster to stage and two ends to locate.
 template <int DPS, int NU>
 __device__ void split_work(const SolveCfg* cfg, SolveSmem<DPS, NU>& sm, int tid, Team team) {
   const ClusterView& cv = cfg->clusters[sm.b.level];
@@ -1375,17 +1385,19 @@ __device__ void split_work(const SolveCfg* cfg, SolveSmem<DPS, NU>& sm, int tid,
     const long long v = __shfl_up_sync(kFull, incl, off);
     if (lane >= off) incl += v;
   }
-  if (lane == 31) sm.wsum[warp] = incl;
+  if (lane == 31) sm.split.wsum[warp] = incl;
   __syncthreads();
   long long TW = 0;
 #pragma unroll
   for (int w = 0; w < kWarps; ++w) {
-    if (w < warp) incl += sm.wsum[w];
-    TW += sm.wsum[w];
+    if (w < warp) incl += sm.split.wsum[w];
+    TW += sm.split.wsum[w];
   }
-  sm.scan[tid] = incl;
+  sm.split.scan[tid] = incl;
   const long long NW = (long long)team.size * kWarps;
-  const int nr = (int)min((long long)kMaxRanges, max(1ll, TW / (NW * kRangeWork)));
+  const int nr = team.size <= kCompactTeamMax || TW < NW * kRangeFrom
+                     ? 1
+                     : (int)min((long long)kMaxRanges, TW / (NW * kRangeWork));
   __syncthreads();
   // end h of the k-th piece of warp w on thread (k kWarps + w) 2 + h: the thread
   // whose run of groups holds it, by binary search, then the group
@@ -1398,10 +1410,10 @@ __device__ void split_work(const SolveCfg* cfg, SolveSmem<DPS, NU>& sm, int tid,
       int lo = 0, hi = kThreads - 1;   // the first thread whose inclusive sum is beyond `at`
       while (lo < hi) {
         const int mid = (lo + hi) >> 1;
-        if (sm.scan[mid] > at) hi = mid;
+        if (sm.split.scan[mid] > at) hi = mid;
         else lo = mid + 1;
       }
-      base = lo > 0 ? sm.scan[lo - 1] : 0;
+      base = lo > 0 ? sm.split.scan[lo - 1] : 0;
       const int ge = min(ng, (lo + 1) * per);
       for (int gi = lo * per; gi < ge; ++gi) {
         const long long w = __ldcg(&cfg->group_agg[gi]);
@@ -1412,9 +1424,9 @@ __device__ void split_work(const SolveCfg* cfg, SolveSmem<DPS, NU>& sm, int tid,
         base += w;
       }
     }
-    sm.bnd_group[tid] = group;
-    sm.bnd_base[tid] = base;
-    sm.bnd_at[tid] = at;
+    sm.split.group[tid] = group;
+    sm.split.base[tid] = base;
+    sm.split.at[tid] = at;
   }
   if (tid == 0) sm.b.n_range = nr;
   __syncthreads();
@@ -1423,8 +1435,8 @@ __device__ void split_work(const SolveCfg* cfg, SolveSmem<DPS, NU>& sm, int tid,
     for (int h = 0; h < 2; ++h) {
       const int q = 2 * (k * kWarps + warp) + h;
       int c = cv.ncl, jj = 0, gg = 0;   // past the end: no chunk
-      if (sm.bnd_group[q] >= 0)
-        locate(cfg, cv, sm.bnd_group[q], sm.bnd_base[q], sm.bnd_at[q], lane, &c, &jj, &gg,
+      if (sm.split.group[q] >= 0)
+        locate(cfg, cv, sm.split.group[q], sm.split.base[q], sm.split.at[q], lane, &c, &jj, &gg,
                sm.b.use_kept != 0, sm.b.use_act != 0);
       if (lane == 0) {
         if (h == 0) {
@@ -1866,13 +1878,13 @@ __device__ __forceinline__ int stage_from_global(const SolveCfg* cfg, SolveSmem<
 // current chunk runs.
 template <bool STEP, int DP, int MODE, int DPS, int NU>
 __device__ void pass_stream(const SolveCfg* cfg, SolveSmem<DPS, NU>& sm, int warp, int lane,
-                            int range, float* ring, float acc[7], unsigned& nnz, unsigned& cand) {
+                            WarpRange r, float* ring, float acc[7], unsigned& nnz,
+                            unsigned& cand) {
   const BlockCtx& b = sm.b;
   const GridView& g = cfg->grids[b.level];
   const ClusterView& cv = cfg->clusters[b.level];
   const float rc2 = b.rc2, A = b.A;
   const float rp2 = b.rplan_f * b.rplan_f;
-  const WarpRange r = warp_range(b, warp, range);
   const bool collect = !STEP && b.collect_kept;
   float4* rxyz = reinterpret_cast<float4*>(ring);
   float* rfeat = ring + 4 * 64;
@@ -2050,9 +2062,10 @@ __device__ void pass_stream(const SolveCfg* cfg, SolveSmem<DPS, NU>& sm, int war
 // 32-point slot for each took about a third of the cache). The items follow in
 // order in cache_hdr: a cluster (kSlotCluster | its size), then its chunks
 // (number of valid candidates | first source group << 6 | end source group
-// << 10). Filled once per plan when the warp's whole share fits, so that the
-// passes of every iteration that reuses the plan (at the lengthscale floor, most
-// of the solve) read no global memory.
+// << 10). Filled once per plan, so that the passes of every iteration that reuses
+// the plan (at the lengthscale floor, most of the solve) read no global memory. A
+// share of a reused plan that is too large is cached as far as it goes, with the
+// first two slots left to the streamed pass for the rest of it (BlockCtx::rest).
 constexpr int kCacheSlots = 32;                 // items per warp
 constexpr unsigned short kSlotCluster = 0x8000;
 constexpr unsigned short kSlotList = 0x4000;      // cluster whose pairs are listed
@@ -2152,20 +2165,37 @@ __device__ void fill_cache(const SolveCfg* cfg, SolveSmem<DPS, NU>& sm, int warp
     items += 2 + je - jb;
     if (need > cap || items > kCacheSlots) break;
   }
-  if (need > cap || items > kCacheSlots) {
+  const bool part = need > cap || items > kCacheSlots;
+  if (part && (b.n_range > 1 || !b.plan_filter)) {
     if (lane == 0) sm.cache_n[warp] = -1;
     __syncwarp();
     return;
   }
   float* base = cache + (size_t)warp * cap;
-  int n = 0, k = 0, coff = cap;   // items, chunk slots, where the clusters begin
-  for (int c = r.c0; c <= r.c1 && c < cv.ncl; ++c) {
+  if (part) base += 2 * slot_floats<DP>();
+  int room = part ? cap - 2 * slot_floats<DP>() : cap;
+  int n = 0, k = 0, coff = room;   // items, chunk slots, where the clusters begin
+  int rest_c = -1, rest_j = 0, rest_g = 0;
+  for (int c = r.c0; c <= r.c1 && c < cv.ncl && rest_c < 0; ++c) {
     const int tc = __ldcg(&cfg->cl_cand[c]);
     const int fc = __ldcg(&cfg->cl_fcand[c]);
     int jb, je;
     if (!range_chunks(r, c, (fc + 31) >> 5, jb, je)) continue;
     const int p0 = cv.cstart[c];
     const int cs = cv.cstart[c + 1] - p0, cs4 = (cs + 3) & ~3;
+    room -= cluster_floats<DP>(cs);
+    if (part) {
+      // the chunks of this cluster that still fit; the rest is streamed
+      const int fit = min(kCacheSlots - n - 1, room < 0 ? 0 : room / slot_floats<DP>());
+      if (1 + je - jb > fit) {
+        rest_c = c;
+        rest_j = jb + max(fit, 0);
+        rest_g = c == r.c0 && rest_j == r.j0 ? r.g0 : 0;
+        je = rest_j - 1;
+        if (je < jb) break;
+      }
+    }
+    room -= (1 + je - jb) * slot_floats<DP>();
     coff -= cluster_floats<DP>(cs);
     float* sl = base + coff;
     if (lane < cs) {
@@ -2221,9 +2251,15 @@ __device__ void fill_cache(const SolveCfg* cfg, SolveSmem<DPS, NU>& sm, int warp
     k += nchk;
     __syncwarp();   // the segment arrays are reused by the next cluster
   }
-  if (lane == 0) sm.cache_n[warp] = (short)n;
+  if (lane == 0) {
+    sm.cache_n[warp] = (short)n;
+    sm.b.rest_c[warp] = rest_c;
+    sm.b.rest_j[warp] = rest_j;
+    sm.b.rest_g[warp] = rest_g;
+  }
   __syncwarp();
-  if (b.plan_filter) build_lists<DP, DPS, NU>(sm, warp, lane, base, cap, n);
+  // (the segments of a streamed rest take the place of the lists)
+  if (b.plan_filter && !part) build_lists<DP, DPS, NU>(sm, warp, lane, base, cap, n);
 }
 
 // One entry of a cluster's pair list (build_lists) against the staged
@@ -2344,6 +2380,10 @@ __device__ void pass_cached(const SolveCfg* cfg, SolveSmem<DPS, NU>& sm, int war
   const float rc2 = sm.b.rc2, A = sm.b.A;
   const bool collect = !STEP && sm.b.collect_kept;
   const float* base = cache + (size_t)warp * cap;
+  if (sm.b.rest_c[warp] >= 0) {   // the streamed rest has the first two slots
+    base += 2 * slot_floats<DP>();
+    cap -= 2 * slot_floats<DP>();
+  }
   const unsigned short* pl = sm.ws[warp].list;
   const int n = sm.cache_n[warp];
   int cs = 0, cs4 = 0, cur = -1, loff = 0, k = 0, coff = cap;
@@ -2410,12 +2450,21 @@ template <bool STEP, int DP, int MODE, int DPS, int NU>
 __device__ __forceinline__ void pass_warp(const SolveCfg* cfg, SolveSmem<DPS, NU>& sm, int warp,
                                           int lane, float* cache, int cap, float acc[7],
                                           unsigned& nnz, unsigned& cand) {
-  if (sm.cache_n[warp] >= 0)
+  const BlockCtx& b = sm.b;
+  int streamed = b.n_range;
+  WarpRange r = warp_range(b, warp, 0);
+  if (sm.cache_n[warp] >= 0) {
     pass_cached<STEP, DP, MODE, DPS, NU>(cfg, sm, warp, lane, cache, cap, acc, nnz, cand);
-  else
-    for (int k = 0; k < sm.b.n_range; ++k)
-      pass_stream<STEP, DP, MODE, DPS, NU>(cfg, sm, warp, lane, k,
-                                           cache + (size_t)warp * cap, acc, nnz, cand);
+    streamed = b.rest_c[warp] >= 0 ? 1 : 0;
+    r.c0 = b.rest_c[warp];
+    r.j0 = b.rest_j[warp];
+    r.g0 = b.rest_g[warp];
+  }
+  for (int k = 0; k < streamed; ++k) {
+    if (k > 0) r = warp_range(b, warp, k);
+    pass_stream<STEP, DP, MODE, DPS, NU>(cfg, sm, warp, lane, r, cache + (size_t)warp * cap, acc,
+                                         nnz, cand);
+  }
 }
 
 // One pass over the block's warps, then the block partial (fixed order).
