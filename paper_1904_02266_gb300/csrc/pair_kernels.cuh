@@ -879,61 +879,110 @@ __device__ bool grid_sync(SolveState* st, unsigned& gen, int* s_flag, int nblk, 
   return *s_flag != 0;
 }
 
-// Fixed-order FP64 sum of the nblk block partials (nvals <= 10 values each,
-// value-major; the last two are counts, held as 64-bit integers in the
-// doubles' bits), by one block. Warp w < nvals - 2 sums value w, one
-// contiguous run of nblk doubles: lane l adds the value of blocks l, l + 32,
-// l + 64, ... in sequence (its loads issued first), then the 32 lane
-// sums are added along a fixed shuffle tree, so every FP64 instruction has all
-// its lanes busy (on GB300 an FP64 instruction costs the same with one lane or
-// 32). The last warp adds the two counts as integers. Results land in out[] (shared).
-// Every thread of the block calls it.
-template <class Smem>
-__device__ void reduce_partials(const double* partials, int nvals, double* out, int nblk,
-                                Smem& sm) {
-  static_assert(kWarps >= 8, "seven FP values and the counts need eight warps");
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  constexpr int kMaxPer = 16;   // nblk <= 512 blocks: 16 per lane
-  const int nf = nvals - 2;     // FP64 values; nf <= 7
-  if (warp < nf) {
-    const int i = warp;
-    const bool f32 = sm.b.tc.reduce_fp32 != 0;
-    double v[kMaxPer];
+// Sum over a warp of 64-bit integers of magnitude below 2^62 / 32: three 32-bit
+// reductions of its parts (26 + 26 low bits, the signed rest).
+__device__ __forceinline__ long long warp_sum_i64(long long v) {
+  const unsigned lo = __reduce_add_sync(kFull, (unsigned)v & 0x3ffffffu);
+  const unsigned mid = __reduce_add_sync(kFull, (unsigned)(v >> 26) & 0x3ffffffu);
+  const int hi = __reduce_add_sync(kFull, (int)(v >> 52));
+  return ((long long)hi << 52) + ((long long)mid << 26) + (long long)lo;
+}
+
+// The sum of the nblk values at p (one warp, every lane gets it): exact up to a
+// truncation of each value 52 bits below the largest, no less than FP64
+// additions keep (theirs round at the size of the running sum). The mantissas are
+// aligned to the largest exponent and added as integers, in any order with the
+// same result: on GB300 an FP64 instruction holds its scheduler's FP64 pipe for
+// about 64 cycles, and the ten dependent additions per value (two values to a
+// scheduler) were half of the reduction. Values out of the range in which the
+// aligned sum is a normal number, infinities and NaNs take FP64 additions.
+template <int PER>
+__device__ __forceinline__ double sum_partials(const double* p, int nblk, int lane) {
+  double v[PER];
 #pragma unroll
-    for (int k = 0; k < kMaxPer; ++k) {
-      const int blk = lane + 32 * k;
-      v[k] = blk < nblk ? __ldcg(&partials[(size_t)i * nblk + blk]) : 0.0;
-    }
+  for (int k = 0; k < PER; ++k) {
+    const int blk = lane + 32 * k;
+    v[k] = blk < nblk ? __ldcg(&p[blk]) : 0.0;
+  }
+  unsigned e_max = 0u;
+#pragma unroll
+  for (int k = 0; k < PER; ++k)
+    e_max = max(e_max, ((unsigned)__double2hiint(v[k]) >> 20) & 0x7ffu);
+  e_max = __reduce_max_sync(kFull, e_max);
+  if (e_max == 0u) return 0.0;   // zeros (a subnormal is no sum of FP32 products)
+  if (e_max < 100u || e_max > 2000u) {
     double acc = 0.0;
-    float accf = 0.f;
 #pragma unroll
-    for (int k = 0; k < kMaxPer; ++k) {
-      if (32 * k >= nblk) break;
-      if (f32) accf += (float)v[k];
-      else acc += v[k];
-    }
-    if (f32) {
+    for (int k = 0; k < PER; ++k) acc += v[k];
+#pragma unroll
+    for (int off = 16; off > 0; off >>= 1) acc += __shfl_xor_sync(kFull, acc, off);
+    return acc;
+  }
+  long long acc = 0;
+#pragma unroll
+  for (int k = 0; k < PER; ++k) {
+    const long long bits = __double_as_longlong(v[k]);
+    const unsigned e = (unsigned)(bits >> 52) & 0x7ffu;
+    const unsigned shift = min(e_max - e, 63u);
+    // 53-bit mantissa, aligned; 512 of them stay below 2^62
+    const long long m = ((bits & 0xfffffffffffffll) | 0x10000000000000ll) >> shift;
+    acc += e == 0u ? 0ll : bits < 0 ? -m : m;
+  }
+  acc = warp_sum_i64(acc);
+  if (acc == 0) return 0.0;
+  // acc 2^(e_max - 1075): the conversion, then the exponent field
+  const double d = (double)acc;
+  return __hiloint2double(__double2hiint(d) + (((int)e_max - 1075) << 20), __double2loint(d));
+}
+
+// Fixed-order sum of the nblk block partials (nvals <= 9 values each,
+// value-major; the last two are counts, held as 64-bit integers in the
+// doubles' bits), by one block: warp w < nvals - 2 sums value w, one contiguous
+// run of nblk doubles, lane l those of blocks l, l + 32, ... (all loads issued
+// first); the last two warps add a count each. Results land in out[] (shared).
+// Every thread of the block calls it.
+template <int PER, class Smem>
+__device__ void reduce_partials_of(const double* partials, int nvals, double* out, int nblk,
+                                   Smem& sm) {
+  static_assert(kWarps >= 9, "seven FP values and the two counts need nine warps");
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const int nf = nvals - 2;     // FP values; nf <= 7
+  if (warp < nf) {
+    const double* p = partials + (size_t)warp * nblk;
+    double acc;
+    if (sm.b.tc.reduce_fp32 != 0) {
+      float accf = 0.f;
+      for (int blk = lane; blk < nblk; blk += 32) accf += (float)__ldcg(&p[blk]);
 #pragma unroll
       for (int off = 16; off > 0; off >>= 1) accf += __shfl_xor_sync(kFull, accf, off);
       acc = (double)accf;
     } else {
-#pragma unroll
-      for (int off = 16; off > 0; off >>= 1) acc += __shfl_xor_sync(kFull, acc, off);
+      acc = sum_partials<PER>(p, nblk, lane);
     }
-    if (lane == 0) out[i] = acc;
-  } else if (warp == kWarps - 1) {
+    if (lane == 0) out[warp] = acc;
+  } else if (warp >= kWarps - 2) {
+    const int c = warp - (kWarps - 2);
+    const double* p = partials + (size_t)(nf + c) * nblk;
+    unsigned long long v[PER], n = 0;
 #pragma unroll
-    for (int c = 0; c < 2; ++c) {
-      unsigned long long n = 0;
-      for (int blk = lane; blk < nblk; blk += 32)
-        n += (unsigned long long)__double_as_longlong(
-            __ldcg(&partials[(size_t)(nf + c) * nblk + blk]));
-#pragma unroll
-      for (int off = 16; off > 0; off >>= 1) n += __shfl_xor_sync(kFull, n, off);
-      if (lane == 0) out[nf + c] = __longlong_as_double((long long)n);
+    for (int k = 0; k < PER; ++k) {
+      const int blk = lane + 32 * k;
+      v[k] = blk < nblk ? (unsigned long long)__double_as_longlong(__ldcg(&p[blk])) : 0ull;
     }
+#pragma unroll
+    for (int k = 0; k < PER; ++k) n += v[k];
+    // counts stay below n m = 2^44 over the team
+    n = (unsigned long long)warp_sum_i64((long long)n);
+    if (lane == 0) out[nf + c] = __longlong_as_double((long long)n);
   }
   __syncthreads();
+}
+
+template <class Smem>
+__device__ __forceinline__ void reduce_partials(const double* partials, int nvals, double* out,
+                                                int nblk, Smem& sm) {
+  if (nblk <= 160) reduce_partials_of<5>(partials, nvals, out, nblk, sm);
+  else reduce_partials_of<16>(partials, nvals, out, nblk, sm);   // nblk <= 512
 }
 
 // Barrier that also reduces the pass: every block adds its arrival (a release
