@@ -194,13 +194,13 @@ struct TailConst {
   int reduce_fp32;   // precision study: block and cross-block sums in FP32
   unsigned wait_polls;                 // barrier polls before a block gives up
   unsigned long long join_limit_ns;    // longest wait of a queued team's join
-  float cXf[3], inv_a2f, inv_b2f, src_radius_f;   // FP32 copies for the FP32 parts of the tail
+  // FP32 copies for the FP32 parts of the tail
+  float cXf[3], inv_a2f, inv_b2f, src_radius_f, eps_pose_f;
 };
 
 struct BlockCtx {
   TailConst tc;
   double P[16];           // current pose
-  double Rp[9], Tp[3];    // centred pose at the last plan
   double xi[6];           // metric gradient (Eq. metric)
   double x0[6];           // its components before the metric factors (FP64 pair sums, centring
                           // back-map applied)
@@ -211,8 +211,6 @@ struct BlockCtx {
   double kf_rot, kf_tr;   // this iteration's metric factors
   int small_grad;         // |xi| below the gradient threshold (or zero): no step, stop test
   int at_floor;           // this iteration's ell is the schedule's floor
-  int fin;                // step pass: warps done with their share (the first does the FP64
-                          // gradient)
   double t, t_prev;
   double ell, inv_l2, r_plan, plan_ell;
   int k, level, plan_level, plan_filter;
@@ -223,7 +221,13 @@ struct BlockCtx {
   int team_rank, team_size;                // this block's place in its team (read after a pass
                                            // from shared memory rather than kept in registers)
   unsigned long long nnz_total, cand_total, nnz_grad, cand_grad;
-  float R[9], T[3];       // FP32 centred pose: z~' = R z' + T
+  float R[9], T[3];       // FP32 centred pose of the passes: z~' = R z' + T'
+  float Rq[9], Tq[3];     // the same at the last plan
+  // the centred FP64 pose in two FP32 parts (rounded, and what the rounding
+  // left), for the FP32 step (quick_step)
+  float Rb[9], Tb[3], Rl[9], Tl[3];
+  int pending;            // P waits for the step of length pend_tau (refined in FP64) along u64
+  float pend_tau;
   float om[3], vc[3];     // unit step direction (centred frame)
   float kw[3];            // (omega . v) omega / 6 l^2
   float c_del, c_eps, k_eps;   // -|omega|^2 / 3, -|omega|^2 / 12, -(omega . v)^2 / 48 l^2
@@ -301,16 +305,37 @@ __device__ __forceinline__ bool is_pos(double x) {
   return hi != 0 || lo != 0u;
 }
 
-// Iteration k's constants (ic = the host table's entry k), the FP32 pose, and
-// whether the traversal plan must be rebuilt. Warp 0, every lane.
-__device__ __noinline__ void begin_iteration(const IterConst& ic, BlockCtx& b, int lane) {
-  // centred pose [R T'] on lanes 0..11, element (r, c) = (l / 4, l % 4):
-  // R = the pose's rotation, T' = R cZ + T - cX
+// The centred pose [R T'] of the FP64 pose in two FP32 parts, rounded to nearest,
+// on lanes 0..11, element (r, c) = (l / 4, l % 4): R = the pose's rotation, T' = R cZ
+// + T - cX. One warp.
+__device__ __forceinline__ void split_pose(BlockCtx& b, int lane, float* hi_out) {
   const int l = min(lane, 11), r = l >> 2, c = l & 3;
   const double t3 = fma(b.P[4 * r + 2], b.tc.cZ[2],
                         fma(b.P[4 * r + 1], b.tc.cZ[1],
                             fma(b.P[4 * r], b.tc.cZ[0], b.P[4 * r + 3] - b.tc.cX[r])));
   const double v = c == 3 ? t3 : b.P[4 * r + c];
+  const float hi = __double2float_rn(v);
+  const float lo = f64_to_f32(v - f32_to_f64(hi));
+  if (lane < 12) {
+    if (c < 3) {
+      b.Rb[3 * r + c] = hi;
+      b.Rl[3 * r + c] = lo;
+    } else {
+      b.Tb[r] = hi;
+      b.Tl[r] = lo;
+    }
+  }
+  *hi_out = hi;
+}
+
+// Iteration k's constants (ic = the host table's entry k), the FP32 pose (from
+// the FP64 pose, unless quick_step has formed it), and whether the traversal plan
+// must be rebuilt. Warp 0, every lane.
+__device__ __noinline__ void begin_iteration(const IterConst& ic, BlockCtx& b, int lane) {
+  const int l = min(lane, 11), r = l >> 2, c = l & 3;
+  float v;
+  if (b.pending) v = c == 3 ? b.T[r] : b.R[3 * r + c];
+  else split_pose(b, lane, &v);
   // is the current plan still a superset of the pairs within the cutoff?
   const float need = ic.rprune;   // 1.001 r_c
   // reuse only at an unchanged lengthscale (the floor of the schedule): while
@@ -318,9 +343,9 @@ __device__ __noinline__ void begin_iteration(const IterConst& ic, BlockCtx& b, i
   bool replan = b.need_plan || ic.level != b.plan_level ||
                 __double_as_longlong(ic.ell) != __double_as_longlong(b.plan_ell);
   if (!replan) {
-    // the differences in FP64, the rest in FP32: the 2e-5 relative and
-    // 1e-6 r_c margins below cover its rounding
-    const float d = f64_to_f32(v - (c == 3 ? b.Tp[r] : b.Rp[3 * r + c]));
+    // between the FP32 poses that the plan and the passes use; the 2e-5 relative
+    // and 1e-6 r_c margins below cover the rounding
+    const float d = v - (c == 3 ? b.Tq[r] : b.Rq[3 * r + c]);
     const float sq = lane < 12 ? d * d : 0.0f;
     float sr = c < 3 ? sq : 0.0f, st = c == 3 ? sq : 0.0f;
 #pragma unroll
@@ -335,14 +360,13 @@ __device__ __noinline__ void begin_iteration(const IterConst& ic, BlockCtx& b, i
     const float rp = b.rplan_f;
     replan = (need + drift > rp) || (rp > (float)kLoose * (need + drift));
   }
-  __syncwarp();   // every lane has read the old plan pose
+  __syncwarp();   // every lane has read the old poses
   if (lane < 12) {
-    // rounded to nearest: the passes' pose
-    if (c < 3) b.R[3 * r + c] = __double2float_rn(v);
-    else b.T[r] = __double2float_rn(v);
+    if (c < 3) b.R[3 * r + c] = v;
+    else b.T[r] = v;
     if (replan) {
-      if (c < 3) b.Rp[3 * r + c] = v;
-      else b.Tp[r] = v;
+      if (c < 3) b.Rq[3 * r + c] = v;
+      else b.Tq[r] = v;
     }
   }
   if (lane == 0) {
@@ -408,20 +432,12 @@ __device__ __forceinline__ double sqrt64(double x) {
 // acos / cos, no FP64 transcendentals), or the bracket's midpoint: a close
 // start takes two steps; a far one (the FP32 form loses the small roots of a
 // cubic whose roots differ by orders of magnitude) a few more.
-__device__ bool first_maximiser(double c0, double c1, double c2, double c3, double* t_out) {
-  // the largest exponent field among the coefficients (integer work: FP64
-  // instructions are the scarce resource here)
-  const int e_max = max(max((__double2hiint(c0) >> 20) & 0x7ff, (__double2hiint(c1) >> 20) & 0x7ff),
-                        max((__double2hiint(c2) >> 20) & 0x7ff, (__double2hiint(c3) >> 20) & 0x7ff));
-  if (e_max == 0x7ff) return false;   // an infinity or a NaN
-  // start: a root of the cubic from the closed form, all in FP32 on the
-  // coefficients scaled by 2^(1022 - e_max) (the largest has magnitude in
-  // [0.5, 1); formed from the bit patterns, truncated: a start needs no
-  // more), refined by two FP32 Newton steps; a negligible cubic term is left
-  // out of the start only
-  const int shift = 1022 - e_max;
-  const float f0 = f64_to_f32_shift(c0, shift), f1 = f64_to_f32_shift(c1, shift);
-  const float f2 = f64_to_f32_shift(c2, shift), f3 = f64_to_f32_shift(c3, shift);
+//
+// The start: a root of the cubic from the closed form, all in FP32 (f0..f3: the
+// coefficients scaled so that the largest has magnitude in [0.5, 1); truncated:
+// a start needs no more), refined by two FP32 Newton steps; a negligible cubic
+// term is left out of the start only. Not positive if there is none.
+__device__ __forceinline__ float cubic_start(float f0, float f1, float f2, float f3) {
   float ts = -1.0f;
   if (fabsf(f3) <= 1e-12f) {
     if (fabsf(f2) <= 1e-12f) {
@@ -468,15 +484,37 @@ __device__ bool first_maximiser(double c0, double c1, double c2, double c3, doub
     const float tn = ts - ff / fd;
     if (fd < 0.0f && tn > 0.0f && isfinite(tn)) ts = tn;
   }
+  return ts;
+}
+
+// G' falls over all of [0, t]: G''(t) < 0 and the vertex test of a concave G'' in
+// FP32 with a 1e-4 relative margin (their rounding is below 1e-6); G''(0) = c1 < 0
+// is the caller's. Then t, if a root, is the first one and a + -> - crossing.
+__device__ __forceinline__ bool falls_to(float f1, float f2, float f3, float ts, float* g2_out) {
+  const float g2 = fmaf(fmaf(3.0f * f3, ts, 2.0f * f2), ts, f1);
+  const float gmag = fabsf(f1) + fabsf(2.0f * f2 * ts) + fabsf(3.0f * f3 * ts * ts);
+  const bool inside = f3 < 0.0f && f2 > 0.0f && f2 < -3.0f * f3 * ts * (1.0f + 1e-4f);
+  const bool vertex_ok = !inside || 3.0f * f1 * f3 > f2 * f2 * (1.0f + 1e-4f);
+  *g2_out = g2;
+  return g2 < -1e-4f * gmag && vertex_ok;
+}
+
+__device__ bool first_maximiser(double c0, double c1, double c2, double c3, double* t_out) {
+  // the largest exponent field among the coefficients (integer work: FP64
+  // instructions are the scarce resource here)
+  const int e_max = max(max((__double2hiint(c0) >> 20) & 0x7ff, (__double2hiint(c1) >> 20) & 0x7ff),
+                        max((__double2hiint(c2) >> 20) & 0x7ff, (__double2hiint(c3) >> 20) & 0x7ff));
+  if (e_max == 0x7ff) return false;   // an infinity or a NaN
+  const int shift = 1022 - e_max;
+  const float f0 = f64_to_f32_shift(c0, shift), f1 = f64_to_f32_shift(c1, shift);
+  const float f2 = f64_to_f32_shift(c2, shift), f3 = f64_to_f32_shift(c3, shift);
+  const float ts = cubic_start(f0, f1, f2, f3);
   const double t32 = f32_to_f64(ts);
   // fast path: one FP64 Newton step from that start on the unscaled
   // coefficients (the roots do not depend on a common scale), accepted when it
-  // moves t by at most 2^-20 t (the step squares the start's error) and
-  // G'' < 0 on [0, t] (then G' falls from c0 > 0 over [0, t], so t is its
-  // first root and a + -> - crossing). G''(0) = c1 < 0 is read from the sign
-  // bit; G''(t) < 0 and the vertex test of a concave G'' are evaluated in FP32
-  // on the scaled coefficients with a 1e-4 relative margin (their rounding is
-  // below 1e-6), and anything within the margin goes to the bracketed search.
+  // moves t by at most 2^-20 t (the step squares the start's error) and G' falls
+  // from c0 > 0 over [0, t]; anything within the margins goes to the bracketed
+  // search
   if (e_max >= 2 && ts > 0.0f && isfinite(ts) && __double2hiint(c1) < 0) {
     const double f = fma(fma(fma(c3, t32, c2), t32, c1), t32, c0);
     const double fp = fma(fma(3.0 * c3, t32, mul_pow2(c2, 1)), t32, c1);
@@ -490,11 +528,8 @@ __device__ bool first_maximiser(double c0, double c1, double c2, double c3, doub
       const int ht = __double2hiint(t), hd = __double2hiint(dt);
       const int et = (ht >> 20) & 0x7ff, ed = (hd >> 20) & 0x7ff;
       const bool settled = ed <= et - 21;   // |dt| < 2^-20 t (dt = 0 has ed = 0)
-      const float g2 = fmaf(fmaf(3.0f * f3, ts, 2.0f * f2), ts, f1);
-      const float gmag = fabsf(f1) + fabsf(2.0f * f2 * ts) + fabsf(3.0f * f3 * ts * ts);
-      const bool inside = f3 < 0.0f && f2 > 0.0f && f2 < -3.0f * f3 * ts * (1.0f + 1e-4f);
-      const bool vertex_ok = !inside || 3.0f * f1 * f3 > f2 * f2 * (1.0f + 1e-4f);
-      if (ht > 0 && et < 0x7ff && settled && g2 < -1e-4f * gmag && vertex_ok) {
+      float g2;
+      if (ht > 0 && et < 0x7ff && settled && falls_to(f1, f2, f3, ts, &g2)) {
         *t_out = t;
         return true;
       }
@@ -629,7 +664,8 @@ __constant__ double kExpSeries[3][7] = {
 // the metric factors, x0 = omega' + cX x v (rotation) or v (translation), in
 // FP64 (the centring back-map may cancel); the common factor sigma^2 / ell^2
 // drops out of the direction, so only 1/a^2 and 1/b^2 are applied. The FP64
-// gradient itself (gradient_fp64) is formed during the step pass.
+// gradient itself (gradient_fp64) is formed while the block waits at the step
+// pass's barrier.
 __device__ void gradient_direction(BlockCtx& b, const double* sums, int lane) {
   const TailConst& tc = b.tc;
   const int a = lane % 3, a1 = a == 2 ? 0 : a + 1, a2 = a == 0 ? 2 : a - 1;
@@ -667,13 +703,12 @@ __device__ void gradient_direction(BlockCtx& b, const double* sums, int lane) {
     b.c_del = -ww * (1.0f / 3.0f);
     b.c_eps = -ww * (1.0f / 12.0f);
     b.k_eps = -wv * wv * b.inv_l2f * (1.0f / 48.0f);
-    b.fin = 0;
   }
   __syncwarp();
 }
 
-// Gradient tail, second part (one warp, during the step pass; it writes only
-// fields the pass does not read): the metric gradient xi (Eq. metric), |xi|,
+// Gradient tail, second part (one warp, while the block waits at the step pass's
+// barrier): the metric gradient xi (Eq. metric), |xi|,
 // xi / |xi| in FP64, F and the gradient pass's counts.
 __device__ void gradient_fp64(BlockCtx& b, const double* sums, int lane) {
   const TailConst& tc = b.tc;
@@ -720,51 +755,8 @@ __device__ __forceinline__ void form_step_sums(BlockCtx& b) {
   }
 }
 
-// Step tail: step length, pose update P <- exp(t xi) P, stop test. Warp 0.
-// The step length is found in tau = |xi| t, the step along xi / |xi|: G'(t) =
-// sum_m m S_m t^(m-1) = sigma^2 |xi| sum_m m s_m tau^(m-1), so the quartic of
-// the pass's own sums has the same roots in tau (no powers of |xi| needed),
-// and the twist is tau (xi / |xi|).
-__device__ void finish_step(BlockCtx& b, const double* sums, int lane) {
-  const TailConst& tc = b.tc;
-  if (lane < 5) b.s_raw[lane] = sums[lane];
-  if (lane == 0) {
-    b.nnz_total += b.nnz_grad + (unsigned long long)__double_as_longlong(sums[5]);
-    b.cand_total += b.cand_grad + (unsigned long long)__double_as_longlong(sums[6]);
-  }
-  if (tc.mode == kModeEval) {
-    __syncwarp();
-    if (lane == 0) {
-      form_step_sums(b);
-      b.done = 1;
-    }
-    __syncwarp();
-    return;
-  }
-  // the step length (the same scalar work on every lane)
-  double tau;
-  int no_ascent = 0, fallback = 0;
-  // no step along a gradient below the stop test's threshold (at rounding
-  // level S1 can still be positive, and the quartic's root is then arbitrary);
-  // S1 > 0 exactly when s1 > 0
-  if (b.small_grad || !is_pos(sums[1])) {
-    tau = 0.0;
-    no_ascent = 1;
-  } else {
-    bool ok;
-    if (tc.step_order == 2) {
-      ok = sums[2] < 0.0;
-      tau = ok ? -sums[1] / mul_pow2(sums[2], 1) : 0.0;
-    } else {
-      ok = first_maximiser(sums[1], mul_pow2(sums[2], 1), 3.0 * sums[3], mul_pow2(sums[4], 2),
-                           &tau);
-    }
-    if (!ok) {
-      fallback = 1;
-      // half the previous step, or 1e-3 / |xi| on the first one (tau = 1e-3)
-      tau = b.have_t_prev ? 0.5 * b.t_prev * b.xi_norm : 1e-3;
-    }
-  }
+// P <- exp(tau xi / |xi|) P in FP64 (Eqs. newstep, step), one warp.
+__device__ void apply_step(BlockCtx& b, double tau, int lane) {
   // twist tau xi / |xi|: rotation phi (lanes 0..2), translation rho (lanes 3..5)
   const double tw = tau * b.u64[min(lane, 5)];
   const double p0 = __shfl_sync(kFull, tw, 0), p1 = __shfl_sync(kFull, tw, 1);
@@ -815,12 +807,161 @@ __device__ void finish_step(BlockCtx& b, const double* sums, int lane) {
   __syncwarp();   // every lane has read the old pose
   if (lane < 12) b.P[lane] = pn;
   if (lane == 0) {
-    b.no_ascent += no_ascent;
-    b.fallback += fallback;
     const double t = tau * b.xi_inv;
     b.t = t;
     b.t_prev = t;
     b.have_t_prev = 1;
+  }
+  __syncwarp();
+}
+
+// The step of the iteration in FP32, for the passes of the next one, when it is
+// small and plain: everything an iteration waits for between its step pass and
+// the next gradient pass, with no FP64 instruction in it. The FP64 step
+// (pending_step) follows while the block waits at the next barrier. The pose is
+// base + (base's rounding rest + the step's change), the change good to about
+// 1e-7 of itself, so for the steps taken here (tau up to 2^-8 / kappa, kappa the
+// condition of the root) the passes' pose is the FP64 pose rounded with 0.02 of
+// an ulp more error; the FP64 pose itself is not touched by it. Returns false,
+// with nothing changed, for anything else: larger steps, a step within 1e-4 of
+// the stop test's, the last iteration, no ascent, fallback, second order. Warp 0.
+__device__ bool quick_step(BlockCtx& b, const double* sums, int lane) {
+  const TailConst& tc = b.tc;
+  if (b.small_grad || tc.step_order != 4 || b.k + 1 >= tc.max_iters || !is_pos(sums[1])) return false;
+  const int h1 = __double2hiint(sums[1]), h2 = __double2hiint(sums[2]);
+  const int h3 = __double2hiint(sums[3]), h4 = __double2hiint(sums[4]);
+  // G'(tau) = s1 + 2 s2 tau + 3 s3 tau^2 + 4 s4 tau^3, scaled below 1
+  const int e_max = max(max((h1 >> 20) & 0x7ff, ((h2 >> 20) & 0x7ff) + 1),
+                        max((h3 >> 20) & 0x7ff, (h4 >> 20) & 0x7ff) + 2);
+  if (e_max >= 0x7ff || e_max < 200 || h2 >= 0) return false;
+  const int shift = 1022 - e_max;
+  const float f0 = f64_to_f32_shift(sums[1], shift), f1 = 2.0f * f64_to_f32_shift(sums[2], shift);
+  const float f2 = 3.0f * f64_to_f32_shift(sums[3], shift);
+  const float f3 = 4.0f * f64_to_f32_shift(sums[4], shift);
+  const float ts = cubic_start(f0, f1, f2, f3);
+  float g2;
+  if (!(ts > 0.0f && ts < 0.00390625f) || !falls_to(f1, f2, f3, ts, &g2)) return false;
+  // the root's error is |G'(ts)| / |G''| plus rounding of about 2^-22 mag / |G''|
+  const float mag = f0 + fabsf(f1 * ts) + fabsf(f2 * ts * ts) + fabsf(f3 * ts * ts * ts);
+  const float res = fabsf(fmaf(fmaf(fmaf(f3, ts, f2), ts, f1), ts, f0));
+  if (!(mag <= -g2 * 0.00390625f && res <= 4.8e-7f * mag)) return false;
+  if (b.at_floor && !(ts > tc.eps_pose_f * (1.0f + 1e-4f))) return false;   // may stop: FP64 decides
+  // in the centred frame the unit twist is (omega, v') as the step pass used it
+  const int l = min(lane, 11), r = l >> 2, c = l & 3;
+  const int r1 = r == 2 ? 0 : r + 1, r2 = r == 0 ? 2 : r - 1;
+  const float p[3] = {ts * b.om[0], ts * b.om[1], ts * b.om[2]};
+  const float x = fmaf(p[0], p[0], fmaf(p[1], p[1], p[2] * p[2]));   // below 2^-16
+  const float A = fmaf(x, -1.0f / 6.0f, 1.0f), B = fmaf(x, -1.0f / 24.0f, 0.5f);
+  const float C = 1.0f / 6.0f;
+  // row r of W = hat(phi) applied to y: phi x y; of W^2: phi (phi . y) - x y
+  float y[3], lo, base;
+#pragma unroll
+  for (int k = 0; k < 3; ++k) y[k] = c == 3 ? b.Tb[k] : b.Rb[3 * k + c];
+  base = c == 3 ? b.Tb[r] : b.Rb[3 * r + c];
+  lo = c == 3 ? b.Tl[r] : b.Rl[3 * r + c];
+  const float pr = r == 0 ? p[0] : r == 1 ? p[1] : p[2];
+  const float p1 = r1 == 0 ? p[0] : r1 == 1 ? p[1] : p[2];
+  const float p2 = r2 == 0 ? p[0] : r2 == 1 ? p[1] : p[2];
+  const auto at = [&](const float* v, int i) { return i == 0 ? v[0] : i == 1 ? v[1] : v[2]; };
+  const auto apply = [&](const float* v, float c1, float c2) {   // (c1 W + c2 W^2) v, row r
+    const float dot = fmaf(p[0], v[0], fmaf(p[1], v[1], p[2] * v[2]));
+    const float cross = fmaf(p1, at(v, r2), -(p2 * at(v, r1)));
+    return fmaf(c1, cross, c2 * fmaf(pr, dot, -(x * at(v, r))));
+  };
+  float d = apply(y, A, B);
+  if (c == 3) {
+    const float rho[3] = {ts * b.vc[0], ts * b.vc[1], ts * b.vc[2]};
+    d += at(rho, r) + apply(rho, B, C);
+  }
+  const float v = base + (lo + d);
+  if (lane < 12) {
+    if (c < 3) b.R[3 * r + c] = v;
+    else b.T[r] = v;
+  }
+  if (lane == 0) {
+    b.pending = 1;
+    b.pend_tau = ts;
+    b.k += 1;
+  }
+  __syncwarp();
+  return true;
+}
+
+// The FP64 part of a quick step: the root refined by FP64 Newton steps from the
+// FP32 one (quick_step has shown that G' falls over [0, tau]), the pose, and its
+// parts for the next quick step. One warp, while the block waits at a barrier.
+__device__ __noinline__ void pending_step(BlockCtx& b, int lane) {
+  const double c0 = b.s_raw[1], c1 = mul_pow2(b.s_raw[2], 1), c2 = 3.0 * b.s_raw[3],
+               c3 = mul_pow2(b.s_raw[4], 2);
+  const double c2x2 = mul_pow2(c2, 1), c3x3 = 3.0 * c3;
+  double tau = f32_to_f64(b.pend_tau);
+  for (int it = 0; it < 4; ++it) {
+    const double f = fma(fma(fma(c3, tau, c2), tau, c1), tau, c0);
+    const double fp = fma(fma(c3x3, tau, c2x2), tau, c1);
+    double r = (double)(1.0f / (float)fp);
+    r = r * fma(-fp, r, 2.0);
+    const double dt = -f * r;
+    tau += dt;
+    // settled: |dt| < 2^-20 tau, so that the next step would change nothing
+    if (((__double2hiint(dt) >> 20) & 0x7ff) <= ((__double2hiint(tau) >> 20) & 0x7ff) - 21) break;
+  }
+  apply_step(b, tau, lane);
+  float hi;
+  split_pose(b, lane, &hi);
+  if (lane == 0) b.pending = 0;
+  __syncwarp();
+}
+
+// Step tail: step length, pose update P <- exp(t xi) P, stop test. Warp 0.
+// The step length is found in tau = |xi| t, the step along xi / |xi|: G'(t) =
+// sum_m m S_m t^(m-1) = sigma^2 |xi| sum_m m s_m tau^(m-1), so the quartic of
+// the pass's own sums has the same roots in tau (no powers of |xi| needed),
+// and the twist is tau (xi / |xi|).
+__device__ void finish_step(BlockCtx& b, const double* sums, int lane) {
+  const TailConst& tc = b.tc;
+  if (lane < 5) b.s_raw[lane] = sums[lane];
+  if (lane == 0) {
+    b.nnz_total += b.nnz_grad + (unsigned long long)__double_as_longlong(sums[5]);
+    b.cand_total += b.cand_grad + (unsigned long long)__double_as_longlong(sums[6]);
+  }
+  if (tc.mode == kModeEval) {
+    __syncwarp();
+    if (lane == 0) {
+      form_step_sums(b);
+      b.done = 1;
+    }
+    __syncwarp();
+    return;
+  }
+  if (quick_step(b, sums, lane)) return;
+  // the step length (the same scalar work on every lane)
+  double tau;
+  int no_ascent = 0, fallback = 0;
+  // no step along a gradient below the stop test's threshold (at rounding
+  // level S1 can still be positive, and the quartic's root is then arbitrary);
+  // S1 > 0 exactly when s1 > 0
+  if (b.small_grad || !is_pos(sums[1])) {
+    tau = 0.0;
+    no_ascent = 1;
+  } else {
+    bool ok;
+    if (tc.step_order == 2) {
+      ok = sums[2] < 0.0;
+      tau = ok ? -sums[1] / mul_pow2(sums[2], 1) : 0.0;
+    } else {
+      ok = first_maximiser(sums[1], mul_pow2(sums[2], 1), 3.0 * sums[3], mul_pow2(sums[4], 2),
+                           &tau);
+    }
+    if (!ok) {
+      fallback = 1;
+      // half the previous step, or 1e-3 / |xi| on the first one (tau = 1e-3)
+      tau = b.have_t_prev ? 0.5 * b.t_prev * b.xi_norm : 1e-3;
+    }
+  }
+  apply_step(b, tau, lane);
+  if (lane == 0) {
+    b.no_ascent += no_ascent;
+    b.fallback += fallback;
     // Table 1: |t xi| = |tau| below eps_pose, or |xi| below eps_grad, at the floor
     const bool conv = b.at_floor && (fabs(tau) < tc.eps_pose || b.small_grad);
     b.k += 1;
@@ -994,9 +1135,11 @@ __device__ __forceinline__ void reduce_partials(const double* partials, int nval
 // writes to the same partial buffer (two generations later) come after that
 // arrival, so one buffer per pass kind is enough. Every thread of every block
 // gets the totals in sums[]. Bounded like grid_sync.
-template <class Smem>
+// `meanwhile` runs on one warp of the block between its arrival and the reduction:
+// FP64 work that nothing needs before the pass's tail.
+template <class Smem, class Meanwhile>
 __device__ bool grid_sync_reduce(SolveState* st, unsigned& gen, Smem& sm, const double* partials,
-                                 int nvals, int nblk) {
+                                 int nvals, int nblk, Meanwhile meanwhile) {
   const unsigned g = gen;
   gen += 1;
   __syncthreads();
@@ -1005,6 +1148,7 @@ __device__ bool grid_sync_reduce(SolveState* st, unsigned& gen, Smem& sm, const 
     const bool last = barrier_arrive_count(st) + 1 == target;
     sm.flag = (last || barrier_wait(st, target, sm.b.tc.wait_polls)) ? 1 : 0;
   }
+  if (threadIdx.x >> 5 == kWarps / 2 + 1) meanwhile((int)(threadIdx.x & 31));
   __syncthreads();
   if (!sm.flag) return false;
   reduce_partials(partials, nvals, sm.sums, nblk, sm);
@@ -2149,9 +2293,9 @@ __device__ void build_lists(SolveSmem<DPS, NU>& sm, int warp, int lane, const fl
   const BlockCtx& b = sm.b;
   float R[9], T[3];
 #pragma unroll
-  for (int i = 0; i < 9; ++i) R[i] = __double2float_rn(b.Rp[i]);
+  for (int i = 0; i < 9; ++i) R[i] = b.Rq[i];
 #pragma unroll
-  for (int i = 0; i < 3; ++i) T[i] = __double2float_rn(b.Tp[i]);
+  for (int i = 0; i < 3; ++i) T[i] = b.Tq[i];
   const float rp2 = b.rplan_f * b.rplan_f;
   const unsigned lt = (1u << lane) - 1u;
   int run = 0, coff = cap, k = 0;
@@ -2528,13 +2672,6 @@ __device__ void run_pass(const SolveCfg* cfg, SolveSmem<DPS, NU>& sm, double* pa
   unsigned nnz = 0, cand = 0;
   pass_warp<STEP, DP, MODE, DPS, NU>(cfg, sm, warp, lane, cache, cap, acc, nnz, cand);
   __syncwarp();
-  if (STEP) {
-    // the first warp done with its share forms the FP64 gradient (it reads
-    // the gradient totals, which stay in place until the step barrier)
-    int first = 0;
-    if (lane == 0) first = atomicAdd(&sm.b.fin, 1) == 0 ? 1 : 0;
-    if (__shfl_sync(kFull, first, 0)) gradient_fp64(sm.b, sm.sums, lane);
-  }
 #pragma unroll
   for (int i = 0; i < NACC; ++i) {
     const float v = warp_sum_f(acc[i]);
@@ -2628,6 +2765,7 @@ __device__ void solve_pair(const SolveCfg* __restrict__ cfg, SolveState* __restr
     tc.inv_a2f = (float)(1.0 / cfg->a2);
     tc.inv_b2f = (float)(1.0 / cfg->b2);
     tc.src_radius_f = (float)cfg->src_radius * (1.0f + 1e-6f);
+    tc.eps_pose_f = (float)cfg->eps_pose;
     for (int i = 0; i < 16; ++i) b.P[i] = st->P0[i];
     b.k = 0;
     b.team_rank = team.rank;
@@ -2641,6 +2779,7 @@ __device__ void solve_pair(const SolveCfg* __restrict__ cfg, SolveState* __restr
     b.use_kept = b.collect_kept = b.rebalance = b.use_act = 0;
     b.compact = team.size <= kCompactTeamMax ? 1 : 0;
     b.t = b.t_prev = 0.0;
+    b.pending = 0;
     b.nnz_total = b.cand_total = b.nnz_grad = b.cand_grad = 0;
     b.F = b.xi_norm = 0.0;
     for (int i = 0; i < 6; ++i) b.xi[i] = 0.0;
@@ -2704,7 +2843,10 @@ __device__ void solve_pair(const SolveCfg* __restrict__ cfg, SolveState* __restr
     // ---- gradient pass ----
     run_pass<false, DP, MODE, DPS, NU>(cfg, sm, part_g, cache, cap);
     if (stamp) tg1 = globaltimer();
-    if (!grid_sync_reduce(st, gen, sm, part_g, 9, team.size)) break;
+    if (!grid_sync_reduce(st, gen, sm, part_g, 9, team.size, [&](int ln) {
+          if (sm.b.pending) pending_step(sm.b, ln);
+        }))
+      break;
     if (stamp) tg2 = globaltimer();
     if (warp == 0) {
       if (lane == 0) sm.b.collect_kept = 0;
@@ -2715,7 +2857,10 @@ __device__ void solve_pair(const SolveCfg* __restrict__ cfg, SolveState* __restr
     // ---- step pass ----
     run_pass<true, DP, MODE, DPS, NU>(cfg, sm, part_s, cache, cap);
     if (stamp) ts1 = globaltimer();
-    if (!grid_sync_reduce(st, gen, sm, part_s, 7, team.size)) break;
+    // (the gradient's totals stay in sm.sums until the reduction)
+    if (!grid_sync_reduce(st, gen, sm, part_s, 7, team.size,
+                          [&](int ln) { gradient_fp64(sm.b, sm.sums, ln); }))
+      break;
     if (stamp) ts2 = globaltimer();
     if (warp == 0) {
       BlockCtx& b = sm.b;
