@@ -297,7 +297,7 @@ int reserve_plan(cvo_ctx* ctx, Plan* p, int iters, int ncl, int nblocks) {
   if (rc == CVO_OK) rc = dev_alloc(ctx, (void**)&p->cl_kept, sizeof(int) * ncl, &p->bytes);
   if (rc == CVO_OK) rc = dev_alloc(ctx, (void**)&p->ch_act, sizeof(unsigned) * 32 * (size_t)ncl, &p->bytes);
   if (rc == CVO_OK) rc = dev_alloc(ctx, (void**)&p->cl_act, sizeof(int) * ncl, &p->bytes);
-  if (rc == CVO_OK) rc = dev_alloc(ctx, (void**)&p->group_agg, sizeof(long long) * ng, &p->bytes);
+  if (rc == CVO_OK) rc = dev_alloc(ctx, (void**)&p->group_agg, sizeof(long long) * 2 * ng, &p->bytes);
   if (rc != CVO_OK) {
     free_plan_buffers(ctx, p);
     return rc;
@@ -390,6 +390,7 @@ int configure_plan(cvo_ctx* ctx, Plan* p, Cloud* t, Cloud* s, const std::vector<
   cfg.ch_act = p->ch_act;
   cfg.cl_act = p->cl_act;
   cfg.group_agg = p->group_agg;
+  cfg.agg_stride = (p->cap_ncl + 31) / 32;
   cfg.src_radius = s->radius;
   cfg.cost_chunk = prm.cost_chunk;
   cfg.cost_cluster = prm.cost_cluster;

@@ -107,7 +107,8 @@ struct SolveCfg {
   unsigned* ch_act;        // per cluster, 32 words: bit g of word j is set when source group g
                            //   of chunk j kept a pair in the plan's first gradient pass
   int* cl_act;             // per cluster: the number of such bits
-  long long* group_agg;    // work of each group of 32 consecutive clusters
+  long long* group_agg;    // work of each group of 32 consecutive clusters, two buffers of
+  int agg_stride;          //   agg_stride groups that plans use in turn
   double src_radius;       // max |z'| over the centred source (bounds pose drift)
   int cost_chunk;          // work model: a chunk costs cs4 + cost_chunk pair tests,
   int cost_cluster;        //   staging a cluster cost_cluster, and once kept pairs are

@@ -1194,6 +1194,15 @@ __device__ __forceinline__ float box_dist2(float4 x, float4 lo, float4 hi) {
   return fmaf(dx, dx, fmaf(dy, dy, dz * dz));
 }
 
+// Work of a cluster of cs points with fc filtered candidates, in pair-test units
+// (cluster_work without what only a pass can tell).
+__device__ __forceinline__ long long plan_work(const SolveCfg* cfg, int cs, int fc) {
+  const int nch = (fc + 31) >> 5;
+  return nch > 0 ? (long long)cfg->cost_cluster +
+                       (long long)nch * (((cs + 3) & ~3) + cfg->cost_chunk)
+                 : 0ll;
+}
+
 // Plan of one cluster (one warp): transform its points, bounding box, cell
 // rows within the plan radius -> segments, candidate count; then the
 // candidates themselves are read once and those farther than the plan radius
@@ -1202,9 +1211,11 @@ __device__ __forceinline__ float box_dist2(float4 x, float4 lo, float4 hi) {
 // at the current pose lies within r_c + drift < plan radius of its plan-pose
 // position, which is inside the box). Per segment, the number of candidates
 // that pass gives the filtered offsets the work split and the passes use.
-// s_xs, s_pf, s_cnt: the warp's shared arrays (kMaxSeg + 1 entries).
+// s_xs, s_pf, s_cnt: the warp's shared arrays (kMaxSeg + 1 entries). agg (may be
+// NULL): the work totals of the groups of 32 clusters, to which the cluster's is
+// added (integers: the same total in any order).
 __device__ void plan_cluster(const SolveCfg* cfg, const BlockCtx& b, SolveState* st, int c,
-                             int lane, int* s_xs, int* s_pf, int* s_cnt) {
+                             int lane, int* s_xs, int* s_pf, int* s_cnt, long long* agg) {
   const GridView& g = cfg->grids[b.level];
   const ClusterView& cv = cfg->clusters[b.level];
   __syncwarp();   // the shared arrays of the warp's previous cluster are free
@@ -1351,6 +1362,10 @@ __device__ void plan_cluster(const SolveCfg* cfg, const BlockCtx& b, SolveState*
     cfg->cl_cand[c] = total;
     cfg->cl_fcand[c] = t0 + t1;
     cfg->cl_kept[c] = 0;
+    if (agg) {
+      const long long w = plan_work(cfg, cs, t0 + t1);
+      if (w) atomicAdd(reinterpret_cast<unsigned long long*>(agg + (c >> 5)), (unsigned long long)w);
+    }
     // the box at the plan pose, whether or not the plan filtered (w = 1: the
     // segment offsets count the candidates within the plan radius of it)
     cfg->cl_box[2 * (size_t)c] = make_float4(blo[0], blo[1], blo[2], filt ? 1.f : 0.f);
@@ -1371,11 +1386,13 @@ __device__ void plan_cluster(const SolveCfg* cfg, const BlockCtx& b, SolveState*
 // kCostActive more (its pair bodies); chunks beyond the recorded ones count
 // every group as active.
 __device__ __forceinline__ long long cluster_work(const SolveCfg* cfg, const ClusterView& cv,
-                                                  int c, int* k_out, bool use_kept,
-                                                  bool use_act) {
+                                                  int c, int* k_out, int* cs4_out, int* nch_out,
+                                                  bool use_kept, bool use_act) {
   const int tc = __ldcg(&cfg->cl_fcand[c]);
   const int cs4 = ((cv.cstart[c + 1] - cv.cstart[c]) + 3) & ~3;
   const int nch = (tc + 31) >> 5;
+  *cs4_out = cs4;
+  *nch_out = nch;
   int k = cs4 + cfg->cost_chunk;
   if (use_kept && nch > 0)
     k += (int)(cfg->cost_kept * (float)__ldcg(&cfg->cl_kept[c]) / (float)nch);
@@ -1463,8 +1480,8 @@ __device__ void locate(const SolveCfg* cfg, const ClusterView& cv, int group, lo
                        bool use_kept, bool use_act) {
   const int c = group * 32 + lane;
   long long w = 0;
-  int kk = 4;
-  if (c < cv.ncl) w = cluster_work(cfg, cv, c, &kk, use_kept, use_act);
+  int kk = 4, cs4_l = 4, nch_l = 0;
+  if (c < cv.ncl) w = cluster_work(cfg, cv, c, &kk, &cs4_l, &nch_l, use_kept, use_act);
   long long incl = w;
 #pragma unroll
   for (int off = 1; off < 32; off <<= 1) {
@@ -1478,10 +1495,10 @@ __device__ void locate(const SolveCfg* cfg, const ClusterView& cv, int group, lo
     const int cc = group * 32 + src;
     const long long e = __shfl_sync(kFull, excl, src) + cfg->cost_cluster;
     const int k4 = __shfl_sync(kFull, kk, src);
-    const int cs4 = ((cv.cstart[cc + 1] - cv.cstart[cc]) + 3) & ~3;
+    const int cs4 = __shfl_sync(kFull, cs4_l, src);
     const int oh = k4 - cs4;
     const int G = cs4 >> 2;
-    const int nch = (__ldcg(&cfg->cl_fcand[cc]) + 31) >> 5;
+    const int nch = __shfl_sync(kFull, nch_l, src);
     int j = 0, gq = 0;
     if (use_act && s > e) {
       // chunk j costs k4 + kCostActive x (its active groups; all of them past
@@ -1563,14 +1580,15 @@ __device__ void locate(const SolveCfg* cfg, const ClusterView& cv, int group, lo
 // block left the slowest block 1.2 to 1.3 times the mean. Each further piece costs
 // its warp a cluster to stage and two ends to locate.
 template <int DPS, int NU>
-__device__ void split_work(const SolveCfg* cfg, SolveSmem<DPS, NU>& sm, int tid, Team team) {
+__device__ void split_work(const SolveCfg* cfg, SolveSmem<DPS, NU>& sm, int tid, Team team,
+                           const long long* agg) {
   const ClusterView& cv = cfg->clusters[sm.b.level];
   const int lane = tid & 31, warp = tid >> 5;
   const int ng = (cv.ncl + 31) / 32;
   const int per = (ng + kThreads - 1) / kThreads;
   const int g0 = min(ng, tid * per), g1 = min(ng, g0 + per);
   long long local = 0;
-  for (int gi = g0; gi < g1; ++gi) local += __ldcg(&cfg->group_agg[gi]);
+  for (int gi = g0; gi < g1; ++gi) local += __ldcg(&agg[gi]);
   // inclusive scan over the block's threads: within warps, then the warp totals
   long long incl = local;
 #pragma unroll
@@ -1609,7 +1627,7 @@ __device__ void split_work(const SolveCfg* cfg, SolveSmem<DPS, NU>& sm, int tid,
       base = lo > 0 ? sm.split.scan[lo - 1] : 0;
       const int ge = min(ng, (lo + 1) * per);
       for (int gi = lo * per; gi < ge; ++gi) {
-        const long long w = __ldcg(&cfg->group_agg[gi]);
+        const long long w = __ldcg(&agg[gi]);
         if (at < base + w) {
           group = gi;
           break;
@@ -2796,6 +2814,8 @@ __device__ void solve_pair(const SolveCfg* __restrict__ cfg, SolveState* __restr
   }
   if (team.rank == 0 && tid == 0) st->t_begin_ns = globaltimer();
 
+  int plans = 0;               // plans built by this solve
+  long long* agg = nullptr;    // group totals of the current plan
   while (!sm.b.done) {
     unsigned long long t0 = 0, t1 = 0, t2 = 0, tg1 = 0, tg2 = 0, ts1 = 0, ts2 = 0;
     const bool stamp = records != nullptr && team.rank == 0 && tid == 0;
@@ -2807,9 +2827,19 @@ __device__ void solve_pair(const SolveCfg* __restrict__ cfg, SolveState* __restr
     const int rebalance = !replan && sm.b.rebalance;
     if (replan || rebalance) {
       const ClusterView& cv = cfg->clusters[sm.b.level];
+      const int ng = (cv.ncl + 31) / 32;
       if (replan) {
+        // the plan's own group totals are added up while its clusters are planned,
+        // in one of two buffers in turn; the other is zeroed for the next plan
+        // (every block has long read it). The first plan of a solve finds its
+        // buffer as the last solve left it and forms the totals after a barrier
+        // of their own, as a rebalance does (15 us a plan became 11)
+        agg = cfg->group_agg + (size_t)(plans & 1) * cfg->agg_stride;
+        long long* other = cfg->group_agg + (size_t)((plans + 1) & 1) * cfg->agg_stride;
+        for (long long i = gw * 32 + lane; i < cfg->agg_stride; i += NW * 32) other[i] = 0;
         for (long long c = gw; c < cv.ncl; c += NW)
-          plan_cluster(cfg, sm.b, st, (int)c, lane, sm.ws[warp].seg.xs, sm.ws[warp].seg.pf, sm.ws[warp].seg.fpf);
+          plan_cluster(cfg, sm.b, st, (int)c, lane, sm.ws[warp].seg.xs, sm.ws[warp].seg.pf,
+                       sm.ws[warp].seg.fpf, plans > 0 ? agg : nullptr);
         if (!grid_sync(st, gen, &sm.flag, team.size, sm.b.tc.wait_polls)) break;
       }
       if (tid == 0) {
@@ -2817,19 +2847,21 @@ __device__ void solve_pair(const SolveCfg* __restrict__ cfg, SolveState* __restr
         sm.b.use_act = rebalance && sm.b.plan_filter;
       }
       __syncthreads();
-      const int ng = (cv.ncl + 31) / 32;
-      for (long long gi = gw; gi < ng; gi += NW) {
-        const int c = (int)gi * 32 + lane;
-        int kk;
-        long long w = c < cv.ncl ? cluster_work(cfg, cv, c, &kk, sm.b.use_kept != 0,
-                                                sm.b.use_act != 0)
-                                 : 0;
+      if (rebalance || plans == 0) {
+        for (long long gi = gw; gi < ng; gi += NW) {
+          const int c = (int)gi * 32 + lane;
+          int kk, cs4, nch;
+          long long w = c < cv.ncl ? cluster_work(cfg, cv, c, &kk, &cs4, &nch, sm.b.use_kept != 0,
+                                                  sm.b.use_act != 0)
+                                   : 0;
 #pragma unroll
-        for (int off = 16; off > 0; off >>= 1) w += __shfl_down_sync(kFull, w, off);
-        if (lane == 0) cfg->group_agg[gi] = w;
+          for (int off = 16; off > 0; off >>= 1) w += __shfl_down_sync(kFull, w, off);
+          if (lane == 0) agg[gi] = w;
+        }
+        if (!grid_sync(st, gen, &sm.flag, team.size, sm.b.tc.wait_polls)) break;
       }
-      if (!grid_sync(st, gen, &sm.flag, team.size, sm.b.tc.wait_polls)) break;
-      split_work<DPS, NU>(cfg, sm, tid, team);
+      if (replan) ++plans;
+      split_work<DPS, NU>(cfg, sm, tid, team, agg);
       fill_cache<DP, MODE, DPS, NU>(cfg, sm, warp, lane, cache, cap);
       if (tid == 0) {
         sm.b.need_plan = 0;
