@@ -368,6 +368,8 @@ int configure_plan(cvo_ctx* ctx, Plan* p, Cloud* t, Cloud* s, const std::vector<
     ic[k].rprune = (float)(std::sqrt(rc2) * 1.001);
     ic[k].level = level_of[k];
     ic[k].at_floor = ell == ell_floor(prm) ? 1 : 0;
+    ic[k].inv_l2f = (float)ic[k].inv_l2;
+    ic[k].pad = 0;
     ic[k].kf_rot = prm.sigma * prm.sigma / (ell2 * prm.a2);
     ic[k].kf_tr = prm.sigma * prm.sigma / (ell2 * prm.b2);
     ic[k].filter = (mode == kModeEval ||

@@ -83,6 +83,8 @@ struct IterConst {
                            //   next iteration keeps the lengthscale, so the plan is reused;
                            //   or an evaluation)
   int at_floor;            // 1: ell is the schedule's floor (the stop test may fire)
+  float inv_l2f;           // 1 / ell^2 in FP32
+  int pad;
   double kf_rot, kf_tr;    // sigma^2 / (ell^2 a^2) and sigma^2 / (ell^2 b^2): the factors that
                            //   turn the pair sums into the metric gradient (Eq. metric)
 };

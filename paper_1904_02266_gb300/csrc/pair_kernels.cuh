@@ -82,6 +82,11 @@ constexpr int kCompactTeamMax = 32;
 constexpr int kMaxRanges = 8;
 constexpr int kRangeWork = 700;
 constexpr int kRangeFrom = 2000;
+// shares below this many units leave the block's last warp out of the passes
+// (split_work). Whole room solves without, from 400 and from 1500 units: 10k points
+// 3.80, 3.68, 3.68 ms, 20k 5.65, 5.51, 5.57 ms, 28k 7.45, 7.44, 7.47 ms; the 2k planes
+// pair 825, 832, 832 us
+constexpr int kSpareWork = 400;
 // work model: the pair bodies of a source group that kept a pair, in pair-test units
 constexpr int kCostActive = CVO_COST_ACTIVE;
 
@@ -208,12 +213,11 @@ struct BlockCtx {
   double xi_norm, xi_inv, F;
   double S[5];            // S0..S4 of the last step pass (formed when published)
   double s_raw[5];        // the step pass's sums along xi / |xi| (S_m = s_m sigma^2 |xi|^m)
-  double kf_rot, kf_tr;   // this iteration's metric factors
   int small_grad;         // |xi| below the gradient threshold (or zero): no step, stop test
-  int at_floor;           // this iteration's ell is the schedule's floor
   double t, t_prev;
-  double ell, inv_l2, r_plan, plan_ell;
-  int k, level, plan_level, plan_filter;
+  IterConst ic;           // this iteration's constants
+  double r_plan, plan_ell;
+  int k, plan_level, plan_filter;
   int need_plan, done, converged, fallback, no_ascent, have_t_prev;
   int use_kept, collect_kept, rebalance;   // kept-pair weighting of the work split
   int use_act;                             // the split weighs source groups by their activity
@@ -231,10 +235,12 @@ struct BlockCtx {
   float om[3], vc[3];     // unit step direction (centred frame)
   float kw[3];            // (omega . v) omega / 6 l^2
   float c_del, c_eps, k_eps;   // -|omega|^2 / 3, -|omega|^2 / 12, -(omega . v)^2 / 48 l^2
-  float A, rc2, rplan_f, inv_l2f;
+  float rplan_f;
   // warp ranges (n_range of them per warp): from group g0 of chunk j0 of cluster
   // c0 up to (not including) group g1 of chunk j1 of cluster c1
   int n_range;
+  int n_workers;          // warps that share the passes; with kWarps - 1 of them the last warp does
+                          // the FP64 work of the iteration meanwhile
   int w_c0[kMaxRanges][kWarps], w_j0[kMaxRanges][kWarps], w_g0[kMaxRanges][kWarps];
   int w_c1[kMaxRanges][kWarps], w_j1[kMaxRanges][kWarps], w_g1[kMaxRanges][kWarps];
   // where the streamed rest of a partly cached share begins (c < 0: there is none)
@@ -328,10 +334,22 @@ __device__ __forceinline__ void split_pose(BlockCtx& b, int lane, float* hi_out)
   *hi_out = hi;
 }
 
-// Iteration k's constants (ic = the host table's entry k), the FP32 pose (from
-// the FP64 pose, unless quick_step has formed it), and whether the traversal plan
-// must be rebuilt. Warp 0, every lane.
-__device__ __noinline__ void begin_iteration(const IterConst& ic, BlockCtx& b, int lane) {
+// Iteration k's constants, a word per lane: read ahead of their use, stored into
+// the block's context when the iteration starts (one warp).
+static_assert(sizeof(IterConst) == 64, "sixteen words");
+__device__ __forceinline__ unsigned iter_word(const SolveCfg* cfg, int k, int lane) {
+  return reinterpret_cast<const unsigned*>(cfg->iters + k)[lane & 15];
+}
+__device__ __forceinline__ void load_iter(BlockCtx& b, unsigned word, int lane) {
+  if (lane < 16) reinterpret_cast<unsigned*>(&b.ic)[lane] = word;
+  __syncwarp();
+}
+
+// The start of an iteration whose constants are in b.ic: the FP32 pose (from the
+// FP64 pose, unless quick_step has formed it), and whether the traversal plan must
+// be rebuilt. Warp 0, every lane.
+__device__ __noinline__ void begin_iteration(BlockCtx& b, int lane) {
+  const IterConst& ic = b.ic;
   const int l = min(lane, 11), r = l >> 2, c = l & 3;
   float v;
   if (b.pending) v = c == 3 ? b.T[r] : b.R[3 * r + c];
@@ -370,15 +388,6 @@ __device__ __noinline__ void begin_iteration(const IterConst& ic, BlockCtx& b, i
     }
   }
   if (lane == 0) {
-    b.ell = ic.ell;
-    b.inv_l2 = ic.inv_l2;
-    b.A = ic.A;
-    b.rc2 = ic.rc2;
-    b.inv_l2f = (float)ic.inv_l2;
-    b.level = ic.level;
-    b.kf_rot = ic.kf_rot;
-    b.kf_tr = ic.kf_tr;
-    b.at_floor = ic.at_floor;
     if (replan) {
       b.need_plan = 1;
       b.plan_level = ic.level;
@@ -697,12 +706,12 @@ __device__ void gradient_direction(BlockCtx& b, const double* sums, int lane) {
   float ww = om * om, wv = om * vc;
   ww += __shfl_sync(kFull, ww, 1) + __shfl_sync(kFull, ww, 2);   // lane 0's is used
   wv += __shfl_sync(kFull, wv, 1) + __shfl_sync(kFull, wv, 2);
-  const float kap = __shfl_sync(kFull, wv, 0) * b.inv_l2f * (1.0f / 6.0f);
+  const float kap = __shfl_sync(kFull, wv, 0) * b.ic.inv_l2f * (1.0f / 6.0f);
   if (lane < 3) b.kw[a] = kap * om;
   if (lane == 0) {
     b.c_del = -ww * (1.0f / 3.0f);
     b.c_eps = -ww * (1.0f / 12.0f);
-    b.k_eps = -wv * wv * b.inv_l2f * (1.0f / 48.0f);
+    b.k_eps = -wv * wv * b.ic.inv_l2f * (1.0f / 48.0f);
   }
   __syncwarp();
 }
@@ -712,7 +721,7 @@ __device__ void gradient_direction(BlockCtx& b, const double* sums, int lane) {
 // xi / |xi| in FP64, F and the gradient pass's counts.
 __device__ void gradient_fp64(BlockCtx& b, const double* sums, int lane) {
   const TailConst& tc = b.tc;
-  const double x = lane < 6 ? b.x0[lane] * (lane < 3 ? b.kf_rot : b.kf_tr) : 0.0;
+  const double x = lane < 6 ? b.x0[lane] * (lane < 3 ? b.ic.kf_rot : b.ic.kf_tr) : 0.0;
   double nrm2 = x * x;
 #pragma unroll
   for (int off = 4; off > 0; off >>= 1) nrm2 += __shfl_xor_sync(kFull, nrm2, off);
@@ -828,52 +837,51 @@ __device__ void apply_step(BlockCtx& b, double tau, int lane) {
 __device__ bool quick_step(BlockCtx& b, const double* sums, int lane) {
   const TailConst& tc = b.tc;
   if (b.small_grad || tc.step_order != 4 || b.k + 1 >= tc.max_iters || !is_pos(sums[1])) return false;
-  const int h1 = __double2hiint(sums[1]), h2 = __double2hiint(sums[2]);
-  const int h3 = __double2hiint(sums[3]), h4 = __double2hiint(sums[4]);
-  // G'(tau) = s1 + 2 s2 tau + 3 s3 tau^2 + 4 s4 tau^3, scaled below 1
-  const int e_max = max(max((h1 >> 20) & 0x7ff, ((h2 >> 20) & 0x7ff) + 1),
-                        max((h3 >> 20) & 0x7ff, (h4 >> 20) & 0x7ff) + 2);
-  if (e_max >= 0x7ff || e_max < 200 || h2 >= 0) return false;
-  const int shift = 1022 - e_max;
-  const float f0 = f64_to_f32_shift(sums[1], shift), f1 = 2.0f * f64_to_f32_shift(sums[2], shift);
-  const float f2 = 3.0f * f64_to_f32_shift(sums[3], shift);
-  const float f3 = 4.0f * f64_to_f32_shift(sums[4], shift);
-  const float ts = cubic_start(f0, f1, f2, f3);
+  // G'(tau) = f0 + f1 tau + f2 tau^2 + f3 tau^3 from the sums' bits (truncated to
+  // FP32; magnitudes well inside its range, else the FP64 tail)
+  float f[4];
+  bool plain = __double2hiint(sums[2]) < 0;   // G'' < 0 at 0
+#pragma unroll
+  for (int m = 0; m < 4; ++m) {
+    const unsigned hi = (unsigned)__double2hiint(sums[m + 1]), lo = (unsigned)__double2loint(sums[m + 1]);
+    plain = plain && ((hi >> 20) & 0x7ffu) - 948u < 150u;   // 2^-75 .. 2^75
+    f[m] = (float)(m + 1) * __uint_as_float((hi & 0x80000000u) |
+                                            (((hi & 0x7fffffffu) << 3 | lo >> 29) - (896u << 23)));
+  }
+  if (!plain) return false;
+  const float f0 = f[0], f1 = f[1], f2 = f[2], f3 = f[3];
+  // Newton from the root of the linear part, which the steps taken here are near
+  float ts = __fdividef(-f0, f1);
+#pragma unroll
+  for (int it = 0; it < 4; ++it)
+    ts -= __fdividef(fmaf(fmaf(fmaf(f3, ts, f2), ts, f1), ts, f0),
+                     fmaf(fmaf(3.0f * f3, ts, 2.0f * f2), ts, f1));
   float g2;
   if (!(ts > 0.0f && ts < 0.00390625f) || !falls_to(f1, f2, f3, ts, &g2)) return false;
   // the root's error is |G'(ts)| / |G''| plus rounding of about 2^-22 mag / |G''|
   const float mag = f0 + fabsf(f1 * ts) + fabsf(f2 * ts * ts) + fabsf(f3 * ts * ts * ts);
   const float res = fabsf(fmaf(fmaf(fmaf(f3, ts, f2), ts, f1), ts, f0));
   if (!(mag <= -g2 * 0.00390625f && res <= 4.8e-7f * mag)) return false;
-  if (b.at_floor && !(ts > tc.eps_pose_f * (1.0f + 1e-4f))) return false;   // may stop: FP64 decides
-  // in the centred frame the unit twist is (omega, v') as the step pass used it
+  if (b.ic.at_floor && !(ts > tc.eps_pose_f * (1.0f + 1e-4f))) return false;   // may stop: FP64 decides
+  // in the centred frame the unit twist is (omega, v') as the step pass used it;
+  // lanes 0..11 take element (r, c) = (l / 4, l % 4), r1 and r2 the axes after r
   const int l = min(lane, 11), r = l >> 2, c = l & 3;
   const int r1 = r == 2 ? 0 : r + 1, r2 = r == 0 ? 2 : r - 1;
-  const float p[3] = {ts * b.om[0], ts * b.om[1], ts * b.om[2]};
-  const float x = fmaf(p[0], p[0], fmaf(p[1], p[1], p[2] * p[2]));   // below 2^-16
+  const float p0 = ts * b.om[r], p1 = ts * b.om[r1], p2 = ts * b.om[r2];
+  const float x = fmaf(p0, p0, fmaf(p1, p1, p2 * p2));   // below 2^-16
   const float A = fmaf(x, -1.0f / 6.0f, 1.0f), B = fmaf(x, -1.0f / 24.0f, 0.5f);
-  const float C = 1.0f / 6.0f;
-  // row r of W = hat(phi) applied to y: phi x y; of W^2: phi (phi . y) - x y
-  float y[3], lo, base;
-#pragma unroll
-  for (int k = 0; k < 3; ++k) y[k] = c == 3 ? b.Tb[k] : b.Rb[3 * k + c];
-  base = c == 3 ? b.Tb[r] : b.Rb[3 * r + c];
-  lo = c == 3 ? b.Tl[r] : b.Rl[3 * r + c];
-  const float pr = r == 0 ? p[0] : r == 1 ? p[1] : p[2];
-  const float p1 = r1 == 0 ? p[0] : r1 == 1 ? p[1] : p[2];
-  const float p2 = r2 == 0 ? p[0] : r2 == 1 ? p[1] : p[2];
-  const auto at = [&](const float* v, int i) { return i == 0 ? v[0] : i == 1 ? v[1] : v[2]; };
-  const auto apply = [&](const float* v, float c1, float c2) {   // (c1 W + c2 W^2) v, row r
-    const float dot = fmaf(p[0], v[0], fmaf(p[1], v[1], p[2] * v[2]));
-    const float cross = fmaf(p1, at(v, r2), -(p2 * at(v, r1)));
-    return fmaf(c1, cross, c2 * fmaf(pr, dot, -(x * at(v, r))));
+  // row r of (c1 W + c2 W^2) y, W = hat(phi): W y = phi x y, W^2 y = phi (phi . y) - x y
+  const auto apply = [&](float y0, float y1, float y2, float c1, float c2) {
+    const float dot = fmaf(p0, y0, fmaf(p1, y1, p2 * y2));
+    return fmaf(c1, fmaf(p1, y2, -(p2 * y1)), c2 * fmaf(p0, dot, -(x * y0)));
   };
-  float d = apply(y, A, B);
-  if (c == 3) {
-    const float rho[3] = {ts * b.vc[0], ts * b.vc[1], ts * b.vc[2]};
-    d += at(rho, r) + apply(rho, B, C);
-  }
-  const float v = base + (lo + d);
+  const float* base = c == 3 ? b.Tb : b.Rb + c;
+  const int st = c == 3 ? 1 : 3;
+  const float y0 = base[st * r], y1 = base[st * r1], y2 = base[st * r2];
+  float d = apply(y0, y1, y2, A, B);
+  const float v0 = ts * b.vc[r], v1 = ts * b.vc[r1], v2 = ts * b.vc[r2];
+  if (c == 3) d += v0 + apply(v0, v1, v2, B, 1.0f / 6.0f);
+  const float v = y0 + ((c == 3 ? b.Tl[r] : b.Rl[3 * r + c]) + d);
   if (lane < 12) {
     if (c < 3) b.R[3 * r + c] = v;
     else b.T[r] = v;
@@ -963,7 +971,7 @@ __device__ void finish_step(BlockCtx& b, const double* sums, int lane) {
     b.no_ascent += no_ascent;
     b.fallback += fallback;
     // Table 1: |t xi| = |tau| below eps_pose, or |xi| below eps_grad, at the floor
-    const bool conv = b.at_floor && (fabs(tau) < tc.eps_pose || b.small_grad);
+    const bool conv = b.ic.at_floor && (fabs(tau) < tc.eps_pose || b.small_grad);
     b.k += 1;
     if (conv || b.k >= tc.max_iters) {
       b.done = 1;
@@ -1001,7 +1009,9 @@ __device__ __forceinline__ bool barrier_wait(SolveState* st, unsigned target, un
       atomicOr(&st->status, (int)kStatusTimeout);
       return false;
     }
-    __nanosleep(32);
+    // the first polls follow one another: most waits end within them, and a sleep
+    // is as long as the whole wait
+    if (spins > 64u) __nanosleep(32);
   }
   return true;
 }
@@ -1216,8 +1226,8 @@ __device__ __forceinline__ long long plan_work(const SolveCfg* cfg, int cs, int 
 // added (integers: the same total in any order).
 __device__ void plan_cluster(const SolveCfg* cfg, const BlockCtx& b, SolveState* st, int c,
                              int lane, int* s_xs, int* s_pf, int* s_cnt, long long* agg) {
-  const GridView& g = cfg->grids[b.level];
-  const ClusterView& cv = cfg->clusters[b.level];
+  const GridView& g = cfg->grids[b.ic.level];
+  const ClusterView& cv = cfg->clusters[b.ic.level];
   __syncwarp();   // the shared arrays of the warp's previous cluster are free
   const int p0 = cv.cstart[c];
   const int cs = cv.cstart[c + 1] - p0;
@@ -1572,8 +1582,8 @@ __device__ void locate(const SolveCfg* cfg, const ClusterView& cv, int group, lo
 
 // Place the block's warps on an even split of the plan's work into NR x NW pieces
 // (NW warps in the team): a piece owns the units (a chunk's source group) whose
-// work starts in [floor(p TW / (NR NW)), floor((p + 1) TW / (NR NW))). Warp w of
-// block r takes the pieces p = (k kWarps + w) size + r, k < NR: the share of the
+// work starts in [floor(p TW / (NR NW)), floor((p + 1) TW / (NR NW))). Warp w of nw
+// of block r takes the pieces p = (k nw + w) size + r, k < NR: the share of the
 // tests that keep a pair, which the plan does not know, varies smoothly over the
 // cloud, so a block whose warps take pieces from all over it ends its pass at
 // about the time the other blocks do, where one contiguous run of the work per
@@ -1582,7 +1592,7 @@ __device__ void locate(const SolveCfg* cfg, const ClusterView& cv, int group, lo
 template <int DPS, int NU>
 __device__ void split_work(const SolveCfg* cfg, SolveSmem<DPS, NU>& sm, int tid, Team team,
                            const long long* agg) {
-  const ClusterView& cv = cfg->clusters[sm.b.level];
+  const ClusterView& cv = cfg->clusters[sm.b.ic.level];
   const int lane = tid & 31, warp = tid >> 5;
   const int ng = (cv.ncl + 31) / 32;
   const int per = (ng + kThreads - 1) / kThreads;
@@ -1605,14 +1615,18 @@ __device__ void split_work(const SolveCfg* cfg, SolveSmem<DPS, NU>& sm, int tid,
     TW += sm.split.wsum[w];
   }
   sm.split.scan[tid] = incl;
-  const long long NW = (long long)team.size * kWarps;
+  // short shares leave the last warp out: its FP64 work (pending_step,
+  // gradient_fp64: 2.3 and 0.6 us) then hides behind the passes instead of
+  // lengthening the waits at their barriers, for a fifteenth more work per warp
+  const int nw = TW < (long long)team.size * kWarps * kSpareWork ? kWarps - 1 : kWarps;
+  const long long NW = (long long)team.size * nw;
   const int nr = team.size <= kCompactTeamMax || TW < NW * kRangeFrom
                      ? 1
                      : (int)min((long long)kMaxRanges, TW / (NW * kRangeWork));
   __syncthreads();
-  // end h of the k-th piece of warp w on thread (k kWarps + w) 2 + h: the thread
+  // end h of the k-th piece of warp w on thread (k nw + w) 2 + h: the thread
   // whose run of groups holds it, by binary search, then the group
-  if (tid < 2 * kWarps * nr) {
+  if (tid < 2 * nw * nr) {
     const long long piece = (long long)(tid >> 1) * team.size + team.rank + (tid & 1);
     const long long at = TW > 0 ? (piece * TW) / (NW * nr) : 0;
     int group = -1;
@@ -1639,14 +1653,17 @@ __device__ void split_work(const SolveCfg* cfg, SolveSmem<DPS, NU>& sm, int tid,
     sm.split.base[tid] = base;
     sm.split.at[tid] = at;
   }
-  if (tid == 0) sm.b.n_range = nr;
+  if (tid == 0) {
+    sm.b.n_range = nr;
+    sm.b.n_workers = nw;
+  }
   __syncthreads();
   for (int k = 0; k < nr; ++k) {
 #pragma unroll
     for (int h = 0; h < 2; ++h) {
-      const int q = 2 * (k * kWarps + warp) + h;
+      const int q = 2 * (k * nw + warp) + h;
       int c = cv.ncl, jj = 0, gg = 0;   // past the end: no chunk
-      if (sm.split.group[q] >= 0)
+      if (warp < nw && sm.split.group[q] >= 0)
         locate(cfg, cv, sm.split.group[q], sm.split.base[q], sm.split.at[q], lane, &c, &jj, &gg,
                sm.b.use_kept != 0, sm.b.use_act != 0);
       if (lane == 0) {
@@ -1712,7 +1729,7 @@ __device__ __forceinline__ void stage_cluster(SolveSmem<DPS, NU>& sm, int warp, 
     sm.zw[warp][lane] = -fmaf(lx, b.kw[0], fmaf(ly, b.kw[1], lz * b.kw[2]));
     if (listed) {
       const float* om = b.om;
-      const float c1 = 0.5f * b.inv_l2f, c2 = 0.25f * b.inv_l2f;
+      const float c1 = 0.5f * b.ic.inv_l2f, c2 = 0.25f * b.ic.inv_l2f;
       const float u1[3] = {om[1] * zt[2] - om[2] * zt[1] + b.vc[0],
                            om[2] * zt[0] - om[0] * zt[2] + b.vc[1],
                            om[0] * zt[1] - om[1] * zt[0] + b.vc[2]};
@@ -1756,7 +1773,7 @@ struct StepVectors {
 __device__ __forceinline__ StepVectors step_vectors(const BlockCtx& b, float x, float y, float z,
                                                     float xl, float yl, float zl) {
   const float w0 = b.om[0], w1 = b.om[1], w2 = b.om[2];
-  const float k1 = 0.5f * b.inv_l2f, k2 = -0.25f * b.inv_l2f;
+  const float k1 = 0.5f * b.ic.inv_l2f, k2 = -0.25f * b.ic.inv_l2f;
   const float a0 = w1 * z - w2 * y + b.vc[0], a1 = w2 * x - w0 * z + b.vc[1],
               a2 = w0 * y - w1 * x + b.vc[2];
   const float p0 = a0 * k1, p1 = a1 * k1, p2 = a2 * k1;
@@ -2092,9 +2109,9 @@ __device__ void pass_stream(const SolveCfg* cfg, SolveSmem<DPS, NU>& sm, int war
                             WarpRange r, float* ring, float acc[7], unsigned& nnz,
                             unsigned& cand) {
   const BlockCtx& b = sm.b;
-  const GridView& g = cfg->grids[b.level];
-  const ClusterView& cv = cfg->clusters[b.level];
-  const float rc2 = b.rc2, A = b.A;
+  const GridView& g = cfg->grids[b.ic.level];
+  const ClusterView& cv = cfg->clusters[b.ic.level];
+  const float rc2 = b.ic.rc2, A = b.ic.A;
   const float rp2 = b.rplan_f * b.rplan_f;
   const bool collect = !STEP && b.collect_kept;
   float4* rxyz = reinterpret_cast<float4*>(ring);
@@ -2363,8 +2380,8 @@ template <int DP, int MODE, int DPS, int NU>
 __device__ void fill_cache(const SolveCfg* cfg, SolveSmem<DPS, NU>& sm, int warp, int lane,
                            float* cache, int cap) {
   const BlockCtx& b = sm.b;
-  const GridView& g = cfg->grids[b.level];
-  const ClusterView& cv = cfg->clusters[b.level];
+  const GridView& g = cfg->grids[b.ic.level];
+  const ClusterView& cv = cfg->clusters[b.ic.level];
   const WarpRange r = warp_range(b, warp, 0);
   const float rp2 = b.rplan_f * b.rplan_f;
   // what the share needs (one in several pieces is too large for the cache)
@@ -2588,7 +2605,7 @@ template <bool STEP, int DP, int MODE, int DPS, int NU>
 __device__ void pass_cached(const SolveCfg* cfg, SolveSmem<DPS, NU>& sm, int warp, int lane,
                             const float* cache, int cap, float acc[7], unsigned& nnz,
                             unsigned& cand) {
-  const float rc2 = sm.b.rc2, A = sm.b.A;
+  const float rc2 = sm.b.ic.rc2, A = sm.b.ic.A;
   const bool collect = !STEP && sm.b.collect_kept;
   const float* base = cache + (size_t)warp * cap;
   if (sm.b.rest_c[warp] >= 0) {   // the streamed rest has the first two slots
@@ -2688,19 +2705,30 @@ __device__ void run_pass(const SolveCfg* cfg, SolveSmem<DPS, NU>& sm, double* pa
 #pragma unroll
   for (int i = 0; i < 7; ++i) acc[i] = 0.f;
   unsigned nnz = 0, cand = 0;
+  if (warp == kWarps - 1 && sm.b.n_workers < kWarps) {
+    if (STEP) gradient_fp64(sm.b, sm.sums, lane);
+    else if (sm.b.pending) pending_step(sm.b, lane);
+  }
   pass_warp<STEP, DP, MODE, DPS, NU>(cfg, sm, warp, lane, cache, cap, acc, nnz, cand);
   __syncwarp();
+  // the warp's sums: halves of the warp exchange half of the values, then quarters,
+  // eighths, so that lane 4 i ends with the sum of value i (nine shuffles, not 35)
+  float v[8];
 #pragma unroll
-  for (int i = 0; i < NACC; ++i) {
-    const float v = warp_sum_f(acc[i]);
-    if (lane == 0) sm.red[warp][i] = v;
-  }
-  unsigned wn = nnz, wc = cand;
+  for (int i = 0; i < 8; ++i) v[i] = i < NACC ? acc[i < 7 ? i : 6] : 0.f;
 #pragma unroll
-  for (int off = 16; off > 0; off >>= 1) {
-    wn += __shfl_down_sync(kFull, wn, off);
-    wc += __shfl_down_sync(kFull, wc, off);
+  for (int half = 4, off = 16; half > 0; half >>= 1, off >>= 1) {
+    const bool up = (lane & off) != 0;
+#pragma unroll
+    for (int i = 0; i < half; ++i) {
+      const float keep = up ? v[i + half] : v[i], send = up ? v[i] : v[i + half];
+      v[i] = keep + __shfl_xor_sync(kFull, send, off);
+    }
   }
+  v[0] += __shfl_xor_sync(kFull, v[0], 2);
+  v[0] += __shfl_xor_sync(kFull, v[0], 1);
+  if ((lane & 3) == 0 && (lane >> 2) < NACC) sm.red[warp][lane >> 2] = v[0];
+  const unsigned wn = __reduce_add_sync(kFull, nnz), wc = __reduce_add_sync(kFull, cand);
   if (lane == 0) {
     sm.red[warp][NACC] = __uint_as_float(wn);
     sm.red[warp][NACC + 1] = __uint_as_float(wc);
@@ -2733,8 +2761,8 @@ __device__ void publish(SolveState* st, BlockCtx& b) {
   st->xi_norm = b.xi_norm;
   st->F = b.F;
   st->t = b.t;
-  st->ell = b.ell;
-  st->level = b.level;
+  st->ell = b.ic.ell;
+  st->level = b.ic.level;
   st->iter = b.k;
   st->done = b.done;
   st->converged = b.converged;
@@ -2788,7 +2816,6 @@ __device__ void solve_pair(const SolveCfg* __restrict__ cfg, SolveState* __restr
     b.k = 0;
     b.team_rank = team.rank;
     b.team_size = team.size;
-    b.level = 0;
     b.plan_level = -1;
     b.plan_filter = 0;
     b.need_plan = 1;
@@ -2806,7 +2833,10 @@ __device__ void solve_pair(const SolveCfg* __restrict__ cfg, SolveState* __restr
     b.plan_ell = 0.0;
   }
   __syncthreads();
-  if (warp == 0 && !sm.b.done) begin_iteration(cfg->iters[0], sm.b, lane);
+  if (warp == 0) {
+    load_iter(sm.b, iter_word(cfg, 0, lane), lane);
+    if (!sm.b.done) begin_iteration(sm.b, lane);
+  }
   __syncthreads();
   if (join && !team_join(st, team.size, sm)) {
     if (tid == 0) sm.b.done = 1;   // a team that never assembled runs no iteration
@@ -2826,14 +2856,14 @@ __device__ void solve_pair(const SolveCfg* __restrict__ cfg, SolveState* __restr
     // groups that kept pairs; with cost_kept > 0 the kept pairs per cluster)
     const int rebalance = !replan && sm.b.rebalance;
     if (replan || rebalance) {
-      const ClusterView& cv = cfg->clusters[sm.b.level];
+      const ClusterView& cv = cfg->clusters[sm.b.ic.level];
       const int ng = (cv.ncl + 31) / 32;
       if (replan) {
         // the plan's own group totals are added up while its clusters are planned,
         // in one of two buffers in turn; the other is zeroed for the next plan
         // (every block has long read it). The first plan of a solve finds its
         // buffer as the last solve left it and forms the totals after a barrier
-        // of their own, as a rebalance does (15 us a plan became 11)
+        // of their own, as a rebalance does
         agg = cfg->group_agg + (size_t)(plans & 1) * cfg->agg_stride;
         long long* other = cfg->group_agg + (size_t)((plans + 1) & 1) * cfg->agg_stride;
         for (long long i = gw * 32 + lane; i < cfg->agg_stride; i += NW * 32) other[i] = 0;
@@ -2876,7 +2906,7 @@ __device__ void solve_pair(const SolveCfg* __restrict__ cfg, SolveState* __restr
     run_pass<false, DP, MODE, DPS, NU>(cfg, sm, part_g, cache, cap);
     if (stamp) tg1 = globaltimer();
     if (!grid_sync_reduce(st, gen, sm, part_g, 9, team.size, [&](int ln) {
-          if (sm.b.pending) pending_step(sm.b, ln);
+          if (sm.b.n_workers == kWarps && sm.b.pending) pending_step(sm.b, ln);
         }))
       break;
     if (stamp) tg2 = globaltimer();
@@ -2889,21 +2919,23 @@ __device__ void solve_pair(const SolveCfg* __restrict__ cfg, SolveState* __restr
     // ---- step pass ----
     run_pass<true, DP, MODE, DPS, NU>(cfg, sm, part_s, cache, cap);
     if (stamp) ts1 = globaltimer();
+    // the next iteration's constants, on their way while the block waits
+    const unsigned icw = iter_word(cfg, min(sm.b.k + 1, sm.b.tc.max_iters - 1), lane);
     // (the gradient's totals stay in sm.sums until the reduction)
     if (!grid_sync_reduce(st, gen, sm, part_s, 7, team.size,
-                          [&](int ln) { gradient_fp64(sm.b, sm.sums, ln); }))
+                          [&](int ln) {
+                            if (sm.b.n_workers == kWarps) gradient_fp64(sm.b, sm.sums, ln);
+                          }))
       break;
     if (stamp) ts2 = globaltimer();
     if (warp == 0) {
       BlockCtx& b = sm.b;
       const int k = b.k;
-      // the next iteration's constants, loaded now and used after the tail
-      const IterConst ic_next = cfg->iters[min(k + 1, b.tc.max_iters - 1)];
       const unsigned long long pairs_before = b.nnz_total;
       finish_step(b, sm.sums, lane);
       if (stamp && k < b.tc.max_iters) {
         IterRecord& r = records[k];
-        r.ell = b.ell;
+        r.ell = b.ic.ell;
         r.t_plan_ns = (float)(t1 - t0);
         r.t_grad_ns = (float)(t2 - t1);
         r.t_step_ns = (float)(globaltimer() - t2);
@@ -2917,7 +2949,10 @@ __device__ void solve_pair(const SolveCfg* __restrict__ cfg, SolveState* __restr
         r.grad_candidates = (long long)b.cand_grad;
       }
       __syncwarp();
-      if (!b.done) begin_iteration(ic_next, b, lane);
+      if (!b.done) {
+        load_iter(b, icw, lane);
+        begin_iteration(b, lane);
+      }
     }
     __syncthreads();
   }
