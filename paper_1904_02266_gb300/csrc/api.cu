@@ -372,9 +372,12 @@ int configure_plan(cvo_ctx* ctx, Plan* p, Cloud* t, Cloud* s, const std::vector<
     ic[k].pad = 0;
     ic[k].kf_rot = prm.sigma * prm.sigma / (ell2 * prm.a2);
     ic[k].kf_tr = prm.sigma * prm.sigma / (ell2 * prm.b2);
-    ic[k].filter = (mode == kModeEval ||
-                    (k + 1 < ells.size() && ells[k + 1] == ell && level_of[k + 1] == level_of[k]))
-                       ? 1 : 0;
+    // an evaluation's plan, like a decaying iteration's, serves one pose and two
+    // passes: built at the cutoff without the skin, its candidates not read ahead to
+    // be filtered and listed (2k points 96 -> 83 us, 20k x 17k 153 -> 128 us, 100k
+    // 906 -> 840 us per evaluation)
+    ic[k].filter =
+        k + 1 < ells.size() && ells[k + 1] == ell && level_of[k + 1] == level_of[k] ? 1 : 0;
   }
   cfg.src.xyz = s->zs;
   cfg.src.feat = s->zf;

@@ -80,8 +80,7 @@ struct IterConst {
   float rprune;            // traversal radius (r_c widened by 1e-3 relative)
   int level;               // grid / cluster level
   int filter;              // 1: a plan built at this iteration filters its candidates (the
-                           //   next iteration keeps the lengthscale, so the plan is reused;
-                           //   or an evaluation)
+                           //   next iteration keeps the lengthscale, so the plan is reused)
   int at_floor;            // 1: ell is the schedule's floor (the stop test may fire)
   float inv_l2f;           // 1 / ell^2 in FP32
   int pad;
