@@ -64,11 +64,15 @@ constexpr double kSkin = 0.10;              // plan radius margin (fraction of t
 constexpr double kLoose = 1.25;             // replan when the plan radius exceeds this factor
 constexpr int kFilterMax = 1024;            // candidates of a cluster the plan filters at most
 constexpr int kActChunks = 32;              // chunks per cluster whose source-group activity is kept
-// teams of at most this many blocks box-test the candidates of unfiltered
-// clusters in the streamed passes (their warps' shares are long runs of
-// chunks); larger teams, whose shares are short and whose work split counts
-// unfiltered candidates, stream them unfiltered
-constexpr int kCompactTeamMax = 32;
+// Teams of at most kSmallTeam blocks hold long shares. The streamed passes box-test
+// the candidates of unfiltered clusters on the way in such teams, and wherever a
+// warp's share is at least kCompactWork pair-test units; shorter shares of larger
+// teams, whose split counts unfiltered candidates, come out more uneven than the
+// test saves. Whole-GPU teams with every share tested, from 3000 units, and none:
+// 20k room solve 5.55, 5.51, 5.51 ms, 100k evaluation 827, 820, 844 us, 16 served
+// requests 95.6, 96.2, 98.1 ms
+constexpr int kSmallTeam = 32;
+constexpr int kCompactWork = 3000;
 #ifndef CVO_COST_ACTIVE
 #define CVO_COST_ACTIVE 12
 #endif
@@ -77,11 +81,12 @@ constexpr int kCompactTeamMax = 32;
 // kMaxRanges, from kRangeFrom units on. Whole-GPU teams, 100k room pair: up to 4
 // pieces of 1500 units 46.9 ms, 8 of 1500 46.2, 8 of 700 45.4; at 20k points
 // (about 1000 units a warp) a second piece costs a cluster and two ends more than
-// it evens out. Teams of at most kCompactTeamMax blocks hold long shares already:
-// one piece (64-pair batch: 1 to 4 pieces 110.1, 110.9, 111.8, 113.4 ms)
+// it evens out. Small teams: two pieces from kSmallTeamFrom units on (64-pair batch:
+// one piece 105.0 ms, two 104.0, up to eight 111.9)
 constexpr int kMaxRanges = 8;
 constexpr int kRangeWork = 700;
 constexpr int kRangeFrom = 2000;
+constexpr int kSmallTeamFrom = 20000;
 // shares below this many units leave the block's last warp out of the passes
 // (split_work). Whole room solves without, from 400 and from 1500 units: 10k points
 // 3.80, 3.68, 3.68 ms, 20k 5.65, 5.51, 5.57 ms, 28k 7.45, 7.44, 7.47 ms; the 2k planes
@@ -1620,9 +1625,10 @@ __device__ void split_work(const SolveCfg* cfg, SolveSmem<DPS, NU>& sm, int tid,
   // lengthening the waits at their barriers, for a fifteenth more work per warp
   const int nw = TW < (long long)team.size * kWarps * kSpareWork ? kWarps - 1 : kWarps;
   const long long NW = (long long)team.size * nw;
-  const int nr = team.size <= kCompactTeamMax || TW < NW * kRangeFrom
-                     ? 1
-                     : (int)min((long long)kMaxRanges, TW / (NW * kRangeWork));
+  const long long share = TW / NW;
+  const bool small = team.size <= kSmallTeam;
+  const int nr = share < (small ? kSmallTeamFrom : kRangeFrom) ? 1
+                 : small ? 2 : (int)min((long long)kMaxRanges, share / kRangeWork);
   __syncthreads();
   // end h of the k-th piece of warp w on thread (k nw + w) 2 + h: the thread
   // whose run of groups holds it, by binary search, then the group
@@ -1656,6 +1662,7 @@ __device__ void split_work(const SolveCfg* cfg, SolveSmem<DPS, NU>& sm, int tid,
   if (tid == 0) {
     sm.b.n_range = nr;
     sm.b.n_workers = nw;
+    sm.b.compact = small || share >= kCompactWork ? 1 : 0;
   }
   __syncthreads();
   for (int k = 0; k < nr; ++k) {
@@ -1976,40 +1983,73 @@ __device__ __forceinline__ void range_groups(const WarpRange& r, int c, int j, i
   ghi = (c == r.c1 && j == r.j1) ? min(r.g1, G) : G;
 }
 
-// Segments of cluster c into the warp's shared arrays: first target index,
-// candidate offset (then tc) and filtered offset (then fc) of each segment.
+// The nseg segments of cluster c into the warp's shared arrays: first target
+// index, candidate offset (then tc) and filtered offset (then fc) of each segment.
 template <int DPS, int NU>
-__device__ __forceinline__ int load_segments(const SolveCfg* cfg, SolveSmem<DPS, NU>& sm, int warp,
-                                             int lane, int c, int tc, int fc) {
-  const int nseg = __ldcg(&cfg->cl_nseg[c]);
-  for (int i = lane; i < nseg; i += 32) {
-    sm.ws[warp].seg.xs[i] = __ldcg(&cfg->seg_xs[(size_t)c * kMaxSeg + i]);
-    sm.ws[warp].seg.pf[i] = __ldcg(&cfg->seg_pref[(size_t)c * kMaxSeg + i]);
-    sm.ws[warp].seg.fpf[i] = __ldcg(&cfg->seg_fpref[(size_t)c * kMaxSeg + i]);
+__device__ __forceinline__ void load_segments(const SolveCfg* cfg, SolveSmem<DPS, NU>& sm, int warp,
+                                              int lane, int c, int nseg, int tc, int fc) {
+  static_assert(kMaxSeg == 64, "two segments per lane");
+  const size_t at = (size_t)c * kMaxSeg + lane;
+  int v[2][3];
+#pragma unroll
+  for (int h = 0; h < 2; ++h) {
+    const bool have = lane + 32 * h < nseg;
+    v[h][0] = have ? __ldcg(&cfg->seg_xs[at + 32 * h]) : 0;
+    v[h][1] = have ? __ldcg(&cfg->seg_pref[at + 32 * h]) : 0;
+    v[h][2] = have ? __ldcg(&cfg->seg_fpref[at + 32 * h]) : 0;
+  }
+  WarpSeg& seg = sm.ws[warp].seg;
+#pragma unroll
+  for (int h = 0; h < 2; ++h) {
+    if (lane + 32 * h >= nseg) continue;
+    seg.xs[lane + 32 * h] = v[h][0];
+    seg.pf[lane + 32 * h] = v[h][1];
+    seg.fpf[lane + 32 * h] = v[h][2];
   }
   if (lane == 0) {
-    sm.ws[warp].seg.pf[nseg] = tc;
-    sm.ws[warp].seg.fpf[nseg] = fc;
+    seg.pf[nseg] = tc;
+    seg.fpf[nseg] = fc;
   }
   __syncwarp();
-  return nseg;
+}
+
+// Position of candidate q of the staged cluster (-1 beyond tc), advancing seg.
+template <int DPS, int NU>
+__device__ __forceinline__ int candidate_at(const SolveSmem<DPS, NU>& sm, int warp, int q, int tc,
+                                            int& seg) {
+  if (q >= tc) return -1;
+  const WarpSeg& sg = sm.ws[warp].seg;
+  while (sg.pf[seg + 1] <= q) ++seg;
+  return sg.xs[seg] + (q - sg.pf[seg]);
+}
+
+// Features of target point xi (zeros for -1).
+template <int DP, int DPS, bool FB>
+__device__ __forceinline__ void load_features(const GridView& g, int xi, float xf[DPS]) {
+#pragma unroll
+  for (int d = 0; d < DPS; ++d) xf[d] = 0.f;
+  if (xi < 0) return;
+#pragma unroll
+  for (int d = 0; d < DP; ++d) xf[d] = load_feat<FB>(g.feat, (size_t)d * g.n_pad + xi);
 }
 
 // Candidate q of the staged cluster (padding beyond tc), advancing seg.
 template <int DP, int DPS, int NU, bool FB>
 __device__ __forceinline__ float4 load_candidate(const GridView& g, SolveSmem<DPS, NU>& sm, int warp,
                                                  int q, int tc, int& seg, float xf[DPS]) {
-  float4 xp = make_float4(-kFar, -kFar, -kFar, 1.f);
-#pragma unroll
-  for (int d = 0; d < DPS; ++d) xf[d] = 0.f;
-  if (q < tc) {
-    while (sm.ws[warp].seg.pf[seg + 1] <= q) ++seg;
-    const int xi = sm.ws[warp].seg.xs[seg] + (q - sm.ws[warp].seg.pf[seg]);
-    xp = g.xyz[xi];
-#pragma unroll
-    for (int d = 0; d < DP; ++d) xf[d] = load_feat<FB>(g.feat, (size_t)d * g.n_pad + xi);
-  }
-  return xp;
+  const int xi = candidate_at<DPS, NU>(sm, warp, q, tc, seg);
+  load_features<DP, DPS, FB>(g, xi, xf);
+  return xi >= 0 ? g.xyz[xi] : make_float4(-kFar, -kFar, -kFar, 1.f);
+}
+
+// The same without its features, its position in place of w.
+template <int DPS, int NU>
+__device__ __forceinline__ float4 load_point(const GridView& g, const SolveSmem<DPS, NU>& sm, int warp,
+                                             int q, int tc, int& seg) {
+  const int xi = candidate_at<DPS, NU>(sm, warp, q, tc, seg);
+  float4 p = xi >= 0 ? g.xyz[xi] : make_float4(-kFar, -kFar, -kFar, 0.f);
+  p.w = __int_as_float(xi);
+  return p;
 }
 
 // Cursor over the filtered candidates of the cluster whose segments are
@@ -2076,14 +2116,13 @@ __device__ __forceinline__ void add_active(const SolveCfg* cfg, int c, int j, un
   }
 }
 
-// Stage cluster c for the warp from global memory (raw centred source points
-// and features, transformed by stage_cluster).
+// Stage the cluster of cs points from p0 on for the warp from global memory (raw
+// centred source points and features, transformed by stage_cluster), and its
+// segments, whose loads are issued with the points'.
 template <bool STEP, int DP, int MODE, int DPS, int NU>
-__device__ __forceinline__ int stage_from_global(const SolveCfg* cfg, SolveSmem<DPS, NU>& sm,
-                                                 const ClusterView& cv, int c, int warp,
-                                                 int lane) {
-  const int p0 = cv.cstart[c];
-  const int cs = cv.cstart[c + 1] - p0;
+__device__ __forceinline__ void stage_from_global(const SolveCfg* cfg, SolveSmem<DPS, NU>& sm, int c,
+                                                  int p0, int cs, int nseg, int tc, int fc, int warp,
+                                                  int lane) {
   const bool zv = lane < cs;
   float4 p = make_float4(0.f, 0.f, 0.f, 0.f);
   float pf[DPS];
@@ -2095,15 +2134,20 @@ __device__ __forceinline__ int stage_from_global(const SolveCfg* cfg, SolveSmem<
     for (int d = 0; d < DP; ++d)
       pf[d] = load_feat<bf16_of(MODE)>(cfg->src.feat, (size_t)d * cfg->src.m_pad + p0 + lane);
   }
+  load_segments<DPS, NU>(cfg, sm, warp, lane, c, nseg, tc, fc);
   stage_cluster<STEP, DP, DPS, NU>(sm, warp, lane, zv, p, pf, false);
-  return cs;
+  __syncwarp();
 }
 
 // One range of a warp's share of a pair pass, streamed from global memory (L2): lane
 // sums in acc, counts in nnz / cand. The filtered candidates of each chunk
-// are gathered through a ring of 64 entries in the warp's (otherwise unused)
-// cache region, with the next block of 32 candidates loading while the
-// current chunk runs.
+// are gathered through a ring of 64 entries (position and coordinates) in the
+// warp's (otherwise unused) cache region, with the next block of 32 candidates
+// loading while the current chunk runs; their features are read once they are
+// known to pass, ahead of the chunk's distance tests, which do not need them.
+// Lane l holds the numbers of cluster base + l, read 32 clusters at a time, so
+// that a cluster waits for one round trip to L2 (its points, segments and box)
+// instead of four.
 template <bool STEP, int DP, int MODE, int DPS, int NU>
 __device__ void pass_stream(const SolveCfg* cfg, SolveSmem<DPS, NU>& sm, int warp, int lane,
                             WarpRange r, float* ring, float acc[7], unsigned& nnz,
@@ -2115,18 +2159,27 @@ __device__ void pass_stream(const SolveCfg* cfg, SolveSmem<DPS, NU>& sm, int war
   const float rp2 = b.rplan_f * b.rplan_f;
   const bool collect = !STEP && b.collect_kept;
   float4* rxyz = reinterpret_cast<float4*>(ring);
-  float* rfeat = ring + 4 * 64;
-  for (int c = r.c0; c <= r.c1 && c < cv.ncl; ++c) {
-    const int tc = __ldcg(&cfg->cl_cand[c]);
-    const int fc = __ldcg(&cfg->cl_fcand[c]);
+  const int c_end = min(r.c1, cv.ncl - 1);
+  int l_tc = 0, l_fc = 0, l_p0 = 0, l_cs = 0, l_nseg = 0;
+  for (int c = r.c0; c <= c_end; ++c) {
+    const int li = (c - r.c0) & 31;
+    if (li == 0 && c + lane <= c_end) {
+      l_tc = __ldcg(&cfg->cl_cand[c + lane]);
+      l_fc = __ldcg(&cfg->cl_fcand[c + lane]);
+      l_nseg = __ldcg(&cfg->cl_nseg[c + lane]);
+      l_p0 = cv.cstart[c + lane];
+      l_cs = cv.cstart[c + lane + 1] - l_p0;
+    }
+    const int tc = __shfl_sync(kFull, l_tc, li), fc = __shfl_sync(kFull, l_fc, li);
     int jb, je;
     if (!range_chunks(r, c, (fc + 31) >> 5, jb, je)) continue;
-    __syncwarp();   // every lane is done with the previous cluster
-    const int cs = stage_from_global<STEP, DP, MODE, DPS, NU>(cfg, sm, cv, c, warp, lane);
+    const int cs = __shfl_sync(kFull, l_cs, li), nseg = __shfl_sync(kFull, l_nseg, li);
     const int cs4 = (cs + 3) & ~3;
-    const int nseg = load_segments<DPS, NU>(cfg, sm, warp, lane, c, tc, fc);
     const float4 lo = __ldcg(&cfg->cl_box[2 * (size_t)c]);
     const float4 hi = __ldcg(&cfg->cl_box[2 * (size_t)c + 1]);
+    __syncwarp();   // every lane is done with the previous cluster
+    stage_from_global<STEP, DP, MODE, DPS, NU>(cfg, sm, c, __shfl_sync(kFull, l_p0, li), cs, nseg, tc,
+                                               fc, warp, lane);
     FCursor cur = fcursor_at<DPS, NU>(sm, warp, nseg, jb * 32);
     const int want = min(fc, 32 * (je + 1)) - 32 * jb;
     const unsigned nnz0 = nnz;
@@ -2163,39 +2216,29 @@ __device__ void pass_stream(const SolveCfg* cfg, SolveSmem<DPS, NU>& sm, int war
         FCursor cf = fcursor_at<DPS, NU>(sm, warp, nseg, j0 * 32);
         cf.u = j0 * 32;
         cf.skip = 0;
-        float xfn[DPS];
-        float4 xpn = load_candidate<DP, DPS, NU, bf16_of(MODE)>(g, sm, warp, cf.u + lane, uend,
-                                                                cf.seg, xfn);
+        float4 xpn = load_point<DPS, NU>(g, sm, warp, cf.u + lane, uend, cf.seg);
         int used = 0;
         for (;;) {
           // place blocks of 32 until a chunk is full or the range is done (at
           // most 63 entries are unread, so the ring never overwrites one)
           while (cf.made - used < 32 && cf.u < uend) {
             const int o = fplace(cf, xpn, lo, hi, rp2, lane, uend);
-            if (o >= 0) {
-              const int e = o & 63;
-              rxyz[e] = xpn;
-#pragma unroll
-              for (int d = 0; d < DP; ++d) rfeat[d * 64 + e] = xfn[d];
-            }
-            if (cf.u < uend)
-              xpn = load_candidate<DP, DPS, NU, bf16_of(MODE)>(g, sm, warp, cf.u + lane, uend,
-                                                               cf.seg, xfn);
+            if (o >= 0) rxyz[o & 63] = xpn;
+            if (cf.u < uend) xpn = load_point<DPS, NU>(g, sm, warp, cf.u + lane, uend, cf.seg);
           }
           const int cnt = min(32, cf.made - used);
           if (cnt <= 0) break;
           __syncwarp();
           float4 xp = make_float4(-kFar, -kFar, -kFar, 1.f);
-          float xf[DPS];
-#pragma unroll
-          for (int d = 0; d < DPS; ++d) xf[d] = 0.f;
+          int xi = -1;
           if (lane < cnt) {
-            const int e = (used + lane) & 63;
-            xp = rxyz[e];
-#pragma unroll
-            for (int d = 0; d < DP; ++d) xf[d] = rfeat[d * 64 + e];
+            xp = rxyz[(used + lane) & 63];
+            xi = __float_as_int(xp.w);
+            xp.w = 0.f;
             cand += (unsigned)cs;
           }
+          float xf[DPS];
+          load_features<DP, DPS, bf16_of(MODE)>(g, xi, xf);
           __syncwarp();   // read before the next placement reuses the entries
           chunk_pairs<STEP, DP, MODE, DPS, NU>(sm, warp, xp, xf, 0, cs4, rc2, A, acc, nnz);
           used += cnt;
@@ -2233,9 +2276,7 @@ __device__ void pass_stream(const SolveCfg* cfg, SolveSmem<DPS, NU>& sm, int war
       if (collect) add_kept(cfg, c, nnz - nnz0, lane);
       continue;
     }
-    float xfn[DPS];
-    float4 xpn = load_candidate<DP, DPS, NU, bf16_of(MODE)>(g, sm, warp, cur.u + lane, tc,
-                                                            cur.seg, xfn);
+    float4 xpn = load_point<DPS, NU>(g, sm, warp, cur.u + lane, tc, cur.seg);
     int used = 0;
     for (int j = jb; j <= je; ++j) {
       const int cnt = min(32, want - used);
@@ -2243,28 +2284,20 @@ __device__ void pass_stream(const SolveCfg* cfg, SolveSmem<DPS, NU>& sm, int war
       // unread, so the ring never overwrites one)
       while (cur.made - used < cnt && cur.u < tc) {
         const int o = fplace(cur, xpn, lo, hi, rp2, lane, tc);
-        if (o >= 0) {
-          const int e = o & 63;
-          rxyz[e] = xpn;
-#pragma unroll
-          for (int d = 0; d < DP; ++d) rfeat[d * 64 + e] = xfn[d];
-        }
-        if (cur.u < tc)
-          xpn = load_candidate<DP, DPS, NU, bf16_of(MODE)>(g, sm, warp, cur.u + lane, tc, cur.seg,
-                                                           xfn);
+        if (o >= 0) rxyz[o & 63] = xpn;
+        if (cur.u < tc) xpn = load_point<DPS, NU>(g, sm, warp, cur.u + lane, tc, cur.seg);
       }
       __syncwarp();
       float4 xp = make_float4(-kFar, -kFar, -kFar, 1.f);
-      float xf[DPS];
-#pragma unroll
-      for (int d = 0; d < DPS; ++d) xf[d] = 0.f;
+      int xi = -1;
       const bool have = lane < cnt && used + lane < cur.made;
       if (have) {
-        const int e = (used + lane) & 63;
-        xp = rxyz[e];
-#pragma unroll
-        for (int d = 0; d < DP; ++d) xf[d] = rfeat[d * 64 + e];
+        xp = rxyz[(used + lane) & 63];
+        xi = __float_as_int(xp.w);
+        xp.w = 0.f;
       }
+      float xf[DPS];
+      load_features<DP, DPS, bf16_of(MODE)>(g, xi, xf);
       __syncwarp();   // read before the next placement reuses the entries
       int glo, ghi;
       range_groups(r, c, j, cs4 >> 2, glo, ghi);
@@ -2293,8 +2326,9 @@ __device__ void pass_stream(const SolveCfg* cfg, SolveSmem<DPS, NU>& sm, int war
 // << 10). Filled once per plan, so that the passes of every iteration that reuses
 // the plan (at the lengthscale floor, most of the solve) read no global memory. A
 // share of a reused plan that is too large is cached as far as it goes, with the
-// first two slots left to the streamed pass for the rest of it (BlockCtx::rest).
+// front left to the streamed pass's ring for the rest of it (BlockCtx::rest_c).
 constexpr int kCacheSlots = 32;                 // items per warp
+constexpr int kRingFloats = 4 * 64;             // the streamed passes' ring
 constexpr unsigned short kSlotCluster = 0x8000;
 constexpr unsigned short kSlotList = 0x4000;      // cluster whose pairs are listed
 
@@ -2400,8 +2434,8 @@ __device__ void fill_cache(const SolveCfg* cfg, SolveSmem<DPS, NU>& sm, int warp
     return;
   }
   float* base = cache + (size_t)warp * cap;
-  if (part) base += 2 * slot_floats<DP>();
-  int room = part ? cap - 2 * slot_floats<DP>() : cap;
+  if (part) base += kRingFloats;
+  int room = part ? cap - kRingFloats : cap;
   int n = 0, k = 0, coff = room;   // items, chunk slots, where the clusters begin
   int rest_c = -1, rest_j = 0, rest_g = 0;
   for (int c = r.c0; c <= r.c1 && c < cv.ncl && rest_c < 0; ++c) {
@@ -2438,7 +2472,8 @@ __device__ void fill_cache(const SolveCfg* cfg, SolveSmem<DPS, NU>& sm, int warp
       sm.cache_cl[warp][n] = c;
     }
     ++n;
-    const int nseg = load_segments<DPS, NU>(cfg, sm, warp, lane, c, tc, fc);
+    const int nseg = __ldcg(&cfg->cl_nseg[c]);
+    load_segments<DPS, NU>(cfg, sm, warp, lane, c, nseg, tc, fc);
     float4 lo = __ldcg(&cfg->cl_box[2 * (size_t)c]);
     float4 hi = __ldcg(&cfg->cl_box[2 * (size_t)c + 1]);
     if (lo.w == 0.f) {   // not filtered by the plan: every candidate of the range is cached
@@ -2608,9 +2643,9 @@ __device__ void pass_cached(const SolveCfg* cfg, SolveSmem<DPS, NU>& sm, int war
   const float rc2 = sm.b.ic.rc2, A = sm.b.ic.A;
   const bool collect = !STEP && sm.b.collect_kept;
   const float* base = cache + (size_t)warp * cap;
-  if (sm.b.rest_c[warp] >= 0) {   // the streamed rest has the first two slots
-    base += 2 * slot_floats<DP>();
-    cap -= 2 * slot_floats<DP>();
+  if (sm.b.rest_c[warp] >= 0) {   // the front is the ring of the streamed rest
+    base += kRingFloats;
+    cap -= kRingFloats;
   }
   const unsigned short* pl = sm.ws[warp].list;
   const int n = sm.cache_n[warp];
@@ -2822,7 +2857,6 @@ __device__ void solve_pair(const SolveCfg* __restrict__ cfg, SolveState* __restr
     b.done = cfg->max_iters <= 0 ? 1 : 0;
     b.converged = b.fallback = b.no_ascent = b.have_t_prev = 0;
     b.use_kept = b.collect_kept = b.rebalance = b.use_act = 0;
-    b.compact = team.size <= kCompactTeamMax ? 1 : 0;
     b.t = b.t_prev = 0.0;
     b.pending = 0;
     b.nnz_total = b.cand_total = b.nnz_grad = b.cand_grad = 0;
@@ -3125,8 +3159,7 @@ const CacheCfg& cache_cfg() {
     const int slot = 32 * (4 + DP);   // slot_floats
     const int avail = smem_sm / CVO_SOLVE_MIN_BLOCKS - reserved - (int)fa.sharedSizeBytes;
     c.cap = std::max(0, std::min(kCacheSlots * slot, avail / kWarps / 64 * 16));
-    // the streamed passes gather candidates through 64 entries of each warp
-    if (c.cap < 2 * slot) {
+    if (c.cap < kRingFloats) {
       c.err = cudaErrorInvalidConfiguration;
       return c;
     }
