@@ -92,9 +92,8 @@ void free_grid(cvo_ctx* ctx, Grid& g) {
 }
 
 void free_plan_buffers(cvo_ctx* ctx, Plan* p) {
-  dev_free(ctx, p->d_cfg);
-  dev_free(ctx, p->d_iters);
-  dev_free(ctx, p->d_state);
+  if (p->d_iters != (p->d_in ? &p->d_in->first : nullptr)) dev_free(ctx, p->d_iters);
+  dev_free(ctx, p->d_in);
   dev_free(ctx, p->d_partials);
   dev_free(ctx, p->d_records);
   dev_free(ctx, p->seg_xs);
@@ -109,6 +108,7 @@ void free_plan_buffers(cvo_ctx* ctx, Plan* p) {
   dev_free(ctx, p->cl_act);
   dev_free(ctx, p->group_agg);
   release_bytes(ctx, p->bytes);
+  p->d_in = nullptr;
   p->d_cfg = nullptr;
   p->d_iters = nullptr;
   p->d_state = nullptr;
@@ -279,9 +279,13 @@ int reserve_plan(cvo_ctx* ctx, Plan* p, int iters, int ncl, int nblocks) {
   iters = std::max(iters, 1);
   ncl = std::max(ncl, 1);
   const int ng = (ncl + 31) / 32;
-  int rc = dev_alloc(ctx, (void**)&p->d_cfg, sizeof(SolveCfg), &p->bytes);
-  if (rc == CVO_OK) rc = dev_alloc(ctx, (void**)&p->d_iters, sizeof(IterConst) * iters, &p->bytes);
-  if (rc == CVO_OK) rc = dev_alloc(ctx, (void**)&p->d_state, sizeof(SolveState), &p->bytes);
+  int rc = dev_alloc(ctx, (void**)&p->d_in, sizeof(SolveInputs), &p->bytes);
+  if (rc == CVO_OK) {
+    p->d_state = &p->d_in->state;
+    p->d_cfg = &p->d_in->cfg;
+    if (iters == 1) p->d_iters = &p->d_in->first;
+    else rc = dev_alloc(ctx, (void**)&p->d_iters, sizeof(IterConst) * iters, &p->bytes);
+  }
   if (rc == CVO_OK)
     rc = dev_alloc(ctx, (void**)&p->d_partials, sizeof(double) * 2 * kPartialStride * nblocks,
                    &p->bytes);
@@ -416,14 +420,20 @@ int configure_plan(cvo_ctx* ctx, Plan* p, Cloud* t, Cloud* s, const std::vector<
   cfg.wait_polls = (unsigned)prm.wait_polls;
   cfg.join_limit_ns = (unsigned long long)(prm.join_limit_ms * 1e6);
   cfg.mode = mode;
-  // pageable sources: the copies complete before the calls return
-  CK(cudaMemcpyAsync(p->d_iters, ic.data(), sizeof(IterConst) * ic.size(), cudaMemcpyHostToDevice,
-                     ctx->stream));
-  CK(cudaMemcpyAsync(p->d_cfg, &cfg, sizeof(SolveCfg), cudaMemcpyHostToDevice, ctx->stream));
   p->h_cfg = cfg;
   p->n_iters = (int)ells.size();
   p->dp = s->dp;
   p->color_mode = kernel_mode(prm);
+  p->staged = mode == kModeEval && p->d_iters == &p->d_in->first;
+  if (p->staged) {   // run_solve sends them up with the state
+    ctx->h_stage->cfg = cfg;
+    ctx->h_stage->first = ic[0];
+    return CVO_OK;
+  }
+  // pageable sources: the copies complete before the calls return
+  CK(cudaMemcpyAsync(p->d_iters, ic.data(), sizeof(IterConst) * ic.size(), cudaMemcpyHostToDevice,
+                     ctx->stream));
+  CK(cudaMemcpyAsync(p->d_cfg, &cfg, sizeof(SolveCfg), cudaMemcpyHostToDevice, ctx->stream));
   return CVO_OK;
 }
 
@@ -445,15 +455,21 @@ int build_plan(cvo_ctx* ctx, int tgt, int src, Plan** out) {
 }
 
 // Stage P0 (and a zeroed state, which also resets the grid barrier) and run
-// the solve kernel.
+// the solve kernel: one copy up (an evaluation's configuration goes with the
+// state), the launch, and a wait; the kernel writes its result to the pinned
+// h_state itself. (Three copies up, two of them pageable, and one down took a
+// quarter of a 2k-point evaluation.)
 int run_solve(cvo_ctx* ctx, Plan* p, const double P0[16], bool records) {
   SolveState* hs = ctx->h_state;
+  SolveInputs* in = ctx->h_stage;
   std::memset(hs, 0, sizeof(SolveState));
-  std::memcpy(hs->P0, P0, sizeof(double) * 16);
-  CK(cudaMemcpyAsync(p->d_state, hs, sizeof(SolveState), cudaMemcpyHostToDevice, ctx->stream));
+  std::memset(&in->state, 0, sizeof(SolveState));
+  std::memcpy(in->state.P0, P0, sizeof(double) * 16);
+  in->state.host = ctx->d_result;
+  CK(cudaMemcpyAsync(p->d_in, in, p->staged ? sizeof(SolveInputs) : sizeof(SolveState),
+                     cudaMemcpyHostToDevice, ctx->stream));
   CK(launch_solve(p->dp, p->color_mode, p->nblocks, p->d_cfg, p->d_state, p->d_partials,
                   records ? p->d_records : nullptr, ctx->stream));
-  CK(cudaMemcpyAsync(hs, p->d_state, sizeof(SolveState), cudaMemcpyDeviceToHost, ctx->stream));
   CK(cudaStreamSynchronize(ctx->stream));
   if (hs->status & kStatusTimeout) return fail(ctx, CVO_ERR_TIMEOUT, "grid barrier timed out");
   if (hs->status != 0) return fail(ctx, CVO_ERR_INTERNAL, "cell-row segment overflow");
@@ -664,7 +680,9 @@ int cvo_create(const cvo_params* params, int device, size_t hbm_budget_bytes, cv
   if (p.feat_dim == 0) ctx->prm.color_mode = CVO_COLOR_NONE;
   ctx->budget = hbm_budget_bytes;
   if (cudaStreamCreateWithFlags(&ctx->stream, cudaStreamNonBlocking) != cudaSuccess ||
-      cudaMallocHost((void**)&ctx->h_state, sizeof(SolveState)) != cudaSuccess ||
+      cudaHostAlloc((void**)&ctx->h_state, sizeof(SolveState), cudaHostAllocMapped) != cudaSuccess ||
+      cudaHostGetDevicePointer((void**)&ctx->d_result, ctx->h_state, 0) != cudaSuccess ||
+      cudaMallocHost((void**)&ctx->h_stage, sizeof(SolveInputs)) != cudaSuccess ||
       cudaMallocHost((void**)&ctx->h_stats, sizeof(CloudStats)) != cudaSuccess ||
       cudaMallocHost((void**)&ctx->h_int, sizeof(int) * 2 * kMaxLevels) != cudaSuccess ||
       cudaMalloc((void**)&ctx->d_stats, sizeof(CloudStats)) != cudaSuccess ||
@@ -705,6 +723,7 @@ int cvo_destroy(cvo_ctx* ctx) {
   if (ctx->h_stats) cudaFreeHost(ctx->h_stats);
   if (ctx->h_int) cudaFreeHost(ctx->h_int);
   if (ctx->h_state) cudaFreeHost(ctx->h_state);
+  if (ctx->h_stage) cudaFreeHost(ctx->h_stage);
   if (ctx->stream) cudaStreamSynchronize(ctx->stream);   // stream-ordered frees complete
   if (ctx->pool) cudaMemPoolDestroy(ctx->pool);
   if (ctx->stream) cudaStreamDestroy(ctx->stream);

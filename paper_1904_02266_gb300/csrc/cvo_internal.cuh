@@ -146,6 +146,8 @@ struct SolveState {
   unsigned int join_count, leave_count;     // queued solves: blocks of the team that have started
                                             // and that are done with the entry
   unsigned long long t_begin_ns, t_end_ns;  // global timer at the start and end of the solve
+  SolveState* host;                         // device address of the host's pinned copy that the
+                                            // result is written to, or NULL: it stays here
 };
 
 // Per-iteration record of a profiled solve (device timestamps).

@@ -1003,6 +1003,12 @@ __device__ __forceinline__ unsigned barrier_arrive_count(SolveState* st) {
   return old;
 }
 
+// An error bit of the solve, also where the host reads its result from.
+__device__ __forceinline__ void raise_status(SolveState* st, int bits) {
+  atomicOr(&st->status, bits);
+  if (st->host) atomicOr_system(&st->host->status, bits);
+}
+
 // Wait until `target` arrivals (thread 0). A block that polls `limit` times
 // raises kStatusTimeout and returns false; its team then leaves the solve loop
 // when the other blocks' own waits run out at the next barrier, which the
@@ -1011,7 +1017,7 @@ __device__ __forceinline__ bool barrier_wait(SolveState* st, unsigned target, un
   unsigned spins = 0;
   while (ld_acquire(&st->bar_count) < target) {
     if (++spins > limit) {
-      atomicOr(&st->status, (int)kStatusTimeout);
+      raise_status(st, (int)kStatusTimeout);
       return false;
     }
     // the first polls follow one another: most waits end within them, and a sleep
@@ -1187,7 +1193,7 @@ __device__ bool team_join(SolveState* st, int team_size, Smem& sm) {
     while (ld_acquire(&st->join_count) < (unsigned)team_size) {
       if ((++polls & 255u) == 0 && globaltimer() - t_start > sm.b.tc.join_limit_ns) {
         ok = 0;
-        atomicOr(&st->status, (int)kStatusTimeout);
+        raise_status(st, (int)kStatusTimeout);
         break;
       }
       __nanosleep(256);
@@ -1309,7 +1315,7 @@ __device__ void plan_cluster(const SolveCfg* cfg, const BlockCtx& b, SolveState*
     nseg += __popc(m);
     total += __shfl_sync(kFull, incl, 31);
   }
-  if (__any_sync(kFull, overflow) && lane == 0) atomicOr(&st->status, (int)kStatusSegOverflow);
+  if (__any_sync(kFull, overflow) && lane == 0) raise_status(st, (int)kStatusSegOverflow);
   nseg = min(nseg, kMaxSeg);
   if (lane == 0) s_pf[nseg] = total;
   for (int i = lane; i < nseg; i += 32) s_cnt[i] = 0;
@@ -2788,8 +2794,7 @@ __device__ void run_pass(const SolveCfg* cfg, SolveSmem<DPS, NU>& sm, double* pa
   }
 }
 
-__device__ void publish(SolveState* st, BlockCtx& b) {
-  form_step_sums(b);
+__device__ void publish(SolveState* st, const BlockCtx& b) {
   for (int i = 0; i < 16; ++i) st->P[i] = b.P[i];
   for (int i = 0; i < 6; ++i) st->xi[i] = b.xi[i];
   for (int i = 0; i < 5; ++i) st->S[i] = b.S[i];
@@ -2991,8 +2996,12 @@ __device__ void solve_pair(const SolveCfg* __restrict__ cfg, SolveState* __restr
     __syncthreads();
   }
   if (team.rank == 0 && tid == 0) {
-    publish(st, sm.b);
-    st->t_end_ns = globaltimer();
+    form_step_sums(sm.b);
+    // a single solve's result goes straight to the host's pinned copy
+    SolveState* out = st->host ? st->host : st;
+    publish(out, sm.b);
+    out->t_begin_ns = st->t_begin_ns;
+    out->t_end_ns = globaltimer();
   }
   __syncthreads();
 }

@@ -55,12 +55,22 @@ struct Cloud {
   int refs = 0;           // batches that use the cloud
 };
 
+// Inputs of a solve in one device block and one pinned block of the same layout:
+// the state, the configuration and (an evaluation's) first iteration constants.
+struct SolveInputs {
+  SolveState state;
+  alignas(16) SolveCfg cfg;
+  alignas(16) IterConst first;
+};
+
 struct Plan {
   int tgt = -1, src = -1;
   SolveCfg h_cfg{};
+  SolveInputs* d_in = nullptr;   // holds d_state, d_cfg and, for one iteration, d_iters
   SolveCfg* d_cfg = nullptr;
   IterConst* d_iters = nullptr;
   SolveState* d_state = nullptr;
+  bool staged = false;           // cfg and the one iteration go up with the state (cvo_eval)
   double* d_partials = nullptr;
   IterRecord* d_records = nullptr;
   int* seg_xs = nullptr;
@@ -121,7 +131,9 @@ struct cvo_ctx {
   std::map<std::pair<int, int>, cvo::Plan*> plans;
   std::vector<cvo_batch*> batches;
   cvo::Plan* eval_plan = nullptr;      // reused by cvo_eval
-  cvo::SolveState* h_state = nullptr;  // pinned
+  cvo::SolveState* h_state = nullptr;  // pinned: a solve's result
+  cvo::SolveState* d_result = nullptr; // its device address
+  cvo::SolveInputs* h_stage = nullptr; // pinned: a solve's inputs, one copy up
   cvo::CloudStats* d_stats = nullptr;
   cvo::CloudStats* h_stats = nullptr;  // pinned
   int* h_int = nullptr;           // pinned scratch for small read-backs
