@@ -250,6 +250,7 @@ struct BlockCtx {
   int w_c1[kMaxRanges][kWarps], w_j1[kMaxRanges][kWarps], w_g1[kMaxRanges][kWarps];
   // where the streamed rest of a partly cached share begins (c < 0: there is none)
   int rest_c[kWarps], rest_j[kWarps], rest_g[kWarps];
+  int ring_floats;        // front of a warp's cache region that the streamed passes use
   double dR[9], V[9];     // tail scratch: exp map rotation and its V matrix
 };
 
@@ -1822,42 +1823,99 @@ __device__ __forceinline__ StepVectors step_vectors(const BlockCtx& b, float x, 
 // its beta, whose fourth power would be the first of its step terms to
 // overflow). Testing all groups first keeps the chain of loads, test, vote and
 // branch out of the bodies, which repeat the test's six packed FMAs instead.
-template <bool STEP, int DP, int MODE, int DPS, int NU>
-__device__ __forceinline__ unsigned chunk_pairs(SolveSmem<DPS, NU>& sm, int warp, float4 xp,
-                                                const float xf[DPS], int jlo, int jhi, float rc2,
-                                                float A, float acc[7], unsigned& nnz) {
-  const float4 o = sm.zo[warp];
-  const float xl = xp.x - o.x, yl = xp.y - o.y, zl = xp.z - o.z;
-  const float x2 = fmaf(xl, xl, fmaf(yl, yl, zl * zl));
-  const float thr = rc2 - x2;   // about -3e36 for a padding candidate: never kept
-  const f32x2 X = dup2(xl), Y = dup2(yl), Z = dup2(zl);
+// A candidate against the cluster staged for the warp.
+struct ChunkLane {
+  f32x2 X, Y, Z;          // x_l
+  float xl, yl, zl, x2, thr;
+};
+
+__device__ __forceinline__ ChunkLane chunk_lane(float4 xp, float4 o, float rc2) {
+  ChunkLane k;
+  k.xl = xp.x - o.x;
+  k.yl = xp.y - o.y;
+  k.zl = xp.z - o.z;
+  k.x2 = fmaf(k.xl, k.xl, fmaf(k.yl, k.yl, k.zl * k.zl));
+  k.thr = rc2 - k.x2;   // about -3e36 for a padding candidate: never kept
+  k.X = dup2(k.xl);
+  k.Y = dup2(k.yl);
+  k.Z = dup2(k.zl);
+  return k;
+}
+
+// Four staged source points as planes, two packed pairs.
+struct SourceGroup {
+  ulonglong2 x, y, z, w;
+};
+
+__device__ __forceinline__ SourceGroup source_group(const float* pl, int j0) {
+  SourceGroup g;
+  g.x = *reinterpret_cast<const ulonglong2*>(pl + j0);
+  g.y = *reinterpret_cast<const ulonglong2*>(pl + kClusterMax + j0);
+  g.z = *reinterpret_cast<const ulonglong2*>(pl + 2 * kClusterMax + j0);
+  g.w = *reinterpret_cast<const ulonglong2*>(pl + 3 * kClusterMax + j0);
+  return g;
+}
+
+__device__ __forceinline__ void group_tests(const SourceGroup& g, const ChunkLane& k, f32x2 t[2]) {
+  t[0] = fma2(k.X, g.x.x, fma2(k.Y, g.y.x, fma2(k.Z, g.z.x, g.w.x)));
+  t[1] = fma2(k.X, g.x.y, fma2(k.Y, g.y.y, fma2(k.Z, g.z.y, g.w.y)));
+}
+
+// The lane keeps one of the group's four pairs.
+__device__ __forceinline__ bool group_kept(const SourceGroup& g, const ChunkLane& k) {
+  f32x2 t[2];
+  group_tests(g, k, t);
+  float t0, t1, t2, t3;
+  unpack2(t[0], t0, t1);
+  unpack2(t[1], t2, t3);
+  return fminf(fminf(t0, t1), fminf(t2, t3)) <= k.thr;
+}
+
+// The source groups in [jlo, jhi) of which any lane keeps a pair with its candidate
+// (bit g: group g), the same in every lane.
+template <int DPS, int NU>
+__device__ __forceinline__ unsigned chunk_groups(const SolveSmem<DPS, NU>& sm, int warp,
+                                                 const ChunkLane& k, int jlo, int jhi) {
   const float* pl = reinterpret_cast<const float*>(sm.z[warp]);
-  struct Group {
-    ulonglong2 x, y, z;
-    f32x2 t[2];
-  };
-  const auto test = [&](int j0) {
-    Group g;
-    g.x = *reinterpret_cast<const ulonglong2*>(pl + j0);
-    g.y = *reinterpret_cast<const ulonglong2*>(pl + kClusterMax + j0);
-    g.z = *reinterpret_cast<const ulonglong2*>(pl + 2 * kClusterMax + j0);
-    const ulonglong2 w = *reinterpret_cast<const ulonglong2*>(pl + 3 * kClusterMax + j0);
-    g.t[0] = fma2(X, g.x.x, fma2(Y, g.y.x, fma2(Z, g.z.x, w.x)));
-    g.t[1] = fma2(X, g.x.y, fma2(Y, g.y.y, fma2(Z, g.z.y, w.y)));
-    return g;
-  };
   unsigned mine = 0u;
 #pragma unroll 2
-  for (int j0 = jlo; j0 < jhi; j0 += 4) {
-    const Group g = test(j0);
-    float t0, t1, t2, t3;
-    unpack2(g.t[0], t0, t1);
-    unpack2(g.t[1], t2, t3);
-    if (fminf(fminf(t0, t1), fminf(t2, t3)) <= thr) mine |= 1u << (j0 >> 2);
+  for (int j0 = jlo; j0 < jhi; j0 += 4)
+    if (group_kept(source_group(pl, j0), k)) mine |= 1u << (j0 >> 2);
+  return __reduce_or_sync(kFull, mine);
+}
+
+// The same for two chunks at once over all groups: the tests are bound by their
+// 16-byte broadcast loads (eight cycles of a scheduler each with all four
+// loading), which two candidates share. Queued solves only (TWO): their passes are
+// mostly these chunks (64-pair batch 103.9 -> 102.2 ms, 16 served requests 95.7 ->
+// 94.5); in single solves the registers it takes cost the cached floor passes more
+// (2k pair 819 -> 847 us, 20k 5.49 -> 5.54 ms) than large shares gain (100k 45.3 ->
+// 44.2 ms).
+template <int DPS, int NU>
+__device__ __forceinline__ void chunk_groups2(const SolveSmem<DPS, NU>& sm, int warp, float4 xa,
+                                              float4 xb, int jhi, float rc2, unsigned active[2]) {
+  const ChunkLane ka = chunk_lane(xa, sm.zo[warp], rc2), kb = chunk_lane(xb, sm.zo[warp], rc2);
+  const float* pl = reinterpret_cast<const float*>(sm.z[warp]);
+  unsigned ma = 0u, mb = 0u;
+#pragma unroll 2
+  for (int j0 = 0; j0 < jhi; j0 += 4) {
+    const SourceGroup g = source_group(pl, j0);
+    if (group_kept(g, ka)) ma |= 1u << (j0 >> 2);
+    if (group_kept(g, kb)) mb |= 1u << (j0 >> 2);
   }
-  // bit g: source group g kept a pair (the same in every lane)
-  const unsigned active = __reduce_or_sync(kFull, mine);
-  if (active == 0u) return 0u;
+  active[0] = __reduce_or_sync(kFull, ma);
+  active[1] = __reduce_or_sync(kFull, mb);
+}
+
+// The pair bodies of a chunk's active groups.
+template <bool STEP, int DP, int MODE, int DPS, int NU>
+__device__ __forceinline__ void chunk_bodies(SolveSmem<DPS, NU>& sm, int warp, float4 xp,
+                                             const ChunkLane& lane_k, const float xf[DPS],
+                                             unsigned active, float A, float acc[7],
+                                             unsigned& nnz) {
+  if (active == 0u) return;
+  const float xl = lane_k.xl, yl = lane_k.yl, zl = lane_k.zl, x2 = lane_k.x2, thr = lane_k.thr;
+  const float* pl = reinterpret_cast<const float*>(sm.z[warp]);
   const f32x2 q0 = dup2(A * x2), A2 = dup2(A);
   f32x2 F[DPS];
 #pragma unroll
@@ -1877,7 +1935,9 @@ __device__ __forceinline__ unsigned chunk_pairs(SolveSmem<DPS, NU>& sm, int warp
   f32x2 s[5] = {0ull, 0ull, 0ull, 0ull, 0ull};
   for (unsigned rem = active; rem != 0u; rem &= rem - 1u) {
     const int j0 = 4 * (__ffs(rem) - 1);
-    const Group g = test(j0);
+    const SourceGroup g = source_group(pl, j0);
+    f32x2 t[2];
+    group_tests(g, lane_k, t);
     f32x2 q[2] = {q0, q0};
     f32x2 cdot[2] = {0ull, 0ull};
 #pragma unroll
@@ -1898,9 +1958,9 @@ __device__ __forceinline__ unsigned chunk_pairs(SolveSmem<DPS, NU>& sm, int warp
     for (int h = 0; h < 2; ++h) {
       const f32x2 mx = h ? g.x.y : g.x.x, my = h ? g.y.y : g.y.x, mz = h ? g.z.y : g.z.x;
       float t0, t1, e0, e1, w0, w1;
-      unpack2(g.t[h], t0, t1);
+      unpack2(t[h], t0, t1);
       const bool k0 = t0 <= thr, k1 = t1 <= thr;
-      unpack2(fma2(A2, g.t[h], q[h]), e0, e1);
+      unpack2(fma2(A2, t[h], q[h]), e0, e1);
       w0 = ex2_approx(-e0);
       w1 = ex2_approx(-e1);
       if (color_of(MODE) == kColorDot) {
@@ -1960,6 +2020,16 @@ __device__ __forceinline__ unsigned chunk_pairs(SolveSmem<DPS, NU>& sm, int warp
     acc[3] = fmaf(4.0f, sum2(s[3]), acc[3]);
     acc[4] = fmaf(2.0f, sum2(s[4]), acc[4]);
   }
+}
+
+// One chunk against source points [jlo, jhi); returns its active groups.
+template <bool STEP, int DP, int MODE, int DPS, int NU>
+__device__ __forceinline__ unsigned chunk_pairs(SolveSmem<DPS, NU>& sm, int warp, float4 xp,
+                                                const float xf[DPS], int jlo, int jhi, float rc2,
+                                                float A, float acc[7], unsigned& nnz) {
+  const ChunkLane k = chunk_lane(xp, sm.zo[warp], rc2);
+  const unsigned active = chunk_groups<DPS, NU>(sm, warp, k, jlo, jhi);
+  chunk_bodies<STEP, DP, MODE, DPS, NU>(sm, warp, xp, k, xf, active, A, acc, nnz);
   return active;
 }
 
@@ -2145,16 +2215,22 @@ __device__ __forceinline__ void stage_from_global(const SolveCfg* cfg, SolveSmem
   __syncwarp();
 }
 
+// Entries of the streamed passes' ring (a power of two), float4 each.
+template <bool TWO>
+__host__ __device__ constexpr int ring_size() {
+  return TWO ? 128 : 64;
+}
+
 // One range of a warp's share of a pair pass, streamed from global memory (L2): lane
 // sums in acc, counts in nnz / cand. The filtered candidates of each chunk
-// are gathered through a ring of 64 entries (position and coordinates) in the
+// are gathered through a ring of entries (position and coordinates) in the
 // warp's (otherwise unused) cache region, with the next block of 32 candidates
 // loading while the current chunk runs; their features are read once they are
 // known to pass, ahead of the chunk's distance tests, which do not need them.
 // Lane l holds the numbers of cluster base + l, read 32 clusters at a time, so
 // that a cluster waits for one round trip to L2 (its points, segments and box)
 // instead of four.
-template <bool STEP, int DP, int MODE, int DPS, int NU>
+template <bool STEP, int DP, int MODE, int DPS, int NU, bool TWO>
 __device__ void pass_stream(const SolveCfg* cfg, SolveSmem<DPS, NU>& sm, int warp, int lane,
                             WarpRange r, float* ring, float acc[7], unsigned& nnz,
                             unsigned& cand) {
@@ -2164,6 +2240,7 @@ __device__ void pass_stream(const SolveCfg* cfg, SolveSmem<DPS, NU>& sm, int war
   const float rc2 = b.ic.rc2, A = b.ic.A;
   const float rp2 = b.rplan_f * b.rplan_f;
   const bool collect = !STEP && b.collect_kept;
+  constexpr int kRing = ring_size<TWO>();
   float4* rxyz = reinterpret_cast<float4*>(ring);
   const int c_end = min(r.c1, cv.ncl - 1);
   int l_tc = 0, l_fc = 0, l_p0 = 0, l_cs = 0, l_nseg = 0;
@@ -2224,29 +2301,53 @@ __device__ void pass_stream(const SolveCfg* cfg, SolveSmem<DPS, NU>& sm, int war
         cf.skip = 0;
         float4 xpn = load_point<DPS, NU>(g, sm, warp, cf.u + lane, uend, cf.seg);
         int used = 0;
+        constexpr int kTake = TWO ? 64 : 32;   // candidates taken at a time
         for (;;) {
-          // place blocks of 32 until a chunk is full or the range is done (at
-          // most 63 entries are unread, so the ring never overwrites one)
-          while (cf.made - used < 32 && cf.u < uend) {
+          // place blocks of 32 until those are there or the range is done (at
+          // most kTake + 31 entries are unread, so the ring never overwrites one)
+          while (cf.made - used < kTake && cf.u < uend) {
             const int o = fplace(cf, xpn, lo, hi, rp2, lane, uend);
-            if (o >= 0) rxyz[o & 63] = xpn;
+            if (o >= 0) rxyz[o & (kRing - 1)] = xpn;
             if (cf.u < uend) xpn = load_point<DPS, NU>(g, sm, warp, cf.u + lane, uend, cf.seg);
           }
-          const int cnt = min(32, cf.made - used);
+          const int cnt = min(kTake, cf.made - used);
           if (cnt <= 0) break;
           __syncwarp();
-          float4 xp = make_float4(-kFar, -kFar, -kFar, 1.f);
-          int xi = -1;
-          if (lane < cnt) {
-            xp = rxyz[(used + lane) & 63];
-            xi = __float_as_int(xp.w);
-            xp.w = 0.f;
-            cand += (unsigned)cs;
-          }
+          // this lane's candidate of the first (h = 0) or second chunk
+          const auto take = [&](int h, int& xi) {
+            float4 xp = make_float4(-kFar, -kFar, -kFar, 1.f);
+            xi = -1;
+            if (lane + 32 * h < cnt) {
+              xp = rxyz[(used + 32 * h + lane) & (kRing - 1)];
+              xi = __float_as_int(xp.w);
+              xp.w = 0.f;
+            }
+            return xp;
+          };
+          int xi;
           float xf[DPS];
-          load_features<DP, DPS, bf16_of(MODE)>(g, xi, xf);
+          if constexpr (TWO) {
+            const float4 xb = take(1, xi);
+            float4 xp = take(0, xi);
+            load_features<DP, DPS, bf16_of(MODE)>(g, xi, xf);
+            unsigned active[2];
+            chunk_groups2<DPS, NU>(sm, warp, xp, xb, cs4, rc2, active);
+            cand += (unsigned)cs * ((lane < cnt ? 1u : 0u) + (lane + 32 < cnt ? 1u : 0u));
+            for (int h = 0; h < 2; ++h) {
+              chunk_bodies<STEP, DP, MODE, DPS, NU>(sm, warp, xp, chunk_lane(xp, sm.zo[warp], rc2),
+                                                    xf, active[0], A, acc, nnz);
+              if (h == 1 || active[1] == 0u) break;
+              active[0] = active[1];
+              xp = take(1, xi);
+              load_features<DP, DPS, bf16_of(MODE)>(g, xi, xf);
+            }
+          } else {
+            const float4 xp = take(0, xi);
+            load_features<DP, DPS, bf16_of(MODE)>(g, xi, xf);
+            cand += lane < cnt ? (unsigned)cs : 0u;
+            chunk_pairs<STEP, DP, MODE, DPS, NU>(sm, warp, xp, xf, 0, cs4, rc2, A, acc, nnz);
+          }
           __syncwarp();   // read before the next placement reuses the entries
-          chunk_pairs<STEP, DP, MODE, DPS, NU>(sm, warp, xp, xf, 0, cs4, rc2, A, acc, nnz);
           used += cnt;
         }
       }
@@ -2290,7 +2391,7 @@ __device__ void pass_stream(const SolveCfg* cfg, SolveSmem<DPS, NU>& sm, int war
       // unread, so the ring never overwrites one)
       while (cur.made - used < cnt && cur.u < tc) {
         const int o = fplace(cur, xpn, lo, hi, rp2, lane, tc);
-        if (o >= 0) rxyz[o & 63] = xpn;
+        if (o >= 0) rxyz[o & (kRing - 1)] = xpn;
         if (cur.u < tc) xpn = load_point<DPS, NU>(g, sm, warp, cur.u + lane, tc, cur.seg);
       }
       __syncwarp();
@@ -2298,7 +2399,7 @@ __device__ void pass_stream(const SolveCfg* cfg, SolveSmem<DPS, NU>& sm, int war
       int xi = -1;
       const bool have = lane < cnt && used + lane < cur.made;
       if (have) {
-        xp = rxyz[(used + lane) & 63];
+        xp = rxyz[(used + lane) & (kRing - 1)];
         xi = __float_as_int(xp.w);
         xp.w = 0.f;
       }
@@ -2334,7 +2435,6 @@ __device__ void pass_stream(const SolveCfg* cfg, SolveSmem<DPS, NU>& sm, int war
 // share of a reused plan that is too large is cached as far as it goes, with the
 // front left to the streamed pass's ring for the rest of it (BlockCtx::rest_c).
 constexpr int kCacheSlots = 32;                 // items per warp
-constexpr int kRingFloats = 4 * 64;             // the streamed passes' ring
 constexpr unsigned short kSlotCluster = 0x8000;
 constexpr unsigned short kSlotList = 0x4000;      // cluster whose pairs are listed
 
@@ -2440,8 +2540,8 @@ __device__ void fill_cache(const SolveCfg* cfg, SolveSmem<DPS, NU>& sm, int warp
     return;
   }
   float* base = cache + (size_t)warp * cap;
-  if (part) base += kRingFloats;
-  int room = part ? cap - kRingFloats : cap;
+  if (part) base += b.ring_floats;
+  int room = part ? cap - b.ring_floats : cap;
   int n = 0, k = 0, coff = room;   // items, chunk slots, where the clusters begin
   int rest_c = -1, rest_j = 0, rest_g = 0;
   for (int c = r.c0; c <= r.c1 && c < cv.ncl && rest_c < 0; ++c) {
@@ -2650,8 +2750,8 @@ __device__ void pass_cached(const SolveCfg* cfg, SolveSmem<DPS, NU>& sm, int war
   const bool collect = !STEP && sm.b.collect_kept;
   const float* base = cache + (size_t)warp * cap;
   if (sm.b.rest_c[warp] >= 0) {   // the front is the ring of the streamed rest
-    base += kRingFloats;
-    cap -= kRingFloats;
+    base += sm.b.ring_floats;
+    cap -= sm.b.ring_floats;
   }
   const unsigned short* pl = sm.ws[warp].list;
   const int n = sm.cache_n[warp];
@@ -2715,7 +2815,7 @@ __device__ void pass_cached(const SolveCfg* cfg, SolveSmem<DPS, NU>& sm, int war
   if (collect) add_kept(cfg, cur, nnz - nnz0, lane);
 }
 
-template <bool STEP, int DP, int MODE, int DPS, int NU>
+template <bool STEP, int DP, int MODE, int DPS, int NU, bool TWO>
 __device__ __forceinline__ void pass_warp(const SolveCfg* cfg, SolveSmem<DPS, NU>& sm, int warp,
                                           int lane, float* cache, int cap, float acc[7],
                                           unsigned& nnz, unsigned& cand) {
@@ -2731,13 +2831,13 @@ __device__ __forceinline__ void pass_warp(const SolveCfg* cfg, SolveSmem<DPS, NU
   }
   for (int k = 0; k < streamed; ++k) {
     if (k > 0) r = warp_range(b, warp, k);
-    pass_stream<STEP, DP, MODE, DPS, NU>(cfg, sm, warp, lane, r, cache + (size_t)warp * cap, acc,
+    pass_stream<STEP, DP, MODE, DPS, NU, TWO>(cfg, sm, warp, lane, r, cache + (size_t)warp * cap, acc,
                                          nnz, cand);
   }
 }
 
 // One pass over the block's warps, then the block partial (fixed order).
-template <bool STEP, int DP, int MODE, int DPS, int NU>
+template <bool STEP, int DP, int MODE, int DPS, int NU, bool TWO>
 __device__ void run_pass(const SolveCfg* cfg, SolveSmem<DPS, NU>& sm, double* partials,
                          float* cache, int cap) {
   constexpr int NACC = STEP ? 5 : 7;
@@ -2750,7 +2850,7 @@ __device__ void run_pass(const SolveCfg* cfg, SolveSmem<DPS, NU>& sm, double* pa
     if (STEP) gradient_fp64(sm.b, sm.sums, lane);
     else if (sm.b.pending) pending_step(sm.b, lane);
   }
-  pass_warp<STEP, DP, MODE, DPS, NU>(cfg, sm, warp, lane, cache, cap, acc, nnz, cand);
+  pass_warp<STEP, DP, MODE, DPS, NU, TWO>(cfg, sm, warp, lane, cache, cap, acc, nnz, cand);
   __syncwarp();
   // the warp's sums: halves of the warp exchange half of the values, then quarters,
   // eighths, so that lane 4 i ends with the sum of value i (nine shuffles, not 35)
@@ -2815,7 +2915,7 @@ __device__ void publish(SolveState* st, const BlockCtx& b) {
 }
 
 // The whole solve of one pair (or one evaluation) by one team of blocks.
-template <int DP, int MODE, int DPS, int NU>
+template <int DP, int MODE, int DPS, int NU, bool TWO>
 __device__ void solve_pair(const SolveCfg* __restrict__ cfg, SolveState* __restrict__ st,
                            double* __restrict__ partials, IterRecord* __restrict__ records,
                            Team team, SolveSmem<DPS, NU>& sm, bool join, float* cache,
@@ -2864,6 +2964,7 @@ __device__ void solve_pair(const SolveCfg* __restrict__ cfg, SolveState* __restr
     b.use_kept = b.collect_kept = b.rebalance = b.use_act = 0;
     b.t = b.t_prev = 0.0;
     b.pending = 0;
+    b.ring_floats = 4 * ring_size<TWO>();
     b.nnz_total = b.cand_total = b.nnz_grad = b.cand_grad = 0;
     b.F = b.xi_norm = 0.0;
     for (int i = 0; i < 6; ++i) b.xi[i] = 0.0;
@@ -2942,7 +3043,7 @@ __device__ void solve_pair(const SolveCfg* __restrict__ cfg, SolveState* __restr
     }
     if (stamp) t1 = globaltimer();
     // ---- gradient pass ----
-    run_pass<false, DP, MODE, DPS, NU>(cfg, sm, part_g, cache, cap);
+    run_pass<false, DP, MODE, DPS, NU, TWO>(cfg, sm, part_g, cache, cap);
     if (stamp) tg1 = globaltimer();
     if (!grid_sync_reduce(st, gen, sm, part_g, 9, team.size, [&](int ln) {
           if (sm.b.n_workers == kWarps && sm.b.pending) pending_step(sm.b, ln);
@@ -2956,7 +3057,7 @@ __device__ void solve_pair(const SolveCfg* __restrict__ cfg, SolveState* __restr
     __syncthreads();
     if (stamp) t2 = globaltimer();
     // ---- step pass ----
-    run_pass<true, DP, MODE, DPS, NU>(cfg, sm, part_s, cache, cap);
+    run_pass<true, DP, MODE, DPS, NU, TWO>(cfg, sm, part_s, cache, cap);
     if (stamp) ts1 = globaltimer();
     // the next iteration's constants, on their way while the block waits
     const unsigned icw = iter_word(cfg, min(sm.b.k + 1, sm.b.tc.max_iters - 1), lane);
@@ -3016,7 +3117,7 @@ solve_kernel(const SolveCfg* __restrict__ cfg, SolveState* __restrict__ st,
   constexpr int NU = 2;
   __shared__ SolveSmem<DPS, NU> sm;
   extern __shared__ float4 dyn_smem[];
-  solve_pair<DP, MODE, DPS, NU>(cfg, st, partials, records, Team{(int)blockIdx.x, (int)gridDim.x},
+  solve_pair<DP, MODE, DPS, NU, false>(cfg, st, partials, records, Team{(int)blockIdx.x, (int)gridDim.x},
                                 sm, false, reinterpret_cast<float*>(dyn_smem), cache_cap);
 }
 
@@ -3130,7 +3231,7 @@ queue_kernel(const QueueEntry* __restrict__ entries, const QueueCtl* __restrict_
     if (sm.q_slot < 0) break;
     const QueueEntry en = load_entry(entries + sm.q_entry);
     const Team team{(int)(sm.q_slot - en.slot0), en.team};
-    solve_pair<DP, MODE, DPS, NU>(en.cfg, en.st, en.partials, nullptr, team, sm, true,
+    solve_pair<DP, MODE, DPS, NU, true>(en.cfg, en.st, en.partials, nullptr, team, sm, true,
                                   reinterpret_cast<float*>(dyn_smem), cache_cap);
     if (threadIdx.x == 0) {
       __threadfence();
@@ -3168,7 +3269,7 @@ const CacheCfg& cache_cfg() {
     const int slot = 32 * (4 + DP);   // slot_floats
     const int avail = smem_sm / CVO_SOLVE_MIN_BLOCKS - reserved - (int)fa.sharedSizeBytes;
     c.cap = std::max(0, std::min(kCacheSlots * slot, avail / kWarps / 64 * 16));
-    if (c.cap < kRingFloats) {
+    if (c.cap < 4 * 128) {   // ring_size, twice a single solve's
       c.err = cudaErrorInvalidConfiguration;
       return c;
     }
