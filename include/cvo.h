@@ -450,8 +450,8 @@ int cvo_frontend_cloud(cvo_ctx* ctx, const float* depth, const float* hsv, int w
  * kernels run on `stream` (NULL: the default stream) and the call returns
  * without waiting for them.
  *
- * Scratch: block partials live in a fixed 32 KB array in the library's
- * device memory (512 slots), which every GPU that loads the library holds
+ * Scratch: block partials live in a fixed 38 KB array in the library's
+ * device memory (608 slots), which every GPU that loads the library holds
  * until the process exits. Each call writes every slot it reads, so nothing
  * carries over between calls, but all calls on one device share the array:
  * calls whose kernels overlap on the GPU (different streams, or different

@@ -21,14 +21,15 @@ namespace {
 constexpr int kNaThreads = 128;
 constexpr int kNaSrc = 2 * kNaThreads; // source points of a work item, two per thread
 constexpr int kNaTile = 256;           // its target points at most
-constexpr int kNaMaxBlocks = 512;      // partial slots in the static scratch
-constexpr int kNaGrid = 3 * 152;       // blocks of a full launch: three to an SM
+constexpr int kNaMaxBlocks = 608;      // partial slots in the static scratch
+constexpr int kNaGrid = 4 * 152;       // blocks of a full launch: four to an SM
+constexpr int kNaQueue = 2048;         // pairs a warp appends to its queue at once
 constexpr int kNaStride = 8;           // F, omega'(3), v(3), kept pairs
 constexpr int kNaMaxDevices = 64;
 constexpr int kNaFlush = 256;          // pairs a lane adds in FP32 before its sums go to FP64
 
 // Scratch shared by every call on a device: kNaMaxBlocks block partials
-// (32 KB). Held by every GPU that loads the library until the process exits.
+// (38 KB). Held by every GPU that loads the library until the process exits.
 __device__ __align__(256) double g_na_partials[kNaMaxBlocks * kNaStride];
 
 static_assert(kNaGrid <= kNaMaxBlocks, "one partial slot per block");
@@ -81,7 +82,7 @@ template <int DP>
 struct NaSmem {
   alignas(16) float z[3 + DP][kNaSrc];     // transformed source points and scaled features
   alignas(16) float x[3 + DP][kNaTile];    // target points relative to the first one, features
-  unsigned short queue[kNaThreads / 32][31 + 64 * 32];   // kept pairs: target | source << 8
+  unsigned short queue[kNaThreads / 32][32 + kNaQueue];   // kept pairs: target | source << 8
   double red[7][kNaThreads];
   unsigned long long cnt[kNaThreads / 32];
   float R[9], T[3], x0[3], z0[3];
@@ -93,18 +94,19 @@ struct NaSmem {
 // with every target in turn ran 3 blocks for 600 points and 79 for 20000).
 // Most pairs are out of range and the points come in no particular order, so
 // testing and evaluating are kept apart: a lane holds two source points, tests
-// them against 32 targets (broadcast from shared memory, two per packed
+// them against 64 targets (broadcast from shared memory, two per packed
 // operation: bound by the FMA pipe at six cycles of a scheduler for 32 tests)
-// and notes the kept ones in two masks; the warp appends the pairs to its queue
+// and notes the kept ones in masks; the warp appends the pairs to its queue
 // and evaluates 32 queued pairs at a time, one per lane, whatever points they
 // belong to: F, sum w z~ x e and sum w e need no order. Evaluating in place
 // would run a body for every group of tests in which any lane keeps a pair,
-// which at 1% kept is nearly all of them. 20000 x 20000 points at 1.3% kept: 188
-// us against 1274 us before (the tests alone are 65 us of the FMA pipe).
+// which at 1% kept is nearly all of them. 20000 x 20000 points at 1.3% kept: 160
+// us against 1274 us before (the tests alone are 60 us of the FMA pipe, the queued
+// pairs' scattered shared loads about 30).
 // Coordinates are taken relative to the first target point x0 (one rounding of
 // the difference), so FP32 pair arithmetic never subtracts large coordinates.
 template <int DP, int MODE>
-__global__ void __launch_bounds__(kNaThreads, 3)
+__global__ void __launch_bounds__(kNaThreads, 4)
 na_grad_kernel(const float* __restrict__ x, const float* __restrict__ fx,
                const float* __restrict__ z, const float* __restrict__ fz, NaArgs a,
                double* __restrict__ partials) {
@@ -205,60 +207,76 @@ na_grad_kernel(const float* __restrict__ x, const float* __restrict__ fx,
       for (int c = 0; c < 3; ++c) Z[h][c] = na_dup2(sm.z[c][k]);
     }
     int queued = 0;   // the same in every lane
-    for (int t0 = 0; t0 < tn; t0 += 32) {
-      unsigned keep[2] = {0u, 0u};
+    for (int t0 = 0; t0 < tn; t0 += 64) {
+      // the lane's kept pairs: bit k of keep[h][w] is source h, target t0 + 32 w + k
+      unsigned keep[2][2] = {{0u, 0u}, {0u, 0u}};
 #pragma unroll
-      for (int k = 0; k < 32; k += 4) {
-        const ulonglong2 X = *reinterpret_cast<const ulonglong2*>(&sm.x[0][t0 + k]);
-        const ulonglong2 Y = *reinterpret_cast<const ulonglong2*>(&sm.x[1][t0 + k]);
-        const ulonglong2 W = *reinterpret_cast<const ulonglong2*>(&sm.x[2][t0 + k]);
+      for (int w = 0; w < 2; ++w) {
+        if (t0 + 32 * w >= tn) break;
 #pragma unroll
-        for (int h = 0; h < 2; ++h) {
+        for (int k = 0; k < 32; k += 4) {
+          const int t = t0 + 32 * w + k;
+          const ulonglong2 X = *reinterpret_cast<const ulonglong2*>(&sm.x[0][t]);
+          const ulonglong2 Y = *reinterpret_cast<const ulonglong2*>(&sm.x[1][t]);
+          const ulonglong2 W = *reinterpret_cast<const ulonglong2*>(&sm.x[2][t]);
 #pragma unroll
-          for (int p = 0; p < 2; ++p) {
-            const na_f32x2 ex = na_sub2(p ? X.y : X.x, Z[h][0]);
-            const na_f32x2 ey = na_sub2(p ? Y.y : Y.x, Z[h][1]);
-            const na_f32x2 ez = na_sub2(p ? W.y : W.x, Z[h][2]);
-            const na_f32x2 d2 = na_fma2(ex, ex, na_fma2(ey, ey, na_mul2(ez, ez)));
-            float d20, d21;
-            asm("mov.b64 {%0, %1}, %2;" : "=f"(d20), "=f"(d21) : "l"(d2));
-            if (d20 <= a.rc2) keep[h] |= 1u << (k + 2 * p);
-            if (d21 <= a.rc2) keep[h] |= 1u << (k + 2 * p + 1);
+          for (int h = 0; h < 2; ++h) {
+#pragma unroll
+            for (int p = 0; p < 2; ++p) {
+              const na_f32x2 ex = na_sub2(p ? X.y : X.x, Z[h][0]);
+              const na_f32x2 ey = na_sub2(p ? Y.y : Y.x, Z[h][1]);
+              const na_f32x2 ez = na_sub2(p ? W.y : W.x, Z[h][2]);
+              const na_f32x2 d2 = na_fma2(ex, ex, na_fma2(ey, ey, na_mul2(ez, ez)));
+              float d20, d21;
+              asm("mov.b64 {%0, %1}, %2;" : "=f"(d20), "=f"(d21) : "l"(d2));
+              if (d20 <= a.rc2) keep[h][w] |= 1u << (k + 2 * p);
+              if (d21 <= a.rc2) keep[h][w] |= 1u << (k + 2 * p + 1);
+            }
           }
         }
+        // points past the ends never count, whatever the cutoff
+        const int left = tn - t0 - 32 * w;
+        const unsigned valid = left < 32 ? (1u << left) - 1u : 0xffffffffu;
+        keep[0][w] &= zv[0] ? valid : 0u;
+        keep[1][w] &= zv[1] ? valid : 0u;
       }
-      // points past the ends never count, whatever the cutoff
-      if (tn - t0 < 32) {
-        keep[0] &= (1u << (tn - t0)) - 1u;
-        keep[1] &= (1u << (tn - t0)) - 1u;
-      }
-      if (!zv[0]) keep[0] = 0u;
-      if (!zv[1]) keep[1] = 0u;
-      const int mine = __popc(keep[0]) + __popc(keep[1]);
-      if (!__any_sync(0xffffffffu, mine != 0)) continue;
-      int pos = mine;
+      const int n0 = __popc(keep[0][0]) + __popc(keep[1][0]);
+      const int n1 = __popc(keep[0][1]) + __popc(keep[1][1]);
+      cnt += (unsigned)(n0 + n1);
+      const int total = __reduce_add_sync(0xffffffffu, n0 + n1);
+      if (total == 0) continue;
+      // both words at once, or, should they not fit the queue, one after the other
+      const bool both = total <= kNaQueue;
+      for (int w0 = 0; w0 < 2; ++w0) {
+        const int mine = both ? n0 + n1 : w0 ? n1 : n0;
+        int pos = mine;
 #pragma unroll
-      for (int off = 1; off < 32; off <<= 1) {
-        const int v = __shfl_up_sync(0xffffffffu, pos, off);
-        if (lane >= off) pos += v;
-      }
-      const int total = __shfl_sync(0xffffffffu, pos, 31);
-      pos += queued - mine;
+        for (int off = 1; off < 32; off <<= 1) {
+          const int v = __shfl_up_sync(0xffffffffu, pos, off);
+          if (lane >= off) pos += v;
+        }
+        const int end = queued + __shfl_sync(0xffffffffu, pos, 31);
+        pos += queued - mine;
 #pragma unroll
-      for (int h = 0; h < 2; ++h) {
-        const unsigned src = (unsigned)(warp * 64 + 32 * h + lane) << 8;
-        for (unsigned m = keep[h]; m != 0u; m &= m - 1u)
-          queue[pos++] = (unsigned short)(src | (unsigned)(t0 + __ffs(m) - 1));
+        for (int w = 0; w < 2; ++w) {
+          if (!both && w != w0) continue;
+#pragma unroll
+          for (int h = 0; h < 2; ++h) {
+            const unsigned src = (unsigned)(warp * 64 + 32 * h + lane) << 8 | (unsigned)(t0 + 32 * w);
+            for (unsigned m = keep[h][w]; m != 0u; m &= m - 1u)
+              queue[pos++] = (unsigned short)(src + (unsigned)(__ffs(m) - 1));
+          }
+        }
+        queued = end;
+        __syncwarp();
+        while (queued >= 32) {   // full rounds from the end of the queue; fewer than 32 pairs stay
+          queued -= 32;
+          evaluate(queue[queued + lane]);
+          ++added;
+        }
+        __syncwarp();
+        if (both) break;
       }
-      queued += total;
-      cnt += (unsigned)mine;
-      __syncwarp();
-      while (queued >= 32) {   // full rounds from the end of the queue; fewer than 32 pairs stay
-        queued -= 32;
-        evaluate(queue[queued + lane]);
-        ++added;
-      }
-      __syncwarp();
       if (added >= kNaFlush) {
 #pragma unroll
         for (int k = 0; k < 7; ++k) {
