@@ -22,8 +22,8 @@
 // same on any run. Five launches and one wait: at 640 x 480 every kernel is a few
 // microseconds of latency, so what counts is how few there are (sorting the
 // magnitudes to read two of them took 12 of the 23 launches, and their count had
-// to visit the host): 279 -> 87 us per frame, of which the call's host side, with
-// its allocation, wait and read-back, is about a third.
+// to visit the host): 279 -> 75 us per frame, of which the call's host side, with
+// its allocation, wait and read-back, is about half.
 #include <cuda_runtime.h>
 
 #include <algorithm>
@@ -93,52 +93,52 @@ fe_pixels_kernel(const float* __restrict__ depth, const float* __restrict__ hsv,
   fe_flush(s_hist, c->hist[0]);
 }
 
-// Where rank r falls in 2048 digit counts: the digit, the rank left within it
-// and the total. Every thread of the block calls it (kScanBlock threads, two
-// digits each); a rank at or beyond the total gives digit 2047.
-struct FeDigit {
-  unsigned digit, left, total;
+// 2048 digit counts, two per thread of a block of kScanBlock, with the counts up to
+// and including this thread's and the total. Every thread of the block calls it.
+struct FeScan {
+  unsigned a, b, incl, total;
 };
 
-__device__ FeDigit fe_find(const unsigned* hist, unsigned rank) {
+__device__ FeScan fe_scan(const unsigned* hist) {
   __shared__ unsigned s_warp[kScanBlock / 32];
-  __shared__ FeDigit s_found;
   const int t = threadIdx.x, lane = t & 31, warp = t >> 5;
-  const unsigned a = __ldcg(&hist[2 * t]), b = __ldcg(&hist[2 * t + 1]);
-  unsigned incl = a + b;
+  const uint2 v = __ldcg(reinterpret_cast<const uint2*>(hist) + t);
+  FeScan f{v.x, v.y, v.x + v.y, 0u};
   for (int off = 1; off < 32; off <<= 1) {
-    const unsigned v = __shfl_up_sync(0xffffffffu, incl, off);
-    if (lane >= off) incl += v;
+    const unsigned u = __shfl_up_sync(0xffffffffu, f.incl, off);
+    if (lane >= off) f.incl += u;
   }
   __syncthreads();   // the shared words of an earlier call have been read
-  if (lane == 31) s_warp[warp] = incl;
-  if (t == 0) s_found = FeDigit{2047u, 0u, 0u};
+  if (lane == 31) s_warp[warp] = f.incl;
   __syncthreads();
-  unsigned total = 0u;
-  for (int w = 0; w < kScanBlock / 32; ++w) {
-    if (w < warp) incl += s_warp[w];
-    total += s_warp[w];
-  }
-  const unsigned before = incl - a - b;
-  if (rank >= before && rank < incl) {
-    const bool second = rank >= before + a;
-    s_found.digit = 2u * t + (second ? 1u : 0u);
-    s_found.left = rank - before - (second ? a : 0u);
-  }
-  __syncthreads();
-  FeDigit f = s_found;
-  f.total = total;
+  const unsigned w = s_warp[lane];
+  f.total = __reduce_add_sync(0xffffffffu, w);
+  f.incl += __reduce_add_sync(0xffffffffu, lane < warp ? w : 0u);
   return f;
 }
 
-// The lower order statistic's rank among n values at percentile q, and the FP64
-// position (numpy's 'linear' method).
-__device__ __forceinline__ unsigned fe_rank(unsigned n, double q, double* h) {
-  *h = n > 0u ? (double)(int)(n - 1u) * (q / 100.0) : 0.0;
-  return (unsigned)(int)floor(*h);
+// Where rank r falls: the digit and the rank left within it (digit 2047, rank 0, when
+// r is at or beyond the total). Every thread of the block calls it.
+struct FeDigit {
+  unsigned digit, left;
+};
+
+__device__ FeDigit fe_locate(const FeScan& f, unsigned rank) {
+  __shared__ FeDigit s_found;
+  const unsigned before = f.incl - f.a - f.b;
+  __syncthreads();   // an earlier call's answer has been read
+  if (threadIdx.x == 0 && rank >= f.total) s_found = FeDigit{2047u, 0u};
+  if (rank >= before && rank < f.incl) {
+    const bool second = rank >= before + f.a;
+    s_found = FeDigit{2u * threadIdx.x + (second ? 1u : 0u), rank - before - (second ? f.a : 0u)};
+  }
+  __syncthreads();
+  return s_found;
 }
 
-// The digits found so far: the top one (level 1), and the next (level 2).
+// The valid pixels, the lower order statistic's rank at percentile q among them and
+// the FP64 position it comes from (numpy's 'linear' method), and the digits of that
+// statistic found so far: the top one (level 1), and the next (level 2).
 struct FePrefix {
   unsigned n, rank, d0, d1, left;
   double h;
@@ -148,22 +148,22 @@ __device__ FePrefix fe_prefix(const FeCounts* c, double q, int level) {
   __shared__ unsigned s_rank;
   __shared__ double s_h;
   FePrefix f;
-  FeDigit d = fe_find(c->hist[0], 0u);
-  f.n = d.total;
+  const FeScan top = fe_scan(c->hist[0]);
+  f.n = top.total;
   if (threadIdx.x == 0) {   // FP64 on one thread of one warp
-    double h;
-    s_rank = fe_rank(f.n, q, &h);
+    const double h = f.n > 0u ? (double)(int)(f.n - 1u) * (q / 100.0) : 0.0;
+    s_rank = (unsigned)(int)floor(h);
     s_h = h;
   }
   __syncthreads();
   f.rank = s_rank;
   f.h = s_h;
-  d = fe_find(c->hist[0], f.rank);
+  FeDigit d = fe_locate(top, f.rank);
   f.d0 = d.digit;
   f.left = d.left;
   f.d1 = 0u;
   if (level > 1) {
-    d = fe_find(c->hist[1], f.left);
+    d = fe_locate(fe_scan(c->hist[1]), f.left);
     f.d1 = d.digit;
     f.left = d.left;
   }
@@ -203,12 +203,13 @@ fe_digits_kernel(const unsigned* __restrict__ keys, int n, double q, int level,
 __device__ double fe_threshold(const FeCounts* c, double q) {
   __shared__ double s_thr;
   const FePrefix f = fe_prefix(c, q, 2);
-  const FeDigit lo = fe_find(c->hist[2], f.left), hi = fe_find(c->hist[2], f.left + 1u);
+  const FeScan last = fe_scan(c->hist[2]);
+  const FeDigit lo = fe_locate(last, f.left), hi = fe_locate(last, f.left + 1u);
   if (threadIdx.x == 0) {
     const unsigned pre = (f.d0 << 11 | f.d1) << 10;
     const unsigned ka = pre | lo.digit;
     // the next rank: in the same prefix, beyond it, or (the last rank) the same
-    const unsigned kb = f.rank + 1u >= f.n ? ka : f.left + 1u < hi.total ? pre | hi.digit
+    const unsigned kb = f.rank + 1u >= f.n ? ka : f.left + 1u < last.total ? pre | hi.digit
                                                                          : ~__ldcg(&c->above);
     const double t = f.h - (double)(int)f.rank;
     const double a = (double)__uint_as_float(ka), b = (double)__uint_as_float(kb);
@@ -267,9 +268,9 @@ fe_emit_kernel(const float* __restrict__ depth, const float* __restrict__ hsv,
     r += s_before[w] + (w < warp ? s_warp[w] : 0);
   }
   if (blockIdx.x == 0) {
-    const FeDigit all = fe_find(c->hist[0], 0u);   // its total is every valid pixel
+    const unsigned valid = fe_scan(c->hist[0]).total;
     if (t == 0) {
-      totals[0] = (int)all.total;
+      totals[0] = (int)valid;
       totals[1] = (int)m;
     }
   }
