@@ -1602,7 +1602,7 @@ __device__ void locate(const SolveCfg* cfg, const ClusterView& cv, int group, lo
 // block left the slowest block 1.2 to 1.3 times the mean. Each further piece costs
 // its warp a cluster to stage and two ends to locate.
 template <int DPS, int NU>
-__device__ void split_work(const SolveCfg* cfg, SolveSmem<DPS, NU>& sm, int tid, Team team,
+__device__ __noinline__ void split_work(const SolveCfg* cfg, SolveSmem<DPS, NU>& sm, int tid, Team team,
                            const long long* agg) {
   const ClusterView& cv = cfg->clusters[sm.b.ic.level];
   const int lane = tid & 31, warp = tid >> 5;
@@ -2461,7 +2461,7 @@ __device__ __forceinline__ int cluster_floats(int cs) {
 // warp's shared scratch (list_max entries). A cluster whose list would not
 // fit keeps the chunk-by-chunk evaluation.
 template <int DP, int DPS, int NU>
-__device__ void build_lists(SolveSmem<DPS, NU>& sm, int warp, int lane, const float* base,
+__device__ __noinline__ void build_lists(SolveSmem<DPS, NU>& sm, int warp, int lane, const float* base,
                             int cap, int n) {
   unsigned short* pl = sm.ws[warp].list;
   constexpr int kCap = list_max<DPS>();
@@ -2517,21 +2517,38 @@ __device__ void build_lists(SolveSmem<DPS, NU>& sm, int warp, int lane, const fl
 }
 
 template <int DP, int MODE, int DPS, int NU>
-__device__ void fill_cache(const SolveCfg* cfg, SolveSmem<DPS, NU>& sm, int warp, int lane,
+__device__ __noinline__ void fill_cache(const SolveCfg* cfg, SolveSmem<DPS, NU>& sm, int warp, int lane,
                            float* cache, int cap) {
   const BlockCtx& b = sm.b;
   const GridView& g = cfg->grids[b.ic.level];
   const ClusterView& cv = cfg->clusters[b.ic.level];
   const WarpRange r = warp_range(b, warp, 0);
   const float rp2 = b.rplan_f * b.rplan_f;
+  // the numbers of cluster c + lane and its chunks in the range (none: live false),
+  // read together so that the fill waits for two round trips to L2 per cluster
+  // (these, then its points, segments and box) instead of six
+  const int c_end = min(r.c1, cv.ncl - 1);
+  int l_tc = 0, l_fc = 0, l_p0 = 0, l_cs = 0, l_nseg = 0, l_jb = 0, l_je = -1, at = -1;
+  bool live = false;
+  const auto read = [&](int c) {
+    at = c;
+    live = false;
+    if (c + lane > c_end) return;
+    l_tc = __ldcg(&cfg->cl_cand[c + lane]);
+    l_fc = __ldcg(&cfg->cl_fcand[c + lane]);
+    l_nseg = __ldcg(&cfg->cl_nseg[c + lane]);
+    l_p0 = cv.cstart[c + lane];
+    l_cs = cv.cstart[c + lane + 1] - l_p0;
+    live = range_chunks(r, c + lane, (l_fc + 31) >> 5, l_jb, l_je);
+  };
   // what the share needs (one in several pieces is too large for the cache)
   int need = 0, items = b.n_range > 1 ? kCacheSlots + 1 : 0;
-  for (int c = r.c0; c <= r.c1 && c < cv.ncl; ++c) {
-    int jb, je;
-    if (!range_chunks(r, c, (__ldcg(&cfg->cl_fcand[c]) + 31) >> 5, jb, je)) continue;
-    need += cluster_floats<DP>(cv.cstart[c + 1] - cv.cstart[c]) + (1 + je - jb) * slot_floats<DP>();
-    items += 2 + je - jb;
-    if (need > cap || items > kCacheSlots) break;
+  for (int c = r.c0; c <= c_end && need <= cap && items <= kCacheSlots; c += 32) {
+    read(c);
+    // (a lane's count may be large, the sum is capped)
+    const int nc = live ? min(1 + l_je - l_jb, kCacheSlots) : 0;
+    need += __reduce_add_sync(kFull, live ? cluster_floats<DP>(l_cs) + nc * slot_floats<DP>() : 0);
+    items += __reduce_add_sync(kFull, live ? 1 + nc : 0);
   }
   const bool part = need > cap || items > kCacheSlots;
   if (part && (b.n_range > 1 || !b.plan_filter)) {
@@ -2544,81 +2561,89 @@ __device__ void fill_cache(const SolveCfg* cfg, SolveSmem<DPS, NU>& sm, int warp
   int room = part ? cap - b.ring_floats : cap;
   int n = 0, k = 0, coff = room;   // items, chunk slots, where the clusters begin
   int rest_c = -1, rest_j = 0, rest_g = 0;
-  for (int c = r.c0; c <= r.c1 && c < cv.ncl && rest_c < 0; ++c) {
-    const int tc = __ldcg(&cfg->cl_cand[c]);
-    const int fc = __ldcg(&cfg->cl_fcand[c]);
-    int jb, je;
-    if (!range_chunks(r, c, (fc + 31) >> 5, jb, je)) continue;
-    const int p0 = cv.cstart[c];
-    const int cs = cv.cstart[c + 1] - p0, cs4 = (cs + 3) & ~3;
-    room -= cluster_floats<DP>(cs);
-    if (part) {
-      // the chunks of this cluster that still fit; the rest is streamed
-      const int fit = min(kCacheSlots - n - 1, room < 0 ? 0 : room / slot_floats<DP>());
-      if (1 + je - jb > fit) {
-        rest_c = c;
-        rest_j = jb + max(fit, 0);
-        rest_g = c == r.c0 && rest_j == r.j0 ? r.g0 : 0;
-        je = rest_j - 1;
-        if (je < jb) break;
+  for (int cb = r.c0; cb <= c_end && rest_c < 0; cb += 32) {
+    if (cb != at) read(cb);
+    for (unsigned todo = __ballot_sync(kFull, live); todo && rest_c < 0; todo &= todo - 1u) {
+      const int li = __ffs(todo) - 1, c = cb + li;
+      const int tc = __shfl_sync(kFull, l_tc, li), fc = __shfl_sync(kFull, l_fc, li);
+      const int p0 = __shfl_sync(kFull, l_p0, li), nseg = __shfl_sync(kFull, l_nseg, li);
+      const int cs = __shfl_sync(kFull, l_cs, li), cs4 = (cs + 3) & ~3;
+      const int jb = __shfl_sync(kFull, l_jb, li);
+      int je = __shfl_sync(kFull, l_je, li);
+      room -= cluster_floats<DP>(cs);
+      if (part) {
+        // the chunks of this cluster that still fit; the rest is streamed
+        const int fit = min(kCacheSlots - n - 1, room < 0 ? 0 : room / slot_floats<DP>());
+        if (1 + je - jb > fit) {
+          rest_c = c;
+          rest_j = jb + max(fit, 0);
+          rest_g = c == r.c0 && rest_j == r.j0 ? r.g0 : 0;
+          je = rest_j - 1;
+          if (je < jb) break;
+        }
       }
-    }
-    room -= (1 + je - jb) * slot_floats<DP>();
-    coff -= cluster_floats<DP>(cs);
-    float* sl = base + coff;
-    if (lane < cs) {
-      reinterpret_cast<float4*>(sl)[lane] = cfg->src.xyz[p0 + lane];
+      room -= (1 + je - jb) * slot_floats<DP>();
+      coff -= cluster_floats<DP>(cs);
+      float4 lo = __ldcg(&cfg->cl_box[2 * (size_t)c]);
+      float4 hi = __ldcg(&cfg->cl_box[2 * (size_t)c + 1]);
+      float4 p = make_float4(0.f, 0.f, 0.f, 0.f);
+      float pf[DPS];
+      if (lane < cs) {
+        p = cfg->src.xyz[p0 + lane];
 #pragma unroll
-      for (int d = 0; d < DP; ++d)
-        sl[(4 + d) * cs4 + lane] =
-            load_feat<bf16_of(MODE)>(cfg->src.feat, (size_t)d * cfg->src.m_pad + p0 + lane);
-    }
-    if (lane == 0) {
-      sm.cache_hdr[warp][n] = (unsigned short)(kSlotCluster | cs);
-      sm.cache_cl[warp][n] = c;
-    }
-    ++n;
-    const int nseg = __ldcg(&cfg->cl_nseg[c]);
-    load_segments<DPS, NU>(cfg, sm, warp, lane, c, nseg, tc, fc);
-    float4 lo = __ldcg(&cfg->cl_box[2 * (size_t)c]);
-    float4 hi = __ldcg(&cfg->cl_box[2 * (size_t)c + 1]);
-    if (lo.w == 0.f) {   // not filtered by the plan: every candidate of the range is cached
-      lo = make_float4(-INFINITY, -INFINITY, -INFINITY, 0.f);
-      hi = make_float4(INFINITY, INFINITY, INFINITY, 0.f);
-    }
-    FCursor cur = fcursor_at<DPS, NU>(sm, warp, nseg, jb * 32);
-    const int want = min(fc, 32 * (je + 1)) - 32 * jb;
-    float* s0 = base + (size_t)k * slot_floats<DP>();
-    while (cur.made < want && cur.u < tc) {
-      float xf[DPS];
-      const float4 xp =
-          load_candidate<DP, DPS, NU, bf16_of(MODE)>(g, sm, warp, cur.u + lane, tc, cur.seg, xf);
-      const int o = fplace(cur, xp, lo, hi, rp2, lane, tc);
-      if (o >= 0 && o < want) {
+        for (int d = 0; d < DP; ++d)
+          pf[d] = load_feat<bf16_of(MODE)>(cfg->src.feat, (size_t)d * cfg->src.m_pad + p0 + lane);
+      }
+      load_segments<DPS, NU>(cfg, sm, warp, lane, c, nseg, tc, fc);
+      float* sl = base + coff;
+      if (lane < cs) {
+        reinterpret_cast<float4*>(sl)[lane] = p;
+#pragma unroll
+        for (int d = 0; d < DP; ++d) sl[(4 + d) * cs4 + lane] = pf[d];
+      }
+      if (lane == 0) {
+        sm.cache_hdr[warp][n] = (unsigned short)(kSlotCluster | cs);
+        sm.cache_cl[warp][n] = c;
+      }
+      ++n;
+      if (lo.w == 0.f) {   // not filtered by the plan: every candidate of the range is cached
+        lo = make_float4(-INFINITY, -INFINITY, -INFINITY, 0.f);
+        hi = make_float4(INFINITY, INFINITY, INFINITY, 0.f);
+      }
+      FCursor cur = fcursor_at<DPS, NU>(sm, warp, nseg, jb * 32);
+      const int want = min(fc, 32 * (je + 1)) - 32 * jb;
+      float* s0 = base + (size_t)k * slot_floats<DP>();
+      while (cur.made < want && cur.u < tc) {
+        float xf[DPS];
+        const float4 xp =
+            load_candidate<DP, DPS, NU, bf16_of(MODE)>(g, sm, warp, cur.u + lane, tc, cur.seg, xf);
+        const int o = fplace(cur, xp, lo, hi, rp2, lane, tc);
+        if (o >= 0 && o < want) {
+          float* sk = s0 + (size_t)(o >> 5) * slot_floats<DP>();
+          reinterpret_cast<float4*>(sk)[o & 31] = xp;
+#pragma unroll
+          for (int d = 0; d < DP; ++d) sk[128 + d * 32 + (o & 31)] = xf[d];
+        }
+      }
+      const int nchk = je - jb + 1;
+      for (int o = min(cur.made, want) + lane; o < 32 * nchk; o += 32) {   // padding
         float* sk = s0 + (size_t)(o >> 5) * slot_floats<DP>();
-        reinterpret_cast<float4*>(sk)[o & 31] = xp;
+        reinterpret_cast<float4*>(sk)[o & 31] = make_float4(-kFar, -kFar, -kFar, 1.f);
 #pragma unroll
-        for (int d = 0; d < DP; ++d) sk[128 + d * 32 + (o & 31)] = xf[d];
+        for (int d = 0; d < DP; ++d) sk[128 + d * 32 + (o & 31)] = 0.f;
       }
+      if (lane <= je - jb) {
+        const int j = jb + lane;
+        int glo, ghi;
+        range_groups(r, c, j, cs4 >> 2, glo, ghi);
+        const int cnt = min(32, want - 32 * lane);
+        sm.cache_hdr[warp][n + lane] = (unsigned short)(cnt | (glo << 6) | (ghi << 10));
+        sm.cache_cl[warp][n + lane] = j;   // a chunk slot keeps its chunk index
+      }
+      n += nchk;
+      k += nchk;
+      __syncwarp();   // the segment arrays are reused by the next cluster
     }
-    const int nchk = je - jb + 1;
-    for (int o = min(cur.made, want) + lane; o < 32 * nchk; o += 32) {   // padding
-      float* sk = s0 + (size_t)(o >> 5) * slot_floats<DP>();
-      reinterpret_cast<float4*>(sk)[o & 31] = make_float4(-kFar, -kFar, -kFar, 1.f);
-#pragma unroll
-      for (int d = 0; d < DP; ++d) sk[128 + d * 32 + (o & 31)] = 0.f;
-    }
-    if (lane <= je - jb) {
-      const int j = jb + lane;
-      int glo, ghi;
-      range_groups(r, c, j, ((cs + 3) & ~3) >> 2, glo, ghi);
-      const int cnt = min(32, want - 32 * lane);
-      sm.cache_hdr[warp][n + lane] = (unsigned short)(cnt | (glo << 6) | (ghi << 10));
-      sm.cache_cl[warp][n + lane] = j;   // a chunk slot keeps its chunk index
-    }
-    n += nchk;
-    k += nchk;
-    __syncwarp();   // the segment arrays are reused by the next cluster
   }
   if (lane == 0) {
     sm.cache_n[warp] = (short)n;
