@@ -73,9 +73,6 @@ constexpr int kActChunks = 32;              // chunks per cluster whose source-g
 // requests 95.6, 96.2, 98.1 ms
 constexpr int kSmallTeam = 32;
 constexpr int kCompactWork = 3000;
-#ifndef CVO_COST_ACTIVE
-#define CVO_COST_ACTIVE 12
-#endif
 // a warp's share of the work is cut into pieces taken from different parts of the
 // cloud (split_work): one per kRangeWork pair-test units of it, at most
 // kMaxRanges, from kRangeFrom units on. Whole-GPU teams, 100k room pair: up to 4
@@ -93,7 +90,13 @@ constexpr int kSmallTeamFrom = 20000;
 // pair 825, 832, 832 us
 constexpr int kSpareWork = 400;
 // work model: the pair bodies of a source group that kept a pair, in pair-test units
-constexpr int kCostActive = CVO_COST_ACTIVE;
+constexpr int kCostActive = 12;
+// and for shares in this range: large enough for the bodies to count, small enough
+// that the shares they are weighed into still fit the cache. Whole room solves with 12
+// and 24: 10k points 3.56, 3.58 ms, 15k 4.40, 4.25, 20k 5.36, 5.20, 24k 6.37, 6.16, 28k
+// 7.31, 7.07; from here on 24 overflows the cache: 34k 9.5, 9.9, 45k 13.6, 14.1
+constexpr int kCostActiveShort = 24;
+constexpr int kActShareFrom = 140, kActShareTo = 450;
 
 __device__ __forceinline__ float ex2_approx(float x) {
   float y;
@@ -225,7 +228,8 @@ struct BlockCtx {
   int k, plan_level, plan_filter;
   int need_plan, done, converged, fallback, no_ascent, have_t_prev;
   int use_kept, collect_kept, rebalance;   // kept-pair weighting of the work split
-  int use_act;                             // the split weighs source groups by their activity
+  int use_act;                             // the split weighs active source groups by this (0: not)
+  int cost_act;                            // what a rebalance of this plan will weigh them by
   int compact;                             // streamed passes box-test unfiltered clusters
   int team_rank, team_size;                // this block's place in its team (read after a pass
                                            // from shared memory rather than kept in registers)
@@ -1403,13 +1407,13 @@ __device__ void plan_cluster(const SolveCfg* cfg, const BlockCtx& b, SolveState*
 // spread evenly over its chunks. Chunk j starts at offset cost_cluster + j * k,
 // k = the per-chunk cost; within a chunk, the overhead and the first group of
 // four source points come first, then one group (4 tests) after another.
-// With use_act (a reused plan, once its first gradient pass has recorded
+// With act > 0 (a reused plan, once its first gradient pass has recorded
 // which source groups of which chunks kept a pair), each such group costs
-// kCostActive more (its pair bodies); chunks beyond the recorded ones count
+// act more (its pair bodies); chunks beyond the recorded ones count
 // every group as active.
 __device__ __forceinline__ long long cluster_work(const SolveCfg* cfg, const ClusterView& cv,
                                                   int c, int* k_out, int* cs4_out, int* nch_out,
-                                                  bool use_kept, bool use_act) {
+                                                  bool use_kept, int act) {
   const int tc = __ldcg(&cfg->cl_fcand[c]);
   const int cs4 = ((cv.cstart[c + 1] - cv.cstart[c]) + 3) & ~3;
   const int nch = (tc + 31) >> 5;
@@ -1421,8 +1425,8 @@ __device__ __forceinline__ long long cluster_work(const SolveCfg* cfg, const Clu
   *k_out = k;
   if (nch <= 0) return 0;
   long long w = (long long)cfg->cost_cluster + (long long)nch * k;
-  if (use_act)
-    w += (long long)kCostActive * ((long long)__ldcg(&cfg->cl_act[c]) +
+  if (act)
+    w += (long long)act * ((long long)__ldcg(&cfg->cl_act[c]) +
                                    (long long)max(0, nch - kActChunks) * (cs4 >> 2));
   return w;
 }
@@ -1499,11 +1503,11 @@ struct SolveSmem {
 // cluster's first chunk.
 __device__ void locate(const SolveCfg* cfg, const ClusterView& cv, int group, long long base,
                        long long s, int lane, int* c_out, int* j_out, int* g_out,
-                       bool use_kept, bool use_act) {
+                       bool use_kept, int act) {
   const int c = group * 32 + lane;
   long long w = 0;
   int kk = 4, cs4_l = 4, nch_l = 0;
-  if (c < cv.ncl) w = cluster_work(cfg, cv, c, &kk, &cs4_l, &nch_l, use_kept, use_act);
+  if (c < cv.ncl) w = cluster_work(cfg, cv, c, &kk, &cs4_l, &nch_l, use_kept, act);
   long long incl = w;
 #pragma unroll
   for (int off = 1; off < 32; off <<= 1) {
@@ -1522,8 +1526,8 @@ __device__ void locate(const SolveCfg* cfg, const ClusterView& cv, int group, lo
     const int G = cs4 >> 2;
     const int nch = __shfl_sync(kFull, nch_l, src);
     int j = 0, gq = 0;
-    if (use_act && s > e) {
-      // chunk j costs k4 + kCostActive x (its active groups; all of them past
+    if (act && s > e) {
+      // chunk j costs k4 + act x (its active groups; all of them past
       // the recorded chunks); lane j holds chunk j's mask
       const unsigned gm = (1u << G) - 1u;
       long long cum = 0;   // end of the chunks before this round, relative to e
@@ -1531,7 +1535,7 @@ __device__ void locate(const SolveCfg* cfg, const ClusterView& cv, int group, lo
         const int jj = j0 + lane;
         unsigned mj = gm;
         if (jj < nch && jj < kActChunks) mj = __ldcg(&cfg->ch_act[(size_t)cc * kActChunks + jj]) & gm;
-        const long long kj = jj < nch ? (long long)k4 + (long long)kCostActive * __popc(mj) : 0;
+        const long long kj = jj < nch ? (long long)k4 + (long long)act * __popc(mj) : 0;
         long long in = kj;
 #pragma unroll
         for (int off = 1; off < 32; off <<= 1) {
@@ -1547,15 +1551,15 @@ __device__ void locate(const SolveCfg* cfg, const ClusterView& cv, int group, lo
           j = j0 + src2;
           if (s > start) {
             // units of the chunk: group 0 at start (with the overhead), group
-            // g at start + oh + sum over g' < g of (4 + kCostActive a_g')
-            long long u = start + oh + 4 + kCostActive * (long long)(m & 1u);
+            // g at start + oh + sum over g' < g of (4 + act a_g')
+            long long u = start + oh + 4 + act * (long long)(m & 1u);
             gq = G;
             for (int g = 1; g < G; ++g) {
               if (u >= s) {
                 gq = g;
                 break;
               }
-              u += 4 + kCostActive * (long long)((m >> g) & 1u);
+              u += 4 + act * (long long)((m >> g) & 1u);
             }
             if (gq >= G) {
               ++j;
@@ -1668,6 +1672,8 @@ __device__ __noinline__ void split_work(const SolveCfg* cfg, SolveSmem<DPS, NU>&
   }
   if (tid == 0) {
     sm.b.n_range = nr;
+    if (!sm.b.use_act)
+      sm.b.cost_act = share >= kActShareFrom && share < kActShareTo ? kCostActiveShort : kCostActive;
     sm.b.n_workers = nw;
     sm.b.compact = small || share >= kCompactWork ? 1 : 0;
   }
@@ -1679,7 +1685,7 @@ __device__ __noinline__ void split_work(const SolveCfg* cfg, SolveSmem<DPS, NU>&
       int c = cv.ncl, jj = 0, gg = 0;   // past the end: no chunk
       if (warp < nw && sm.split.group[q] >= 0)
         locate(cfg, cv, sm.split.group[q], sm.split.base[q], sm.split.at[q], lane, &c, &jj, &gg,
-               sm.b.use_kept != 0, sm.b.use_act != 0);
+               sm.b.use_kept != 0, sm.b.use_act);
       if (lane == 0) {
         if (h == 0) {
           sm.b.w_c0[k][warp] = c;
@@ -3039,15 +3045,14 @@ __device__ void solve_pair(const SolveCfg* __restrict__ cfg, SolveState* __restr
       }
       if (tid == 0) {
         sm.b.use_kept = rebalance && cfg->cost_kept > 0.f;
-        sm.b.use_act = rebalance && sm.b.plan_filter;
+        sm.b.use_act = rebalance && sm.b.plan_filter ? sm.b.cost_act : 0;
       }
       __syncthreads();
       if (rebalance || plans == 0) {
         for (long long gi = gw; gi < ng; gi += NW) {
           const int c = (int)gi * 32 + lane;
           int kk, cs4, nch;
-          long long w = c < cv.ncl ? cluster_work(cfg, cv, c, &kk, &cs4, &nch, sm.b.use_kept != 0,
-                                                  sm.b.use_act != 0)
+          long long w = c < cv.ncl ? cluster_work(cfg, cv, c, &kk, &cs4, &nch, sm.b.use_kept != 0, sm.b.use_act)
                                    : 0;
 #pragma unroll
           for (int off = 16; off > 0; off >>= 1) w += __shfl_down_sync(kFull, w, off);
