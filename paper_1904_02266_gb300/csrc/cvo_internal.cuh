@@ -15,8 +15,7 @@ namespace cvo {
 
 // Warps per block of the pair passes: one block of 16 warps per SM (all 64K
 // registers at 128 a thread), so that the team barriers reduce one partial
-// per SM rather than two (on GB300 that FP64 reduction runs at about 64 cycles
-// per warp instruction) at the same 16 warps per SM.
+// per SM rather than two at the same 16 warps per SM.
 #ifndef CVO_WARPS
 #define CVO_WARPS 16
 #endif

@@ -17,24 +17,28 @@
 //              rows of target cells within the plan radius, stored as segments
 //              of the cell-sorted target, and (clusters with at most
 //              kFilterMax candidates) the count of candidates within the plan
-//              radius of the box, per segment.                         barrier
-//              work totals of groups of 32 clusters.                    barrier
+//              radius of the box, per segment; the work of groups of 32
+//              clusters is added up on the way (a queued solve's first plan and
+//              a rebalance total it after a barrier).                   barrier
 //              every block scans the group totals and places its own warps on
-//              an even split of the work, cut at groups of four source points
-//              (no further barrier).
+//              an even split of the work into pieces from all over the cloud,
+//              cut at groups of four source points (no further barrier).
 //  gradient    each warp walks its share of chunks of 32 filtered candidates:
 //  pass        one lane per candidate target point against the cluster's
-//              source points staged in shared memory (broadcast reads). FP32
-//              pairs, one ex2.approx per kept pair, per-lane FP32 sums,
-//              fixed-order reductions.                                 barrier
-//  tail        every block reduces all block partials (value-major) in FP64
-//              in the same fixed order and runs the same FP64 tail, so
-//              nothing is published or broadcast.
+//              source points staged in shared memory (broadcast reads), the
+//              distance tests of a chunk before its pair bodies. FP32 pairs,
+//              two to a packed operation, one ex2.approx per kept pair,
+//              per-lane FP32 sums, fixed-order reductions.             barrier
+//  tail        every block adds all block partials (value-major) as aligned
+//              64-bit integers and forms the same unit direction, so nothing
+//              is published or broadcast.
 //  step pass   as above along the unit direction.                      barrier
-//  tail        step length, exponential-map update, next iteration.
+//  tail        step length, exponential-map update, next iteration: in FP64
+//              at once, or, for small plain steps, the passes' pose in FP32
+//              and the FP64 step behind the next gradient pass.
 // The plan is reused while it still covers the cutoff: it is built with a
 // radius 10% wider than the cutoff and rebuilt when the grid level changes,
-// when the pose has drifted by more than that margin (an FP64 bound over the
+// when the pose has drifted by more than that margin (a bound over the
 // whole source cloud), or when it has become much wider than needed. A warp
 // whose share of a reused plan fits its cache also lists, once per
 // plan, the (candidate, source point) pairs of each cached cluster within the
@@ -1154,8 +1158,8 @@ __device__ __forceinline__ void reduce_partials(const double* partials, int nval
 
 // Barrier that also reduces the pass: every block adds its arrival (a release
 // reduction after the block's partials are written), waits for the
-// generation's last arrival with acquire loads, and then sums all block
-// partials itself in the same fixed FP64 order, so that no block has to
+// generation's last arrival with acquire loads, and then adds all block
+// partials itself (reduce_partials), so that no block has to
 // publish totals and release the others. A block reads the partials of
 // generation g only before it arrives at generation g + 1, and the next
 // writes to the same partial buffer (two generations later) come after that
@@ -2909,7 +2913,7 @@ __device__ void run_pass(const SolveCfg* cfg, SolveSmem<DPS, NU>& sm, double* pa
   if (warp == 0 && lane < NACC + 2) {
     double s = 0.0;
     if (lane < NACC) {
-      // the block's eight warp sums in FP32 (fixed order); FP64 starts with the
+      // the block's sixteen warp sums in FP32 (fixed order); FP64 starts with the
       // cross-block reduction
       float f = 0.f;
 #pragma unroll
