@@ -27,6 +27,11 @@ constexpr int kNaQueue = 2048;         // pairs a warp appends to its queue at o
 constexpr int kNaStride = 8;           // F, omega'(3), v(3), kept pairs
 constexpr int kNaMaxDevices = 64;
 constexpr int kNaFlush = 256;          // pairs a lane adds in FP32 before its sums go to FP64
+                                       //   (tested once a round, which may add 128 more)
+constexpr int kNaSample = 8192;        // source points from which a launch samples the clouds, and
+constexpr int kNaDense = 20;           //   the kept pairs of 128 from which it evaluates in place
+constexpr float kNaFar = 1e18f;        // coordinate of the slots past the ends
+constexpr float kNaWild = 1e15f;       // in place, coordinates from here on go pair by pair
 
 // Scratch shared by every call on a device: kNaMaxBlocks block partials
 // (38 KB). Held by every GPU that loads the library until the process exits.
@@ -62,6 +67,24 @@ __device__ __forceinline__ na_f32x2 na_dup2(float v) {
   asm("mov.b64 %0, {%1, %1};" : "=l"(r) : "f"(v));
   return r;
 }
+__device__ __forceinline__ na_f32x2 na_pack2(float lo, float hi) {
+  na_f32x2 r;
+  asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(lo), "f"(hi));
+  return r;
+}
+__device__ __forceinline__ void na_unpack2(na_f32x2 v, float& lo, float& hi) {
+  asm("mov.b64 {%0, %1}, %2;" : "=f"(lo), "=f"(hi) : "l"(v));
+}
+__device__ __forceinline__ float na_sum2(na_f32x2 v) {
+  float lo, hi;
+  na_unpack2(v, lo, hi);
+  return lo + hi;
+}
+__device__ __forceinline__ na_f32x2 na_add2(na_f32x2 a, na_f32x2 b) {
+  na_f32x2 r;
+  asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+  return r;
+}
 __device__ __forceinline__ na_f32x2 na_sub2(na_f32x2 a, na_f32x2 b) {
   na_f32x2 r;
   asm("sub.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
@@ -88,6 +111,142 @@ struct NaSmem {
   float R[9], T[3], x0[3], z0[3];
 };
 
+// One kept pair: target t against source s of the staged tiles.
+template <int DP, int MODE>
+__device__ __forceinline__ void na_pair(const NaSmem<DP>& sm, int t, int s, float A, float acc[7]) {
+  const float zx = sm.z[0][s], zy = sm.z[1][s], zz = sm.z[2][s];
+  const float ex = sm.x[0][t] - zx, ey = sm.x[1][t] - zy, ez = sm.x[2][t] - zz;
+  const float d2 = fmaf(ex, ex, fmaf(ey, ey, ez * ez));
+  float w;
+  if (MODE == cvo::kColorKernel) {
+    float q = 0.f;
+#pragma unroll
+    for (int d = 0; d < DP; ++d) {
+      const float df = sm.x[3 + d][t] - sm.z[3 + d][s];
+      q = fmaf(df, df, q);
+    }
+    w = na_ex2(-fmaf(A, d2, q));
+  } else if (MODE == cvo::kColorDot) {
+    float c = 0.f;
+#pragma unroll
+    for (int d = 0; d < DP; ++d) c = fmaf(sm.x[3 + d][t], sm.z[3 + d][s], c);
+    w = na_ex2(-A * d2) * c;
+  } else {
+    w = na_ex2(-A * d2);
+  }
+  const float vx = w * ex, vy = w * ey, vz = w * ez;
+  acc[0] += w;
+  acc[1] += zy * vz - zz * vy;   // omega' += z~' x w e, v += w e
+  acc[2] += zz * vx - zx * vz;
+  acc[3] += zx * vy - zy * vx;
+  acc[4] += vx;
+  acc[5] += vy;
+  acc[6] += vz;
+}
+
+// A warp's part of a work item in place: the lane's two source points against every
+// target, two to a packed operation, the weight of a pair that is not kept selected to
+// zero. Its products are then zero as long as the coordinates are below kNaWild, and the
+// slots past the ends are beyond a cutoff below kNaWild; an item with larger ones, or a
+// NaN, goes pair by pair. Adds the lane's sums F, omega', v to acc64 and returns its kept
+// pairs.
+template <int DP, int MODE>
+__device__ __forceinline__ unsigned na_dense(const NaSmem<DP>& sm, int warp, int lane, int tn, int ms,
+                                             float rc2, float A, double acc64[7]) {
+  const int s0 = warp * 64 + lane;
+  bool wild = !(rc2 < kNaWild * kNaWild);
+#pragma unroll
+  for (int c = 0; c < 3; ++c) {
+    wild = wild || (s0 < ms && !(fabsf(sm.z[c][s0]) < kNaWild)) ||
+           (s0 + 32 < ms && !(fabsf(sm.z[c][s0 + 32]) < kNaWild));
+    for (int t = lane; t < tn; t += 32) wild = wild || !(fabsf(sm.x[c][t]) < kNaWild);
+  }
+  if (__any_sync(0xffffffffu, wild)) {
+    float acc[7] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
+    unsigned cnt = 0;
+    for (int s = s0; s < min(ms, s0 + 64); s += 32) {
+      for (int t = 0; t < tn; ++t) {
+        const float ex = sm.x[0][t] - sm.z[0][s], ey = sm.x[1][t] - sm.z[1][s],
+                    ez = sm.x[2][t] - sm.z[2][s];
+        if (!(fmaf(ex, ex, fmaf(ey, ey, ez * ez)) <= rc2)) continue;
+        ++cnt;
+        na_pair<DP, MODE>(sm, t, s, A, acc);
+      }
+    }
+#pragma unroll
+    for (int k = 0; k < 7; ++k) acc64[k] += (double)acc[k];
+    return cnt;
+  }
+  na_f32x2 Z[2][3 + DP];
+#pragma unroll
+  for (int h = 0; h < 2; ++h) {
+#pragma unroll
+    for (int c = 0; c < 3 + DP; ++c) Z[h][c] = na_dup2(sm.z[c][s0 + 32 * h]);
+  }
+  float acc[7] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
+  const na_f32x2 A2 = na_dup2(A);
+  na_f32x2 sum[2][4] = {{0ull, 0ull, 0ull, 0ull}, {0ull, 0ull, 0ull, 0ull}};
+  unsigned cnt = 0;
+  for (int t = 0; t < tn; t += 4) {
+    ulonglong2 X[3 + DP];
+#pragma unroll
+    for (int c = 0; c < 3 + DP; ++c) X[c] = *reinterpret_cast<const ulonglong2*>(&sm.x[c][t]);
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+#pragma unroll
+      for (int p = 0; p < 2; ++p) {
+        const na_f32x2 ex = na_sub2(p ? X[0].y : X[0].x, Z[h][0]);
+        const na_f32x2 ey = na_sub2(p ? X[1].y : X[1].x, Z[h][1]);
+        const na_f32x2 ez = na_sub2(p ? X[2].y : X[2].x, Z[h][2]);
+        const na_f32x2 d2 = na_fma2(ex, ex, na_fma2(ey, ey, na_mul2(ez, ez)));
+        na_f32x2 q = 0ull;   // appearance: sum of squared differences, or inner product
+#pragma unroll
+        for (int d = 0; d < DP; ++d) {
+          const na_f32x2 f = p ? X[3 + d].y : X[3 + d].x;
+          if (MODE == cvo::kColorKernel) {
+            const na_f32x2 df = na_sub2(f, Z[h][3 + d]);
+            q = na_fma2(df, df, q);
+          } else if (MODE == cvo::kColorDot) {
+            q = na_fma2(f, Z[h][3 + d], q);
+          }
+        }
+        float d20, d21, e0, e1;
+        na_unpack2(d2, d20, d21);
+        const bool k0 = d20 <= rc2, k1 = d21 <= rc2;
+        na_unpack2(MODE == cvo::kColorKernel ? na_fma2(A2, d2, q) : na_mul2(A2, d2), e0, e1);
+        float w0 = na_ex2(-e0), w1 = na_ex2(-e1);
+        if (MODE == cvo::kColorDot) {
+          float c0, c1;
+          na_unpack2(q, c0, c1);
+          w0 *= c0;
+          w1 *= c1;
+        }
+        const na_f32x2 w = na_pack2(k0 ? w0 : 0.f, k1 ? w1 : 0.f);
+        cnt += (k0 ? 1u : 0u) + (k1 ? 1u : 0u);
+        sum[h][0] = na_add2(sum[h][0], w);
+        sum[h][1] = na_fma2(w, ex, sum[h][1]);
+        sum[h][2] = na_fma2(w, ey, sum[h][2]);
+        sum[h][3] = na_fma2(w, ez, sum[h][3]);
+      }
+    }
+  }
+#pragma unroll
+  for (int h = 0; h < 2; ++h) {   // omega' += z~' x E, v += E, E = sum w e
+    const float zx = sm.z[0][s0 + 32 * h], zy = sm.z[1][s0 + 32 * h], zz = sm.z[2][s0 + 32 * h];
+    const float Ex = na_sum2(sum[h][1]), Ey = na_sum2(sum[h][2]), Ez = na_sum2(sum[h][3]);
+    acc[0] += na_sum2(sum[h][0]);
+    acc[1] += zy * Ez - zz * Ey;
+    acc[2] += zz * Ex - zx * Ez;
+    acc[3] += zx * Ey - zy * Ex;
+    acc[4] += Ex;
+    acc[5] += Ey;
+    acc[6] += Ez;
+  }
+#pragma unroll
+  for (int k = 0; k < 7; ++k) acc64[k] += (double)acc[k];
+  return cnt;
+}
+
 // The all-pairs gradient pass. A work item is 256 source points against a tile
 // of at most 256 target points; blocks take items in turn and keep one partial
 // sum each, so that small clouds spread over many SMs (a thread per source point
@@ -103,6 +262,14 @@ struct NaSmem {
 // which at 1% kept is nearly all of them. 20000 x 20000 points at 1.3% kept: 160
 // us against 1274 us before (the tests alone are 60 us of the FMA pipe, the queued
 // pairs' scattered shared loads about 30).
+// Where most pairs are kept the queue is the dearer way (20000 x 20000 points, five
+// features, all kept: 2220 us, against 1660 of a thread per source point), so a launch
+// samples the clouds first and evaluates every item in place from a sixth kept on: 335 us
+// whatever is kept, which the queue passes at 14% (328 us; 23%: 471). The choice is the
+// launch's, not an item's: a choice within the items, by a sample, the first round or the
+// item before, cost the queue 1 to 5% in registers and code. Below kNaSample source
+// points nothing is sampled (it takes 1 us): a kept pair costs the queue 5.5 ps, and a
+// thread per source point took 83 ns per target, so the queue loses from 15000 on.
 // Coordinates are taken relative to the first target point x0 (one rounding of
 // the difference), so FP32 pair arithmetic never subtracts large coordinates.
 template <int DP, int MODE>
@@ -132,45 +299,15 @@ na_grad_kernel(const float* __restrict__ x, const float* __restrict__ fx,
   unsigned long long cnt = 0;
   int added = 0;
   const auto evaluate = [&](unsigned e) {
-    const int t = (int)(e & 255u), s = (int)(e >> 8);
-    const float zx = sm.z[0][s], zy = sm.z[1][s], zz = sm.z[2][s];
-    const float ex = sm.x[0][t] - zx, ey = sm.x[1][t] - zy, ez = sm.x[2][t] - zz;
-    const float d2 = fmaf(ex, ex, fmaf(ey, ey, ez * ez));
-    float w;
-    if (MODE == cvo::kColorKernel) {
-      float q = 0.f;
-#pragma unroll
-      for (int d = 0; d < DP; ++d) {
-        const float df = sm.x[3 + d][t] - sm.z[3 + d][s];
-        q = fmaf(df, df, q);
-      }
-      w = na_ex2(-fmaf(a.A, d2, q));
-    } else if (MODE == cvo::kColorDot) {
-      float c = 0.f;
-#pragma unroll
-      for (int d = 0; d < DP; ++d) c = fmaf(sm.x[3 + d][t], sm.z[3 + d][s], c);
-      w = na_ex2(-a.A * d2) * c;
-    } else {
-      w = na_ex2(-a.A * d2);
-    }
-    const float vx = w * ex, vy = w * ey, vz = w * ez;
-    acc[0] += w;
-    acc[1] += zy * vz - zz * vy;   // omega' += z~' x w e, v += w e
-    acc[2] += zz * vx - zx * vz;
-    acc[3] += zx * vy - zy * vx;
-    acc[4] += vx;
-    acc[5] += vy;
-    acc[6] += vz;
+    na_pair<DP, MODE>(sm, (int)(e & 255u), (int)(e >> 8), a.A, acc);
   };
   const int nS = (a.m + kNaSrc - 1) / kNaSrc, nT = (a.n + a.tile - 1) / a.tile;
   const long long items = (long long)nS * nT;
-  for (long long it = blockIdx.x; it < items; it += gridDim.x) {
-    const int j0 = (int)(it / nT) * kNaSrc, i0 = (int)(it % nT) * a.tile;
-    const int tn = min(a.tile, a.n - i0);
-    __syncthreads();   // the tiles of the previous item are free (and R, T are there)
+  // The item's source points from j0 on and target points from i0 on.
+  const auto stage = [&](int j0, int i0) {
     for (int k = tid; k < kNaSrc; k += kNaThreads) {
       const int j = j0 + k;
-      float zx = -1e18f, zy = -1e18f, zz = -1e18f;   // past the end: beyond every cutoff
+      float zx = -kNaFar, zy = -kNaFar, zz = -kNaFar;   // past the end: beyond every cutoff
       if (j < a.m) {
         const float px = z[3 * (size_t)j] - sm.z0[0], py = z[3 * (size_t)j + 1] - sm.z0[1],
                     pz = z[3 * (size_t)j + 2] - sm.z0[2];
@@ -190,11 +327,43 @@ na_grad_kernel(const float* __restrict__ x, const float* __restrict__ fx,
       const int i = i0 + k;
 #pragma unroll
       for (int c = 0; c < 3; ++c)
-        sm.x[c][k] = i < a.n ? x[3 * (size_t)i + c] - sm.x0[c] : 1e18f;
+        sm.x[c][k] = i < a.n ? x[3 * (size_t)i + c] - sm.x0[c] : kNaFar;
 #pragma unroll
       for (int d = 0; d < DP; ++d)
         sm.x[3 + d][k] = i < a.n && d < a.D ? fx[(size_t)a.D * i + d] * a.fscale : 0.f;
     }
+  };
+  // A sample of 128 pairs from all over the clouds, the same for every block: where a
+  // sixth or more are kept, every item is evaluated in place.
+  int sample = 0;
+  if (a.m >= kNaSample) {
+    __syncthreads();   // R and T are there
+    const long long si = (long long)(tid * 37 & 127) * a.n >> 7, sj = (long long)tid * a.m >> 7;
+    float e[3], p[3];
+#pragma unroll
+    for (int c = 0; c < 3; ++c) p[c] = z[3 * sj + c] - sm.z0[c];
+#pragma unroll
+    for (int c = 0; c < 3; ++c)
+      e[c] = x[3 * si + c] - sm.x0[c] -
+             fmaf(sm.R[3 * c], p[0], fmaf(sm.R[3 * c + 1], p[1], fmaf(sm.R[3 * c + 2], p[2], sm.T[c])));
+    sample = __syncthreads_count(fmaf(e[0], e[0], fmaf(e[1], e[1], e[2] * e[2])) <= a.rc2);
+  }
+  const bool in_place = sample >= kNaDense;
+  if (in_place) {
+    for (long long it = blockIdx.x; it < items; it += gridDim.x) {
+      const int j0 = (int)(it / nT) * kNaSrc, i0 = (int)(it % nT) * a.tile;
+      __syncthreads();   // the tiles of the previous item are free
+      stage(j0, i0);
+      __syncthreads();
+      if (j0 + warp * 64 < a.m)
+        cnt += na_dense<DP, MODE>(sm, warp, lane, min(a.tile, a.n - i0), a.m - j0, a.rc2, a.A, acc64);
+    }
+  }
+  for (long long it = in_place ? items : blockIdx.x; it < items; it += gridDim.x) {
+    const int j0 = (int)(it / nT) * kNaSrc, i0 = (int)(it % nT) * a.tile;
+    const int tn = min(a.tile, a.n - i0);
+    __syncthreads();   // the tiles of the previous item are free (and R, T are there)
+    stage(j0, i0);
     __syncthreads();
     if (j0 + warp * 64 >= a.m) continue;   // a warp past the last source point
     na_f32x2 Z[2][3];
@@ -228,7 +397,7 @@ na_grad_kernel(const float* __restrict__ x, const float* __restrict__ fx,
               const na_f32x2 ez = na_sub2(p ? W.y : W.x, Z[h][2]);
               const na_f32x2 d2 = na_fma2(ex, ex, na_fma2(ey, ey, na_mul2(ez, ez)));
               float d20, d21;
-              asm("mov.b64 {%0, %1}, %2;" : "=f"(d20), "=f"(d21) : "l"(d2));
+              na_unpack2(d2, d20, d21);
               if (d20 <= a.rc2) keep[h][w] |= 1u << (k + 2 * p);
               if (d21 <= a.rc2) keep[h][w] |= 1u << (k + 2 * p + 1);
             }
