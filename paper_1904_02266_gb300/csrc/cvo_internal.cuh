@@ -137,7 +137,9 @@ struct SolveState {
   double ell;                // lengthscale of the current iteration
   int level;                 // level of the current iteration
   int iter, done, converged;
-  int fallback_steps, no_ascent_steps, have_t_prev, status;
+  int fallback_steps, no_ascent_steps, status;
+  int spilled;               // the last reused plan (from 1 on) of which a share that was weighed
+                             //   by kCostActiveShort did not fit its warp's cache
   unsigned long long nnz_total, cand_total;
   unsigned long long nnz_pass[2], cand_pass[2];
   unsigned long long nnz_eval, cand_eval;   // gradient pass of the last iteration

@@ -52,6 +52,7 @@
 #include <algorithm>
 
 #include "cvo_internal.cuh"
+#include "split_rule.h"
 
 // Resident blocks per SM the solve kernel is compiled for (register budget).
 #ifndef CVO_SOLVE_MIN_BLOCKS
@@ -93,14 +94,6 @@ constexpr int kSmallTeamFrom = 20000;
 // 3.80, 3.68, 3.68 ms, 20k 5.65, 5.51, 5.57 ms, 28k 7.45, 7.44, 7.47 ms; the 2k planes
 // pair 825, 832, 832 us
 constexpr int kSpareWork = 400;
-// work model: the pair bodies of a source group that kept a pair, in pair-test units
-constexpr int kCostActive = 12;
-// and for shares in this range: large enough for the bodies to count, small enough
-// that the shares they are weighed into still fit the cache. Whole room solves with 12
-// and 24: 10k points 3.56, 3.58 ms, 15k 4.40, 4.25, 20k 5.36, 5.20, 24k 6.37, 6.16, 28k
-// 7.31, 7.07; from here on 24 overflows the cache: 34k 9.5, 9.9, 45k 13.6, 14.1
-constexpr int kCostActiveShort = 24;
-constexpr int kActShareFrom = 140, kActShareTo = 450;
 
 __device__ __forceinline__ float ex2_approx(float x) {
   float y;
@@ -234,6 +227,10 @@ struct BlockCtx {
   int use_kept, collect_kept, rebalance;   // kept-pair weighting of the work split
   int use_act;                             // the split weighs active source groups by this (0: not)
   int cost_act;                            // what a rebalance of this plan will weigh them by
+  int plan_no;                             // reused plans so far
+  int check_fit;                           // a rebalance by more than kCostActive: see check_fits
+  int cap;                                 // floats of a warp's cache
+  SolveState* st;
   int compact;                             // streamed passes box-test unfiltered clusters
   int team_rank, team_size;                // this block's place in its team (read after a pass
                                            // from shared memory rather than kept in registers)
@@ -730,6 +727,19 @@ __device__ void gradient_direction(BlockCtx& b, const double* sums, int lane) {
   __syncwarp();
 }
 
+// In the first iteration of a rebalance that weighed active groups by more than
+// kCostActive, behind its gradient pass (every block has filled its cache before that
+// pass's barrier, so all read the same): if a warp of the team could not cache its share,
+// the next iteration rebalances again, by kCostActive. One warp of 2280 that streams its
+// rest in every pass of a plan holds up the team by 10% of the solve (active_weight has
+// the figures). One lane.
+__device__ __forceinline__ void check_fits(BlockCtx& b) {
+  b.check_fit = 0;
+  if (__ldcg(&b.st->spilled) != b.plan_no) return;
+  b.cost_act = kCostActive;
+  b.rebalance = 1;
+}
+
 // Gradient tail, second part (one warp, while the block waits at the step pass's
 // barrier): the metric gradient xi (Eq. metric), |xi|,
 // xi / |xi| in FP64, F and the gradient pass's counts.
@@ -763,6 +773,7 @@ __device__ void gradient_fp64(BlockCtx& b, const double* sums, int lane) {
     b.F = tc.sigma2 * sums[0];
     b.nnz_grad = (unsigned long long)__double_as_longlong(sums[7]);
     b.cand_grad = (unsigned long long)__double_as_longlong(sums[8]);
+    if (b.check_fit) check_fits(b);
   }
   __syncwarp();
 }
@@ -1676,8 +1687,13 @@ __device__ __noinline__ void split_work(const SolveCfg* cfg, SolveSmem<DPS, NU>&
   }
   if (tid == 0) {
     sm.b.n_range = nr;
-    if (!sm.b.use_act)
-      sm.b.cost_act = share >= kActShareFrom && share < kActShareTo ? kCostActiveShort : kCostActive;
+    // (a plan used once has no rebalance: its chain of round trips is shorter without)
+    if (!sm.b.use_act && sm.b.plan_filter) {
+      sm.b.plan_no += 1;
+      sm.b.cost_act = active_weight(TW, NW, cv.ncl, cfg->src.m, cfg->cost_chunk, cfg->cost_cluster,
+                                    DPS > 1 ? 4 + DPS : 4, sm.b.cap);
+    }
+    sm.b.check_fit = sm.b.use_act > kCostActive ? 1 : 0;
     sm.b.n_workers = nw;
     sm.b.compact = small || share >= kCompactWork ? 1 : 0;
   }
@@ -2561,6 +2577,7 @@ __device__ __noinline__ void fill_cache(const SolveCfg* cfg, SolveSmem<DPS, NU>&
     items += __reduce_add_sync(kFull, live ? 1 + nc : 0);
   }
   const bool part = need > cap || items > kCacheSlots;
+  if (part && lane == 0 && b.use_act > kCostActive) atomicMax(&b.st->spilled, b.plan_no);
   if (part && (b.n_range > 1 || !b.plan_filter)) {
     if (lane == 0) sm.cache_n[warp] = -1;
     __syncwarp();
@@ -2997,6 +3014,9 @@ __device__ void solve_pair(const SolveCfg* __restrict__ cfg, SolveState* __restr
     b.done = cfg->max_iters <= 0 ? 1 : 0;
     b.converged = b.fallback = b.no_ascent = b.have_t_prev = 0;
     b.use_kept = b.collect_kept = b.rebalance = b.use_act = 0;
+    b.plan_no = b.check_fit = 0;
+    b.cap = cap;
+    b.st = st;
     b.t = b.t_prev = 0.0;
     b.pending = 0;
     b.ring_floats = 4 * ring_size<TWO>();
