@@ -411,7 +411,6 @@ int configure_plan(cvo_ctx* ctx, Plan* p, Cloud* t, Cloud* s, const std::vector<
   cfg.sigma2 = prm.sigma * prm.sigma;
   cfg.a2 = prm.a2;
   cfg.b2 = prm.b2;
-  cfg.ell_floor = ell_floor(prm);
   cfg.eps_pose = prm.eps_pose;
   cfg.eps_grad = prm.eps_grad;
   cfg.max_iters = mode == kModeEval ? 1 : prm.max_iters;

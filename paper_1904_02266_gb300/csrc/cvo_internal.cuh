@@ -115,7 +115,7 @@ struct SolveCfg {
   float cost_kept;         //   known cost_kept per kept pair (spread over the chunks)
   double cX[3], cZ[3];     // FP64 centroids
   double sigma2, a2, b2;
-  double ell_floor, eps_pose, eps_grad;
+  double eps_pose, eps_grad;
   int max_iters, step_order, mode;
   int reduce_fp32;         // precision study: block and cross-block sums in FP32
   unsigned wait_polls;     // team barrier: polls before a block gives up

@@ -15,8 +15,11 @@
 
 #include "../../include/cvo.h"
 #include "cvo_internal.cuh"
+#include "packed_f32.cuh"
 
 namespace {
+
+using namespace cvo;
 
 constexpr int kNaThreads = 128;
 constexpr int kNaSrc = 2 * kNaThreads; // source points of a work item, two per thread
@@ -53,54 +56,6 @@ struct NaArgs {
   int tile;                // target points of a work item, a multiple of 32
 };
 
-__device__ __forceinline__ float na_ex2(float x) {
-  float y;
-  asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
-  return y;
-}
-
-// Two FP32 values and the packed operations on them (each half rounded as the
-// scalar operation rounds it): one issue slot for two.
-typedef unsigned long long na_f32x2;
-__device__ __forceinline__ na_f32x2 na_dup2(float v) {
-  na_f32x2 r;
-  asm("mov.b64 %0, {%1, %1};" : "=l"(r) : "f"(v));
-  return r;
-}
-__device__ __forceinline__ na_f32x2 na_pack2(float lo, float hi) {
-  na_f32x2 r;
-  asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(lo), "f"(hi));
-  return r;
-}
-__device__ __forceinline__ void na_unpack2(na_f32x2 v, float& lo, float& hi) {
-  asm("mov.b64 {%0, %1}, %2;" : "=f"(lo), "=f"(hi) : "l"(v));
-}
-__device__ __forceinline__ float na_sum2(na_f32x2 v) {
-  float lo, hi;
-  na_unpack2(v, lo, hi);
-  return lo + hi;
-}
-__device__ __forceinline__ na_f32x2 na_add2(na_f32x2 a, na_f32x2 b) {
-  na_f32x2 r;
-  asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
-  return r;
-}
-__device__ __forceinline__ na_f32x2 na_sub2(na_f32x2 a, na_f32x2 b) {
-  na_f32x2 r;
-  asm("sub.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
-  return r;
-}
-__device__ __forceinline__ na_f32x2 na_mul2(na_f32x2 a, na_f32x2 b) {
-  na_f32x2 r;
-  asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
-  return r;
-}
-__device__ __forceinline__ na_f32x2 na_fma2(na_f32x2 a, na_f32x2 b, na_f32x2 c) {
-  na_f32x2 r;
-  asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c));
-  return r;
-}
-
 template <int DP>
 struct NaSmem {
   alignas(16) float z[3 + DP][kNaSrc];     // transformed source points and scaled features
@@ -118,21 +73,21 @@ __device__ __forceinline__ void na_pair(const NaSmem<DP>& sm, int t, int s, floa
   const float ex = sm.x[0][t] - zx, ey = sm.x[1][t] - zy, ez = sm.x[2][t] - zz;
   const float d2 = fmaf(ex, ex, fmaf(ey, ey, ez * ez));
   float w;
-  if (MODE == cvo::kColorKernel) {
+  if (MODE == kColorKernel) {
     float q = 0.f;
 #pragma unroll
     for (int d = 0; d < DP; ++d) {
       const float df = sm.x[3 + d][t] - sm.z[3 + d][s];
       q = fmaf(df, df, q);
     }
-    w = na_ex2(-fmaf(A, d2, q));
-  } else if (MODE == cvo::kColorDot) {
+    w = ex2_approx(-fmaf(A, d2, q));
+  } else if (MODE == kColorDot) {
     float c = 0.f;
 #pragma unroll
     for (int d = 0; d < DP; ++d) c = fmaf(sm.x[3 + d][t], sm.z[3 + d][s], c);
-    w = na_ex2(-A * d2) * c;
+    w = ex2_approx(-A * d2) * c;
   } else {
-    w = na_ex2(-A * d2);
+    w = ex2_approx(-A * d2);
   }
   const float vx = w * ex, vy = w * ey, vz = w * ez;
   acc[0] += w;
@@ -177,15 +132,15 @@ __device__ __forceinline__ unsigned na_dense(const NaSmem<DP>& sm, int warp, int
     for (int k = 0; k < 7; ++k) acc64[k] += (double)acc[k];
     return cnt;
   }
-  na_f32x2 Z[2][3 + DP];
+  f32x2 Z[2][3 + DP];
 #pragma unroll
   for (int h = 0; h < 2; ++h) {
 #pragma unroll
-    for (int c = 0; c < 3 + DP; ++c) Z[h][c] = na_dup2(sm.z[c][s0 + 32 * h]);
+    for (int c = 0; c < 3 + DP; ++c) Z[h][c] = dup2(sm.z[c][s0 + 32 * h]);
   }
   float acc[7] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
-  const na_f32x2 A2 = na_dup2(A);
-  na_f32x2 sum[2][4] = {{0ull, 0ull, 0ull, 0ull}, {0ull, 0ull, 0ull, 0ull}};
+  const f32x2 A2 = dup2(A);
+  f32x2 sum[2][4] = {{0ull, 0ull, 0ull, 0ull}, {0ull, 0ull, 0ull, 0ull}};
   unsigned cnt = 0;
   for (int t = 0; t < tn; t += 4) {
     ulonglong2 X[3 + DP];
@@ -195,46 +150,46 @@ __device__ __forceinline__ unsigned na_dense(const NaSmem<DP>& sm, int warp, int
     for (int h = 0; h < 2; ++h) {
 #pragma unroll
       for (int p = 0; p < 2; ++p) {
-        const na_f32x2 ex = na_sub2(p ? X[0].y : X[0].x, Z[h][0]);
-        const na_f32x2 ey = na_sub2(p ? X[1].y : X[1].x, Z[h][1]);
-        const na_f32x2 ez = na_sub2(p ? X[2].y : X[2].x, Z[h][2]);
-        const na_f32x2 d2 = na_fma2(ex, ex, na_fma2(ey, ey, na_mul2(ez, ez)));
-        na_f32x2 q = 0ull;   // appearance: sum of squared differences, or inner product
+        const f32x2 ex = sub2(p ? X[0].y : X[0].x, Z[h][0]);
+        const f32x2 ey = sub2(p ? X[1].y : X[1].x, Z[h][1]);
+        const f32x2 ez = sub2(p ? X[2].y : X[2].x, Z[h][2]);
+        const f32x2 d2 = fma2(ex, ex, fma2(ey, ey, mul2(ez, ez)));
+        f32x2 q = 0ull;   // appearance: sum of squared differences, or inner product
 #pragma unroll
         for (int d = 0; d < DP; ++d) {
-          const na_f32x2 f = p ? X[3 + d].y : X[3 + d].x;
-          if (MODE == cvo::kColorKernel) {
-            const na_f32x2 df = na_sub2(f, Z[h][3 + d]);
-            q = na_fma2(df, df, q);
-          } else if (MODE == cvo::kColorDot) {
-            q = na_fma2(f, Z[h][3 + d], q);
+          const f32x2 f = p ? X[3 + d].y : X[3 + d].x;
+          if (MODE == kColorKernel) {
+            const f32x2 df = sub2(f, Z[h][3 + d]);
+            q = fma2(df, df, q);
+          } else if (MODE == kColorDot) {
+            q = fma2(f, Z[h][3 + d], q);
           }
         }
         float d20, d21, e0, e1;
-        na_unpack2(d2, d20, d21);
+        unpack2(d2, d20, d21);
         const bool k0 = d20 <= rc2, k1 = d21 <= rc2;
-        na_unpack2(MODE == cvo::kColorKernel ? na_fma2(A2, d2, q) : na_mul2(A2, d2), e0, e1);
-        float w0 = na_ex2(-e0), w1 = na_ex2(-e1);
-        if (MODE == cvo::kColorDot) {
+        unpack2(MODE == kColorKernel ? fma2(A2, d2, q) : mul2(A2, d2), e0, e1);
+        float w0 = ex2_approx(-e0), w1 = ex2_approx(-e1);
+        if (MODE == kColorDot) {
           float c0, c1;
-          na_unpack2(q, c0, c1);
+          unpack2(q, c0, c1);
           w0 *= c0;
           w1 *= c1;
         }
-        const na_f32x2 w = na_pack2(k0 ? w0 : 0.f, k1 ? w1 : 0.f);
+        const f32x2 w = pack2(k0 ? w0 : 0.f, k1 ? w1 : 0.f);
         cnt += (k0 ? 1u : 0u) + (k1 ? 1u : 0u);
-        sum[h][0] = na_add2(sum[h][0], w);
-        sum[h][1] = na_fma2(w, ex, sum[h][1]);
-        sum[h][2] = na_fma2(w, ey, sum[h][2]);
-        sum[h][3] = na_fma2(w, ez, sum[h][3]);
+        sum[h][0] = add2(sum[h][0], w);
+        sum[h][1] = fma2(w, ex, sum[h][1]);
+        sum[h][2] = fma2(w, ey, sum[h][2]);
+        sum[h][3] = fma2(w, ez, sum[h][3]);
       }
     }
   }
 #pragma unroll
   for (int h = 0; h < 2; ++h) {   // omega' += z~' x E, v += E, E = sum w e
     const float zx = sm.z[0][s0 + 32 * h], zy = sm.z[1][s0 + 32 * h], zz = sm.z[2][s0 + 32 * h];
-    const float Ex = na_sum2(sum[h][1]), Ey = na_sum2(sum[h][2]), Ez = na_sum2(sum[h][3]);
-    acc[0] += na_sum2(sum[h][0]);
+    const float Ex = sum2(sum[h][1]), Ey = sum2(sum[h][2]), Ez = sum2(sum[h][3]);
+    acc[0] += sum2(sum[h][0]);
     acc[1] += zy * Ez - zz * Ey;
     acc[2] += zz * Ex - zx * Ez;
     acc[3] += zx * Ey - zy * Ex;
@@ -366,14 +321,14 @@ na_grad_kernel(const float* __restrict__ x, const float* __restrict__ fx,
     stage(j0, i0);
     __syncthreads();
     if (j0 + warp * 64 >= a.m) continue;   // a warp past the last source point
-    na_f32x2 Z[2][3];
+    f32x2 Z[2][3];
     bool zv[2];
 #pragma unroll
     for (int h = 0; h < 2; ++h) {
       const int k = warp * 64 + 32 * h + lane;
       zv[h] = j0 + k < a.m;
 #pragma unroll
-      for (int c = 0; c < 3; ++c) Z[h][c] = na_dup2(sm.z[c][k]);
+      for (int c = 0; c < 3; ++c) Z[h][c] = dup2(sm.z[c][k]);
     }
     int queued = 0;   // the same in every lane
     for (int t0 = 0; t0 < tn; t0 += 64) {
@@ -392,12 +347,12 @@ na_grad_kernel(const float* __restrict__ x, const float* __restrict__ fx,
           for (int h = 0; h < 2; ++h) {
 #pragma unroll
             for (int p = 0; p < 2; ++p) {
-              const na_f32x2 ex = na_sub2(p ? X.y : X.x, Z[h][0]);
-              const na_f32x2 ey = na_sub2(p ? Y.y : Y.x, Z[h][1]);
-              const na_f32x2 ez = na_sub2(p ? W.y : W.x, Z[h][2]);
-              const na_f32x2 d2 = na_fma2(ex, ex, na_fma2(ey, ey, na_mul2(ez, ez)));
+              const f32x2 ex = sub2(p ? X.y : X.x, Z[h][0]);
+              const f32x2 ey = sub2(p ? Y.y : Y.x, Z[h][1]);
+              const f32x2 ez = sub2(p ? W.y : W.x, Z[h][2]);
+              const f32x2 d2 = fma2(ex, ex, fma2(ey, ey, mul2(ez, ez)));
               float d20, d21;
-              na_unpack2(d2, d20, d21);
+              unpack2(d2, d20, d21);
               if (d20 <= a.rc2) keep[h][w] |= 1u << (k + 2 * p);
               if (d21 <= a.rc2) keep[h][w] |= 1u << (k + 2 * p + 1);
             }
@@ -530,7 +485,7 @@ extern "C" int cvo_eval_gradient_static(const float* d_x, const float* d_fx, int
   g_na_err.clear();
   if (!d_x || !d_z || !d_out || !params || !P)
     return na_fail(CVO_ERR_INVALID_ARG, "NULL pointer argument");
-  if (n < 1 || m < 1 || n > cvo::kMaxPoints || m > cvo::kMaxPoints)
+  if (n < 1 || m < 1 || n > kMaxPoints || m > kMaxPoints)
     return na_fail(CVO_ERR_INVALID_ARG, "point count outside [1, 2^22]");
   const cvo_params& p = *params;
   if (!(ell > 0.0) || !std::isfinite(ell) || !(p.kcut > 0.0 && p.kcut < 1.0) || !(p.sigma > 0.0) ||
@@ -594,15 +549,15 @@ extern "C" int cvo_eval_gradient_static(const float* d_x, const float* d_fx, int
   cudaStream_t s = (cudaStream_t)stream;
   cudaError_t e;
   const int dp = D == 0 ? 0 : D <= 3 ? 3 : D <= 5 ? 5 : 8;
-  if (mode == CVO_COLOR_NONE) e = na_launch<0, cvo::kColorNone>(nblocks, d_x, d_fx, d_z, d_fz, a, partials, s);
+  if (mode == CVO_COLOR_NONE) e = na_launch<0, kColorNone>(nblocks, d_x, d_fx, d_z, d_fz, a, partials, s);
   else if (mode == CVO_COLOR_KERNEL)
-    e = dp == 3 ? na_launch<3, cvo::kColorKernel>(nblocks, d_x, d_fx, d_z, d_fz, a, partials, s)
-      : dp == 5 ? na_launch<5, cvo::kColorKernel>(nblocks, d_x, d_fx, d_z, d_fz, a, partials, s)
-                : na_launch<8, cvo::kColorKernel>(nblocks, d_x, d_fx, d_z, d_fz, a, partials, s);
+    e = dp == 3 ? na_launch<3, kColorKernel>(nblocks, d_x, d_fx, d_z, d_fz, a, partials, s)
+      : dp == 5 ? na_launch<5, kColorKernel>(nblocks, d_x, d_fx, d_z, d_fz, a, partials, s)
+                : na_launch<8, kColorKernel>(nblocks, d_x, d_fx, d_z, d_fz, a, partials, s);
   else
-    e = dp == 3 ? na_launch<3, cvo::kColorDot>(nblocks, d_x, d_fx, d_z, d_fz, a, partials, s)
-      : dp == 5 ? na_launch<5, cvo::kColorDot>(nblocks, d_x, d_fx, d_z, d_fz, a, partials, s)
-                : na_launch<8, cvo::kColorDot>(nblocks, d_x, d_fx, d_z, d_fz, a, partials, s);
+    e = dp == 3 ? na_launch<3, kColorDot>(nblocks, d_x, d_fx, d_z, d_fz, a, partials, s)
+      : dp == 5 ? na_launch<5, kColorDot>(nblocks, d_x, d_fx, d_z, d_fz, a, partials, s)
+                : na_launch<8, kColorDot>(nblocks, d_x, d_fx, d_z, d_fz, a, partials, s);
   if (e != cudaSuccess) return na_fail(CVO_ERR_CUDA, cudaGetErrorString(e));
   na_finish_kernel<<<1, 32 * kNaStride, 0, s>>>(partials, nblocks, d_x, p.sigma * p.sigma, 1.0 / ell2, p.a2,
                                     p.b2, d_out);

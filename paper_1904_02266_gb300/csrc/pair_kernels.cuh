@@ -52,6 +52,7 @@
 #include <algorithm>
 
 #include "cvo_internal.cuh"
+#include "packed_f32.cuh"
 #include "split_rule.h"
 
 // Resident blocks per SM the solve kernel is compiled for (register budget).
@@ -95,54 +96,6 @@ constexpr int kSmallTeamFrom = 20000;
 // pair 825, 832, 832 us
 constexpr int kSpareWork = 400;
 
-__device__ __forceinline__ float ex2_approx(float x) {
-  float y;
-  asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
-  return y;
-}
-
-// Two FP32 values in one 64-bit register pair and the packed operations on
-// them, each half rounded as the scalar operation rounds it. A packed FMA
-// keeps the FMA pipe busy for two cycles of a scheduler (measured: 2.2 against
-// 1.02 for a scalar one, so the rate per FMA is the same) but takes one issue
-// slot, and the pair bodies are short of issue slots, not of FMA lanes.
-typedef unsigned long long f32x2;
-
-__device__ __forceinline__ f32x2 pack2(float lo, float hi) {
-  f32x2 r;
-  asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(lo), "f"(hi));
-  return r;
-}
-__device__ __forceinline__ f32x2 dup2(float v) { return pack2(v, v); }
-__device__ __forceinline__ void unpack2(f32x2 v, float& lo, float& hi) {
-  asm("mov.b64 {%0, %1}, %2;" : "=f"(lo), "=f"(hi) : "l"(v));
-}
-__device__ __forceinline__ float sum2(f32x2 v) {
-  float lo, hi;
-  unpack2(v, lo, hi);
-  return lo + hi;
-}
-__device__ __forceinline__ f32x2 fma2(f32x2 a, f32x2 b, f32x2 c) {
-  f32x2 r;
-  asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c));
-  return r;
-}
-__device__ __forceinline__ f32x2 mul2(f32x2 a, f32x2 b) {
-  f32x2 r;
-  asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
-  return r;
-}
-__device__ __forceinline__ f32x2 add2(f32x2 a, f32x2 b) {
-  f32x2 r;
-  asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
-  return r;
-}
-__device__ __forceinline__ f32x2 sub2(f32x2 a, f32x2 b) {
-  f32x2 r;
-  asm("sub.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
-  return r;
-}
-
 // One feature value: FP32 planes, or BF16 planes widened to FP32 (FB).
 template <bool FB>
 __device__ __forceinline__ float load_feat(const float* planes, size_t idx) {
@@ -171,18 +124,6 @@ __device__ __forceinline__ int cell_floor(float v, float o, float inv_h, int n) 
   return (int)q;
 }
 
-__device__ __forceinline__ float warp_sum_f(float v) {
-#pragma unroll
-  for (int off = 16; off > 0; off >>= 1) v += __shfl_down_sync(kFull, v, off);
-  return v;
-}
-
-__device__ __forceinline__ double warp_sum_d(double v) {
-#pragma unroll
-  for (int off = 16; off > 0; off >>= 1) v += __shfl_down_sync(kFull, v, off);
-  return v;
-}
-
 // ---------------------------------------------------------------------------
 // per-block iteration state (identical in every block of a team)
 // ---------------------------------------------------------------------------
@@ -199,7 +140,7 @@ struct Team {
 struct TailConst {
   double cX[3], cZ[3];
   double sigma2, inv_a2, inv_b2;
-  double ell_floor, eps_pose, eps_grad, src_radius;
+  double eps_pose, eps_grad, src_radius;
   int mode, step_order, max_iters;
   int reduce_fp32;   // precision study: block and cross-block sums in FP32
   unsigned wait_polls;                 // barrier polls before a block gives up
@@ -2989,7 +2930,6 @@ __device__ void solve_pair(const SolveCfg* __restrict__ cfg, SolveState* __restr
     tc.sigma2 = cfg->sigma2;
     tc.inv_a2 = 1.0 / cfg->a2;
     tc.inv_b2 = 1.0 / cfg->b2;
-    tc.ell_floor = cfg->ell_floor;
     tc.eps_pose = cfg->eps_pose;
     tc.eps_grad = cfg->eps_grad;
     tc.src_radius = cfg->src_radius;
