@@ -108,8 +108,9 @@ typedef struct {
        persistent launch whose blocks wait on each other; every wait is
        bounded so that a lost block ends the solve with CVO_ERR_TIMEOUT
        instead of hanging the GPU): */
-    int wait_polls;        /* polls of a team barrier before a block gives up, in [1, 2^30]
-                              (each poll sleeps about 0.5 us); 4194304 (about 2 s) */
+    int wait_polls;        /* polls of a team barrier before a block gives up, in [1, 2^30]; a
+                              poll is a read of L2 (about 0.5 us), from the 65th on with a
+                              sleep of 32 ns or more before the next; 4194304 (about 2 s) */
     double join_limit_ms;  /* how long a queued pair's first block waits for the rest of its
                               team to start, in (0, 1e7] ms; 60000 */
 } cvo_params;

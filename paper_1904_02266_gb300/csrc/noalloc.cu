@@ -25,7 +25,7 @@ constexpr int kNaThreads = 128;
 constexpr int kNaSrc = 2 * kNaThreads; // source points of a work item, two per thread
 constexpr int kNaTile = 256;           // its target points at most
 constexpr int kNaMaxBlocks = 608;      // partial slots in the static scratch
-constexpr int kNaGrid = 4 * 152;       // blocks of a full launch: four to an SM
+constexpr int kNaGrid = 4 * 152;       // blocks of a full launch: four to each of GB300's SMs
 constexpr int kNaQueue = 2048;         // pairs a warp appends to its queue at once
 constexpr int kNaStride = 8;           // F, omega'(3), v(3), kept pairs
 constexpr int kNaMaxDevices = 64;

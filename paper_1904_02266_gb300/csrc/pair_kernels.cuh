@@ -85,7 +85,11 @@ constexpr int kCompactWork = 3000;
 // pieces of 1500 units 46.9 ms, 8 of 1500 46.2, 8 of 700 45.4; at 20k points
 // (about 1000 units a warp) a second piece costs a cluster and two ends more than
 // it evens out. Small teams: two pieces from kSmallTeamFrom units on (64-pair batch:
-// one piece 105.0 ms, two 104.0, up to eight 111.9)
+// one piece 105.0 ms, two 104.0, up to eight 111.9). These lines, kCompactWork and
+// kSpareWork count units of the caller's cost model (cost_chunk 48 and cost_cluster 32
+// by default) and so move with it; with cost_chunk 16, 32, 96 and 256 and with
+// cost_cluster 0, 128 and 1024 room solves of 2k to 100k points took 0.52 to 0.96 of
+// their time before the lines were drawn
 constexpr int kMaxRanges = 8;
 constexpr int kRangeWork = 700;
 constexpr int kRangeFrom = 2000;
@@ -93,7 +97,7 @@ constexpr int kSmallTeamFrom = 20000;
 // shares below this many units leave the block's last warp out of the passes
 // (split_work). Whole room solves without, from 400 and from 1500 units: 10k points
 // 3.80, 3.68, 3.68 ms, 20k 5.65, 5.51, 5.57 ms, 28k 7.45, 7.44, 7.47 ms; the 2k planes
-// pair 825, 832, 832 us
+// pair, whose passes are the shortest, 825, 832, 832 us
 constexpr int kSpareWork = 400;
 
 // One feature value: FP32 planes, or BF16 planes widened to FP32 (FB).
@@ -653,7 +657,7 @@ __device__ void gradient_direction(BlockCtx& b, const double* sums, int lane) {
     b.om[a] = x * inv;
     b.vc[a] = vc;
   }
-  // the step pass's constants (step_terms): |omega|^2 and omega . v'
+  // the step pass's constants (chunk_bodies, list_pair): |omega|^2 and omega . v'
   const float om = x * inv;
   float ww = om * om, wv = om * vc;
   ww += __shfl_sync(kFull, ww, 1) + __shfl_sync(kFull, ww, 2);   // lane 0's is used
@@ -1012,8 +1016,10 @@ __device__ __forceinline__ long long warp_sum_i64(long long v) {
 }
 
 // The sum of the nblk values at p (one warp, every lane gets it): exact up to a
-// truncation of each value 52 bits below the largest, no less than FP64
-// additions keep (theirs round at the size of the running sum). The mantissas are
+// truncation of each value 52 bits below the largest. The block partials are FP32 sums
+// widened to FP64 (run_pass), so that only values 2^29 times smaller than the largest lose
+// bits at all, no more than FP64 additions take from them (theirs round at the size of the
+// running sum; values of 53 bits would fare worse here). The mantissas are
 // aligned to the largest exponent and added as integers, in any order with the
 // same result: on GB300 an FP64 instruction holds its scheduler's FP64 pipe for
 // about 64 cycles, and the ten dependent additions per value (two values to a
@@ -1387,10 +1393,11 @@ __device__ __forceinline__ long long cluster_work(const SolveCfg* cfg, const Clu
   return w;
 }
 
-// Entries of a warp's pair list (build_lists), per padded feature width: as
-// many as fit beside the block's other static shared memory without taking a
-// cache slot from the dynamic part at one block per SM (640 at 5 feature
-// planes, 448 at 3 and 8, 400 without features).
+// Entries of a warp's pair list (build_lists), per padded feature width (640 at 5 feature
+// planes, 448 at 3 and 8, 400 without features). They are static shared memory, so each
+// takes two bytes a warp from the plan cache, which packs clusters and chunks; the
+// counts are those that cost no 32-point slot when the cache was made of slots. The room
+// pair of 20k points lists 250 a warp.
 template <int DPS>
 __host__ __device__ constexpr int list_max() {
   return DPS == 5 ? 640 : DPS == 1 ? 400 : 448;
@@ -1431,7 +1438,7 @@ struct SolveSmem {
   float4 z[kWarps][kClusterMax];
   float4 zo[kWarps];                // origin of each warp's staged cluster (centred frame)
   float zf[kWarps][DPS][kClusterMax];
-  float4 u[kWarps][NU][kClusterMax];   // step vectors of a listed cluster's points (step_terms)
+  float4 u[kWarps][NU][kClusterMax];   // step vectors of a listed cluster's points (stage_cluster)
   float zw[kWarps][kClusterMax];       // step pass: -z_l . kw
   union {
     WarpScratch<DPS> ws[kWarps];    // cell-row segments of the staged cluster, or the pair list
@@ -1773,23 +1780,6 @@ __device__ __forceinline__ StepVectors step_vectors(const BlockCtx& b, float x, 
   return s;
 }
 
-// One 32-candidate chunk against the staged cluster: lane = candidate x'
-// (xp, features xf; padding points lie beyond every cutoff and carry w = 1),
-// over the cluster's points [jlo, jhi) (multiples of 4, at most the cluster
-// size rounded up to 4; padding slots lie beyond the cutoff too). FP32 pair
-// arithmetic, one ex2.approx per pair. Distances are taken relative to the
-// cluster's origin (stage_cluster): t = x_l . (-2 z_l) + |z_l|^2 equals
-// d^2 - |x_l|^2, so a pair is kept when t <= r_c^2 - |x_l|^2, and the
-// exponent A d^2 is A t + A |x_l|^2.
-// Points are taken four at a time, as two packed pairs: the staged planes give
-// both halves of each operand with one 16-byte broadcast load per four points
-// and component. First the distance tests of every group of four, each lane
-// noting the groups in which it keeps a pair; one reduction over the warp then
-// gives the groups to evaluate, whose bodies run without votes or branches (a
-// rejected pair contributes exactly nothing: its weight is selected to zero, and
-// its beta, whose fourth power would be the first of its step terms to
-// overflow). Testing all groups first keeps the chain of loads, test, vote and
-// branch out of the bodies, which repeat the test's six packed FMAs instead.
 // A candidate against the cluster staged for the warp.
 struct ChunkLane {
   f32x2 X, Y, Z;          // x_l
@@ -1989,7 +1979,24 @@ __device__ __forceinline__ void chunk_bodies(SolveSmem<DPS, NU>& sm, int warp, f
   }
 }
 
-// One chunk against source points [jlo, jhi); returns its active groups.
+// One 32-candidate chunk against the staged cluster: lane = candidate x'
+// (xp, features xf; padding points lie beyond every cutoff and carry w = 1),
+// over the cluster's points [jlo, jhi) (multiples of 4, at most the cluster
+// size rounded up to 4; padding slots lie beyond the cutoff too). FP32 pair
+// arithmetic, one ex2.approx per pair. Distances are taken relative to the
+// cluster's origin (stage_cluster): t = x_l . (-2 z_l) + |z_l|^2 equals
+// d^2 - |x_l|^2, so a pair is kept when t <= r_c^2 - |x_l|^2, and the
+// exponent A d^2 is A t + A |x_l|^2.
+// Points are taken four at a time, as two packed pairs: the staged planes give
+// both halves of each operand with one 16-byte broadcast load per four points
+// and component. First the distance tests of every group of four, each lane
+// noting the groups in which it keeps a pair; one reduction over the warp then
+// gives the groups to evaluate, whose bodies run without votes or branches (a
+// rejected pair contributes exactly nothing: its weight is selected to zero, and
+// its beta, whose fourth power would be the first of its step terms to
+// overflow). Testing all groups first keeps the chain of loads, test, vote and
+// branch out of the bodies, which repeat the test's six packed FMAs instead.
+// Returns the active groups.
 template <bool STEP, int DP, int MODE, int DPS, int NU>
 __device__ __forceinline__ unsigned chunk_pairs(SolveSmem<DPS, NU>& sm, int warp, float4 xp,
                                                 const float xf[DPS], int jlo, int jhi, float rc2,
